@@ -7,9 +7,11 @@ re-unitarisation, Gaussian spinors, FP64 storage and arithmetic, 1 RHS.
 One step = one full-lattice D_w application (one kernel launch).
 
 `value` is GFLOP/s of that kernel (1320 flop per site, the hopping term)
-divided by the CUDA-event time.  On GB300 the FP64 dslash is bound by the
-FP64 pipe, so its roofline is the FMA throughput measured in the same run by
-the library's own FMA kernel.  The JSON line also carries algorithmic GB/s,
+divided by the CUDA-event time.  The FP64 dslash multiplies links and spinors
+in 64-bit fixed point on the integer pipes (its error against 64-bit sums is at
+most that of FP64 multiply-adds), so its rate may exceed the FP64 FMA
+throughput that the library's own FMA kernel measures in the same run and that
+the line quotes beside the HBM fraction.  The JSON line also carries algorithmic GB/s,
 the FP32 / FP16 / BF16 / double-float and 12-RHS variants (the FP32 one with
 its HBM roofline), a small propagator solve (12 point sources to the FP64
 true residual 1e-10), an end-to-end figure through the C ABI with host
@@ -59,11 +61,16 @@ VARIANT_UNIT = {0: "dslash_regs.cu", 1: "dslash_regs.cu", 2: "dslash_regs.cu", 3
                 8: "dslash_batched.cu", 9: "dslash_batched.cu", 10: "dslash_pair.cu", 11: "dslash_pair.cu"}
 
 
-def kernel_sources_sha(var: int = 1) -> str:
+WIDE_UNIT = "dslash_split.cu"  # FP64 and double-float, every variant
+
+
+def kernel_sources_sha(var: int = 1, prec: str = "f32") -> str:
     """Hash of the sources of the dslash kernel of launch variant `var`: a DRAM-traffic figure from
     an ncu capture holds only while the kernel it was taken on is unchanged."""
     h = hashlib.sha256()
-    for f in (VARIANT_UNIT[var], "dslash_common.cuh", "ov_internal.cuh", "ov_kernels.h"):
+    wide = prec in ("f64", "df64")
+    for f in ((WIDE_UNIT, "dslash_fix.cuh") if wide else (VARIANT_UNIT[var],)) + (
+            "dslash_common.cuh", "ov_internal.cuh", "ov_kernels.h"):
         with open(os.path.join(ROOT, "paper_1106_4964_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -72,18 +79,17 @@ def kernel_sources_sha(var: int = 1) -> str:
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch, from the ncu captures
 # summarised under profiles/, keyed by (kernel, lattice, sources hash at capture time).  A kernel whose
 # sources changed since its capture gets null.
-NCU_TRAFFIC = {
-    # FP64, 1 rhs, block 256 x 1, register-budget variant 1 (the default run's timed kernel)
-    ("dslash_kernel<f64,f64,variant=1>", (24, 24, 24, 64), "625052d99d5871d2"): 734_775_552 + 153_691_392,
-}
+NCU_TRAFFIC = {}
 
 
-def ncu_traffic(kernel: str, var: int):
-    return NCU_TRAFFIC.get((kernel, tuple(DIMS), kernel_sources_sha(var)))
+def ncu_traffic(kernel: str, var: int, prec: str):
+    return NCU_TRAFFIC.get((kernel, tuple(DIMS), kernel_sources_sha(var, prec)))
 
 
 def kernel_name(prec: str, var: int, nrhs: int = 1) -> str:
     """The CUDA kernel a dslash launch of this precision and launch variant runs."""
+    if prec in ("f64", "df64"):
+        return f"dslash_split_kernel<{prec},variant={var}>"
     if var == 3:
         return f"dslash_staged_kernel<{prec},{prec}>"
     if var in (4, 5):
@@ -303,7 +309,7 @@ def run_gpu(args):
                                    "GFLOPps": round(FLOP_SITE * V / t / 1e6, 1),
                                    "frac_hbm": round(b / t / 1e6 / hbm, 3), "kernel": kernel_name(p, sh[2]),
                                    "shape": list(sh)}
-        variants["df64_r1"]["frac_f32_fma_note"] = "double-float is bound by the FP32 pipe, not HBM"
+        variants["df64_r1"]["frac_f32_fma_note"] = "double-float is bound by the integer pipe, not HBM"
         psi12 = torch.from_numpy(make_inputs_rhs(12)).cuda()
         for p in ("f32", "f16", "f64", "df64"):
             t, sh = time_dslash(ctx, psi12, p, 12, min(300, max(5, args.steps // 2)), args.warmup, torch)
@@ -360,10 +366,12 @@ def run_gpu(args):
                        launches_per_step=reps),
         "GBps": round(gbs * world, 1),
         "roofline": {"bound": "alu", "achieved": round(gflops, 1), "peak": fma_peak, "unit": "GFLOP/s",
-                     "frac": round(gflops / fma_peak, 4), "traffic": ncu_traffic(kern, var),
+                     "frac": round(gflops / fma_peak, 4), "traffic": ncu_traffic(kern, var, prec),
                      "peak_kind": f"measured: {prec if prec in ('f64', 'f32') else 'f32'} FMA throughput of this "
                                   "GPU (ov_measure_fma_peak, same run)",
                      "peak_nominal": FP64_NOMINAL_GFLOPS, "frac_nominal": round(gflops / FP64_NOMINAL_GFLOPS, 4),
+                     "note": ("FP64 and double-float hops multiply in 64-bit fixed point on the integer pipes: the "
+                              "rate may exceed the FP64 FMA peak") if prec in ("f64", "df64") else "",
                      "algorithmic_flops_per_launch": FLOP_SITE * V, "kernel": kern,
                      "hbm": {"achieved": round(gbs, 1), "peak": hbm, "frac": round(gbs / hbm, 4),
                              "peak_kind": peak_kind, "algorithmic_bytes_per_launch": int(bytes_launch)}},

@@ -36,9 +36,16 @@
  *  - Precision (ov_prec): OV_F64 stores and computes in FP64; OV_F32 in FP32;
  *    OV_F16S / OV_BF16S store spinors and links in 16 bits (spinors with one
  *    FP32 scale per site) and compute in FP32; OV_DF64 stores every real as an
- *    unevaluated sum of two FP32 numbers (8 bytes, about 48 significand bits)
- *    and computes with error-free FP32 transformations, an FP64-class result
- *    on the FP32 pipes.  Dot products and norms always accumulate in FP64.
+ *    unevaluated sum of two FP32 numbers (8 bytes, about 48 significand bits),
+ *    an FP64-class result on the FP32 pipes.  The hopping term of the OV_F64
+ *    and OV_DF64 dslash multiplies links and spinors as 64-bit fixed-point
+ *    numbers on the integer pipes, scaled by each neighbour's largest
+ *    component: the rounding, relative to the field around a site, is at most
+ *    that of the floating-point sums.  Sites whose neighbourhood that format
+ *    does not hold (infinities, NaN, exponents near the ends of the range,
+ *    components that differ by more than 2^26 within a neighbour or 2^16
+ *    between neighbours) use the floating-point arithmetic.  Dot products and
+ *    norms always accumulate in FP64.
  */
 #ifndef OVERLAP_GB300_H
 #define OVERLAP_GB300_H
@@ -92,8 +99,8 @@ const char* ov_last_error(const ov_ctx* ctx);
  * transporters on the links).  U: canonical complex128 gauge layout, host or
  * device.  The library packs it to reconstruct-12 form (rows 0 and 1 kept,
  * row 2 = conj(row0 x row1)) in FP32, FP16 and BF16, where the dslash is
- * bound by bandwidth, and keeps all three rows in FP64 and double-float,
- * where it is bound by arithmetic.  Returns OV_EINVAL
+ * bound by bandwidth, and keeps all three rows as 64-bit fixed-point numbers
+ * (one copy) for FP64 and double-float, where it is bound by arithmetic.  Returns OV_EINVAL
  * if any link deviates from SU(3) by more than 1e-9 (|U U^dag - 1| or the
  * reconstructed third row), since reconstruct-12 would change it. */
 int ov_set_gauge(ov_ctx* ctx, const void* U, void* stream);
@@ -372,7 +379,9 @@ int ov_set_option(ov_ctx* ctx, const char* name, double value);
 int ov_get_option(const ov_ctx* ctx, const char* name, double* value);
 /* Launch configuration of the dslash for (prec, nrhs): block = bx sites x by
  * right-hand sides, and a kernel variant: 0 unbounded registers; 1, 2
- * registers capped so that more warps are resident; 3 neighbours staged in
+ * registers capped so that more warps are resident (OV_F64, OV_DF64: blocks of
+ * eight warps, one per hop, that walk over bx / 32 groups of 32 sites and by
+ * right-hand sides; 0, 1, 2: two, three, four blocks per SM); 3 neighbours staged in
  * shared memory by cp.async; 4, 5 staged by bulk copies (bx = 128, by = 1);
  * 6, 7 two or four right-hand sides per thread sharing each link; 8, 9 the
  * loads of four or eight hops issued before their arithmetic (by = 1); 10, 11

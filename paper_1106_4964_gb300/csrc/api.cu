@@ -213,10 +213,19 @@ int eig_vectors(ov_ctx* c, int which, int prec, cudaStream_t st, FieldDesc* out)
 
 static std::tuple<int, int, int> default_shape(int prec, int nrhs)
 {
-    if (nrhs == 1) return {wide(prec) ? 64 : 128, 1, 0};
-    const int cap = wide(prec) ? 8 : 16;
-    int by = nrhs > cap ? cap : nrhs;
-    return {32, by, 0};
+    // FP64, double-float: one block of eight warps per 32 sites and right-hand side, with the registers each
+    // form needs.  us per launch, 32 x 1 / 64 x 1 / 128 x 1: FP64 8^3 x 16 10.3 / 12.4 / 20; 24^3 x 64 488 / 498 /
+    // 505; 12 rhs at 8^4 30.8 / 34.8 / 41; double-float 24^3 x 64 665 / 686 / 687
+    if (wide(prec)) return {32, 1, prec == P_F64 ? 1 : 0};
+    if (nrhs == 1) return {128, 1, 0};
+    return {32, nrhs > 16 ? 16 : nrhs, 0};
+}
+
+// a double as an unevaluated sum of two FP32 numbers
+static float2 split2(double x)
+{
+    const float hi = (float)x;
+    return make_float2(hi, (float)(x - (double)hi));
 }
 
 int dslash_apply(ov_ctx* c, const FieldDesc& in, const FieldDesc& out, double a, double b, int g5_core, int g5_out,
@@ -238,11 +247,14 @@ int dslash_apply(ov_ctx* c, const FieldDesc& in, const FieldDesc& out, double a,
         A.y_n[j] = y[j].norm;
         A.sy[j] = sy[j];
         A.fsy[j] = (float)sy[j];
+        A.dsy[j] = split2(sy[j]);
     }
     A.a = a;
     A.b = b;
     A.fa = (float)a;
     A.fb = (float)b;
+    A.da = split2(a);
+    A.db = split2(b);
     A.nrhs = in.nrhs;
     A.g5_core = g5_core;
     A.g5_out = g5_out;
@@ -832,7 +844,7 @@ int ov_destroy(ov_ctx* c)
     graphs_clear(c);
     net_free(c);
     for (int p = 0; p < NPREC; ++p)
-        if (c->gauge[p]) dev_free(c, c->gauge[p], (size_t)8 * c->g.Vh * gauge_link_bytes(p));
+        if (c->gauge[p] && p != P_DF64) dev_free(c, c->gauge[p], (size_t)8 * c->g.Vh * gauge_link_bytes(p));
     for (auto& e : c->eig) eig_clear(c, e);
     for (auto& kv : c->ws) field_free(c, &kv.second);
     if (c->partials) dev_free(c, c->partials, c->partials_bytes);
@@ -865,10 +877,12 @@ int ov_set_gauge(ov_ctx* c, const void* U, void* stream)
     const double* dU = nullptr;
     OV_TRY(stage_in(c, 0, U, bytes, st, &dU));
     for (int p = 0; p < NPREC; ++p) {
-        if (!c->gauge[p]) OV_TRY(dev_alloc(c, &c->gauge[p], (size_t)8 * c->g.Vh * gauge_link_bytes(p)));
+        if (!c->gauge[p] && p != P_DF64) OV_TRY(dev_alloc(c, &c->gauge[p], (size_t)8 * c->g.Vh * gauge_link_bytes(p)));
     }
+    c->gauge[P_DF64] = c->gauge[P_F64];  // one copy of the 64-bit links
     OV_CUDA(c, cudaMemsetAsync(c->derr, 0, 2 * sizeof(unsigned), st));
-    for (int p = 0; p < NPREC; ++p) OV_CUDA(c, launch_pack_gauge(c->g, dU, c->gauge[p], p, p == 0 ? c->derr : nullptr, st));
+    for (int p = 0; p < NPREC; ++p)
+        if (p != P_DF64) OV_CUDA(c, launch_pack_gauge(c->g, dU, c->gauge[p], p, p == 0 ? c->derr : nullptr, st));
     unsigned herr[2];
     OV_CUDA(c, cudaMemcpyAsync(herr, c->derr, sizeof herr, cudaMemcpyDeviceToHost, st));
     OV_CUDA(c, cudaStreamSynchronize(st));
@@ -1457,7 +1471,13 @@ int ov_tune_dslash(ov_ctx* c, int prec, int nrhs, int* bx, int* by, int* variant
                     if (groups % y == 0 && x * y >= 64) cand.push_back(std::make_tuple(x, y, v));
             continue;
         }
-        const int maxt = v == 0 ? (wide(prec) ? 256 : 512) : (v == 3 ? 128 : 256);
+        if (wide(prec)) {                    // a block walks over x / 32 site groups and y right-hand sides
+            for (int x : {32, 64, 128})
+                for (int y = 1; y <= nrhs && y <= 4; ++y)
+                    if (nrhs % y == 0) cand.push_back(std::make_tuple(x, y, v));
+            continue;
+        }
+        const int maxt = v == 0 ? 512 : (v == 3 ? 128 : 256);
         for (int x : {32, 64, 128, 256})
             for (int y = 1; y <= nrhs && y <= 16; ++y) {
                 if (v == 3 && y != 1) continue;

@@ -11,6 +11,7 @@ cudaError_t launch_dslash(const DslashArgs& A, int sp, int gp, int ny, int bx, i
     const dim3 block(bx, by);
     // one dimension: 2 parities x site blocks x right-hand-side groups (the kernels' block_work)
     const dim3 grid((unsigned)(2 * ((A.g.Vh + bx - 1) / bx) * ((A.nrhs + by - 1) / by)));
+    if (wide(sp)) return launch_dslash_split(A, sp, gp, ny, var, bx, by, st);
     if (var >= 0 && var <= 2) return launch_dslash_regs(A, sp, gp, ny, var, grid, block, st);
     if (var >= 3 && var <= 5) return launch_dslash_staged(A, sp, gp, ny, var, grid, block, st);
     if (var == 6 || var == 7) return launch_dslash_multi(A, sp, gp, ny, var, grid, block, st);

@@ -292,13 +292,12 @@ inline dim3 block_grid(int Vh, int bx, int ngroups)
     return dim3((unsigned)(2 * ((Vh + bx - 1) / bx) * ngroups));
 }
 
-// One launcher per precision pair: G::run<SP, GP> for the seven supported (spinor, link) formats.
+// One launcher per precision pair: G::run<SP, GP> for the supported (spinor, link) formats
+// of FP32 arithmetic (FP64 and double-float: dslash_split.cu).
 template <class G>
 cudaError_t dispatch_prec(const DslashArgs& A, int sp, int gp, int ny, int var, dim3 grid, dim3 block,
                           cudaStream_t st)
 {
-    if (sp == P_F64 && gp == P_F64) return G::template run<P_F64, P_F64>(A, ny, var, grid, block, st);
-    if (sp == P_DF64 && gp == P_DF64) return G::template run<P_DF64, P_DF64>(A, ny, var, grid, block, st);
     if (sp == P_F32 && gp == P_F32) return G::template run<P_F32, P_F32>(A, ny, var, grid, block, st);
     if (sp == P_F16 && gp == P_F16) return G::template run<P_F16, P_F16>(A, ny, var, grid, block, st);
     if (sp == P_BF16 && gp == P_BF16) return G::template run<P_BF16, P_BF16>(A, ny, var, grid, block, st);

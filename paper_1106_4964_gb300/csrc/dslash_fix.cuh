@@ -1,0 +1,266 @@
+// Hopping term of FP64 and double-float fields in block fixed point on the integer pipes.
+//
+// GB300 issues 2 FP64 operations per clock and SM against 128 FP32 or 64 integer ones, and a
+// double-float multiply-add is 18 FP32 operations, so a hop's 72 multiply-adds are its cost.  Here each
+// projected half spinor h (12 reals, formed in the field's arithmetic) is written as 64-bit integers in
+// units of 2^-60 of the power of two above its largest component, the link as 64-bit integers in units
+// of 2^-62, and the colour multiply sums 32 x 32 -> 64-bit products: with x = x1 2^32 + x0, x0 in
+// [-2^31, 2^31),
+//   u h / 2^64 = u1 h1 + (u1 h0 + u0 h1) / 2^32 + (u0 h0) / 2^64,
+// the last term below the unit of the result and dropped.  The sum over the eight hops is a 64-bit
+// integer in units of 2^-58 of the largest component met.  Conversions, dropped terms and shifts are
+// each below 2^-54 (double-float) or 2^-57 (FP64) of a hop's largest component, where FP64 rounds every
+// product and partial sum to 2^-53 of itself: relative to the field around the site the sum's error is
+// that of the floating-point sum or smaller.
+//
+// Bounds (|u row| = 1 to 1e-9, |h| < 2^60): sum of |u1 h0| <= sqrt(6) 2^61, sum of |u0 h1| <=
+// 6 x 2^59, together below 2^63; the sum of u1 h1 stays below 2^60; a hop's result is below
+// 2.45 x 2^58, the sum of eight below 2^62.3.
+//
+// What the format does not hold goes to the field's own arithmetic: infinities, NaN, values near the
+// ends of the exponent range, a hop whose nonzero components differ by more than 2^26, hops whose
+// largest components differ by more than 2^16.
+#pragma once
+
+#include <stdint.h>
+
+namespace ov {
+
+struct Fix {
+    int h, l;  // value = h 2^32 + l
+};
+
+__host__ __device__ __forceinline__ uint32_t fix_shr(uint32_t hi, uint32_t lo, uint32_t n)
+{
+    // low word of (hi : lo) >> min(n, 32)
+#ifdef __CUDA_ARCH__
+    return __funnelshift_rc(lo, hi, n);
+#else
+    const uint64_t v = ((uint64_t)hi << 32) | lo;
+    return (uint32_t)(v >> (n < 32 ? n : 32));
+#endif
+}
+
+__host__ __device__ __forceinline__ uint32_t f64_hi(double x)
+{
+#ifdef __CUDA_ARCH__
+    return (uint32_t)__double2hiint(x);
+#else
+    uint64_t b;
+    __builtin_memcpy(&b, &x, 8);
+    return (uint32_t)(b >> 32);
+#endif
+}
+__host__ __device__ __forceinline__ uint32_t f64_lo(double x)
+{
+#ifdef __CUDA_ARCH__
+    return (uint32_t)__double2loint(x);
+#else
+    uint64_t b;
+    __builtin_memcpy(&b, &x, 8);
+    return (uint32_t)b;
+#endif
+}
+__host__ __device__ __forceinline__ double f64_bits(uint32_t hi, uint32_t lo)
+{
+#ifdef __CUDA_ARCH__
+    return __hiloint2double((int)hi, (int)lo);
+#else
+    const uint64_t b = ((uint64_t)hi << 32) | lo;
+    double x;
+    __builtin_memcpy(&x, &b, 8);
+    return x;
+#endif
+}
+
+constexpr uint32_t FIX_EXP = 0x7ff00000u;        // exponent field of a double's high word
+constexpr uint32_t FIX_ELO = 200u << 20;         // exponents the fixed-point path takes
+constexpr uint32_t FIX_EHI = 1900u << 20;
+constexpr uint32_t FIX_SPAN = 26u << 20;         // nonzero components of one hop
+constexpr int FIX_HOPS = 16;                     // largest components of the eight hops, powers of two
+
+// (hi : lo) >> n, arithmetic, n < 32
+__host__ __device__ __forceinline__ long long fix_sar(int hi, int lo, int n)
+{
+    return (long long)(((unsigned long long)(uint32_t)(hi >> n) << 32) | fix_shr((uint32_t)hi, (uint32_t)lo, n));
+}
+
+// x in units of 2^-60 of the power of two above a component of exponent field emax (f <= emax, within
+// FIX_SPAN of it or zero).  Negative values are complemented: one unit low.
+__host__ __device__ __forceinline__ Fix to_fix(double x, uint32_t emax)
+{
+    const uint32_t hw = f64_hi(x), lw = f64_lo(x), f = hw & FIX_EXP;
+    uint32_t mh = fix_shr(hw, lw, 21) | 0x80000000u;  // 53-bit mantissa, left-aligned in mh : ml
+    uint32_t sg = (uint32_t)((int)hw >> 31);
+    const uint32_t ml = lw << 11;
+    if (f == 0) mh = sg = 0;  // zero (a subnormal is below any unit the path uses)
+    const uint32_t d = 4u + ((emax - f) >> 20);
+    const uint32_t hi = fix_shr(0u, mh, d) ^ sg, lo = fix_shr(mh, ml, d) ^ sg;
+    Fix r;
+    r.l = (int)lo;
+    r.h = (int)(hi + (lo >> 31));
+    return r;
+}
+
+// -x (one unit low in the low word)
+__host__ __device__ __forceinline__ Fix fix_neg(Fix x) { return Fix{-x.h, ~x.l}; }
+
+// links: |u| <= 1 in units of 2^-62
+__host__ __device__ __forceinline__ Fix link_to_fix(double u)
+{
+    const long long q = (long long)rint(u * 4611686018427387904.0);
+    Fix r;
+    r.l = (int)(uint32_t)q;
+    r.h = (int)((q - (long long)r.l) >> 32);
+    return r;
+}
+__host__ __device__ __forceinline__ double fix_to_link(Fix a)
+{
+    return (double)a.h * 9.31322574615478515625e-10 + (double)a.l * 2.16840434497100886801490560173988e-19;
+}
+
+struct FixProd {
+    long long hi, mid;
+};
+__host__ __device__ __forceinline__ void fix_mac(FixProd& s, Fix a, Fix b)
+{
+    s.hi += (long long)a.h * b.h;
+    s.mid += (long long)a.h * b.l;
+    s.mid += (long long)a.l * b.h;
+}
+__host__ __device__ __forceinline__ long long fix_sum(const FixProd& s) { return s.hi + (s.mid >> 32); }
+
+// Exponent field of the largest of the 12 components (0: every component is zero or subnormal), FIX_BAD
+// when the format does not hold them
+constexpr uint32_t FIX_BAD = 0xffffffffu;
+__host__ __device__ __forceinline__ uint32_t fix_range(const double h[12])
+{
+    uint32_t emax = 0, emin = 0xffffffffu;
+#pragma unroll
+    for (int i = 0; i < 12; ++i) {
+        const uint32_t f = f64_hi(h[i]) & FIX_EXP;
+        emax = emax > f ? emax : f;
+        emin = emin < f - 1u ? emin : f - 1u;  // zeros wrap to the top
+    }
+    if (emax == 0) {
+        uint32_t any = 0;
+#pragma unroll
+        for (int i = 0; i < 12; ++i) any |= (f64_hi(h[i]) << 1) | f64_lo(h[i]);
+        return any ? FIX_BAD : 0u;
+    }
+    return emax >= FIX_EHI || emax < FIX_ELO || emax - emin > FIX_SPAN + 1u ? FIX_BAD : emax;
+}
+
+// v 2^-1080 2^e (e: exponent field >> 20 of the sum's unit), rounded to nearest
+__host__ __device__ __forceinline__ int fix_clz(unsigned long long m)
+{
+#ifdef __CUDA_ARCH__
+    return __clzll((long long)m);
+#else
+    return m ? __builtin_clzll(m) : 64;
+#endif
+}
+__host__ __device__ __forceinline__ double fix_to_f64(long long v, int e)
+{
+    const unsigned long long sg = (unsigned long long)(v >> 63);
+    unsigned long long m = ((unsigned long long)v ^ sg) - sg;
+    const int lz = fix_clz(m);
+    m = lz < 64 ? m << lz : 0ull;
+    // m 2^-63 in [1, 2): exponent of the value 63 - lz + e - 1080
+    const unsigned long long r = (m >> 11) + ((m >> 10) & 1ull);
+    const unsigned long long bits =
+        r + ((unsigned long long)(uint32_t)(63 - lz + e - 1080 + 1023 - 1) << 52);
+    return lz < 64 ? f64_bits((uint32_t)(bits >> 32) | ((uint32_t)sg & 0x80000000u), (uint32_t)bits) : 0.0;
+}
+
+// ---- double-float: exponent fields are those of the high words (8 bits at bit 23) ----
+constexpr uint32_t FIXD_EXP = 0x7f800000u;
+constexpr uint32_t FIXD_ELO = 74u << 23;
+constexpr uint32_t FIXD_EHI = 250u << 23;
+constexpr uint32_t FIXD_SPAN = 26u << 23;
+
+__host__ __device__ __forceinline__ uint32_t f32_bits(float x)
+{
+#ifdef __CUDA_ARCH__
+    return __float_as_uint(x);
+#else
+    uint32_t b;
+    __builtin_memcpy(&b, &x, 4);
+    return b;
+#endif
+}
+__host__ __device__ __forceinline__ float bits_f32(uint32_t b)
+{
+#ifdef __CUDA_ARCH__
+    return __uint_as_float(b);
+#else
+    float x;
+    __builtin_memcpy(&x, &b, 4);
+    return x;
+#endif
+}
+
+__host__ __device__ __forceinline__ uint32_t fixd_range(const float hi[12], const float lo[12])
+{
+    uint32_t emax = 0, emin = 0xffffffffu;
+#pragma unroll
+    for (int i = 0; i < 12; ++i) {
+        const uint32_t f = f32_bits(hi[i]) & FIXD_EXP;
+        emax = emax > f ? emax : f;
+        emin = emin < f - 1u ? emin : f - 1u;  // zeros wrap to the top
+    }
+    if (emax == 0) {
+        uint32_t any = 0;
+#pragma unroll
+        for (int i = 0; i < 12; ++i) any |= (f32_bits(hi[i]) | f32_bits(lo[i])) << 1;
+        return any ? FIX_BAD : 0u;
+    }
+    return emax >= FIXD_EHI || emax < FIXD_ELO || emax - emin > FIXD_SPAN + 1u ? FIX_BAD : emax;
+}
+
+__host__ __device__ __forceinline__ Fix fixd_to_fix(float xh, float xl, uint32_t emax)
+{
+    const uint32_t hb = f32_bits(xh), lb = f32_bits(xl), f = hb & FIXD_EXP, fl = lb & FIXD_EXP;
+    uint32_t m = ((hb << 4) & 0x07fffff0u) | 0x08000000u;  // 24-bit mantissa, units of 2^32 below 2^60
+    uint32_t sg = (uint32_t)((int)hb >> 31);
+    if (f == 0) m = sg = 0;
+    const uint32_t d = (emax - f) >> 23;
+    long long x = (long long)(((unsigned long long)(fix_shr(0u, m, d) ^ sg) << 32) | (fix_shr(m, 0u, d) ^ sg));
+    // low word, in units of 2^8 (2^-52 of the hop's largest component): at most 2^-21 of that component,
+    // so that a pair whose low word exceeds half a unit of its high word by a few bits is taken too
+    const uint32_t ml = ((lb << 7) & 0x3fffff80u) | 0x40000000u;
+    const uint32_t q = ((emax - fl) >> 23) - 21u;
+    int l = (int)fix_shr(0u, ml, q);
+    if (fl == 0) l = 0;
+    l = (int)lb < 0 ? -l : l;
+    x += (long long)l * 256;
+    Fix r;
+    r.l = (int)(uint32_t)x;
+    r.h = (int)((uint32_t)(x >> 32) + ((uint32_t)r.l >> 31));
+    return r;
+}
+
+// v 2^-184 2^e as a normalised pair (24 + 24 significand bits)
+__host__ __device__ __forceinline__ void fixd_from_fix(long long v, int e, float& hi, float& lo)
+{
+    const unsigned long long sg = (unsigned long long)(v >> 63);
+    unsigned long long m = ((unsigned long long)v ^ sg) - sg;
+    const int lz = fix_clz(m);
+    m = lz < 64 ? m << lz : 0ull;
+    const int ex = 63 - lz + e - 184 + 127;  // biased exponent of the value
+    const uint32_t s = (uint32_t)sg & 0x80000000u;
+    const uint32_t top = (uint32_t)(m >> 32);
+    const float h0 = bits_f32(((uint32_t)ex << 23) + ((top >> 8) & 0x007fffffu) | s);
+    // the next 24 bits: (1.f - 1) forms of units of 2^(ex - 24)
+    const uint32_t rest = (uint32_t)(m >> 16) & 0x00ffffffu;
+    const float u = bits_f32((uint32_t)(ex - 23) << 23);  // 2^(value exponent - 23): one unit of h0's last place
+    const float l0 = (float)(int)rest * 5.9604644775390625e-8f * (s ? -u : u);
+    if (lz >= 64) {
+        hi = lo = 0.f;
+        return;
+    }
+    hi = h0 + l0;
+    lo = l0 - (hi - h0);
+}
+
+}  // namespace ov

@@ -17,7 +17,8 @@
 // Gauge links: forward links only; FP32 and 16-bit keep only rows 0 and 1 of
 // each SU(3) matrix (reconstruct-12): link[p][mu][k][s] = U_mu(n), n = site (p, s); chunks
 // are 3 float4 (FP32) or 3 x 4 16-bit values; FP64 and double-float keep all
-// three rows, 9 double2 (FP64) or 9 float4 (hi, lo, hi, lo).
+// three rows as 64-bit fixed point (dslash_fix.cuh), 9 int4 (re high, re low, im high,
+// im low), one copy for both.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -28,6 +29,8 @@
 #include <type_traits>
 
 #include <string>
+
+#include "dslash_fix.cuh"
 
 namespace ov {
 
@@ -399,21 +402,13 @@ __device__ __forceinline__ void store_spinor(char* __restrict__ base, float* __r
 template <int P, typename Real>
 __device__ __forceinline__ void load_link_rows(const char* __restrict__ base, int Vh, int s, Real u[18])
 {
-    if constexpr (P == P_DF64) {
-        const float4* b = reinterpret_cast<const float4*>(base);
+    if constexpr (P == P_DF64 || P == P_F64) {
+        const int4* b = reinterpret_cast<const int4*>(base);
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            float4 t = __ldg(b + (size_t)k * Vh + s);
-            u[2 * k] = from_df<Real>(df64(t.x, t.y));
-            u[2 * k + 1] = from_df<Real>(df64(t.z, t.w));
-        }
-    } else if constexpr (P == P_F64) {
-        const double2* b = reinterpret_cast<const double2*>(base);
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            double2 t = __ldg(b + (size_t)k * Vh + s);
-            u[2 * k] = (Real)t.x;
-            u[2 * k + 1] = (Real)t.y;
+            const int4 t = __ldg(b + (size_t)k * Vh + s);
+            u[2 * k] = (Real)fix_to_link(Fix{t.x, t.y});
+            u[2 * k + 1] = (Real)fix_to_link(Fix{t.z, t.w});
         }
     } else if constexpr (P == P_F32) {
         const float4* b = reinterpret_cast<const float4*>(base);
@@ -478,21 +473,13 @@ template <int P, typename Real>
 __device__ __forceinline__ void load_link(const char* __restrict__ base, int Vh, int s, Real u[18])
 {
     load_link_rows<P, Real>(base, Vh, s, u);
-    if constexpr (P == P_DF64) {  // stored third row (9 chunks per link)
-        const float4* b = reinterpret_cast<const float4*>(base);
+    if constexpr (P == P_DF64 || P == P_F64) {  // stored third row (9 chunks per link)
+        const int4* b = reinterpret_cast<const int4*>(base);
 #pragma unroll
         for (int k = 6; k < 9; ++k) {
-            float4 t = __ldg(b + (size_t)k * Vh + s);
-            u[2 * k] = from_df<Real>(df64(t.x, t.y));
-            u[2 * k + 1] = from_df<Real>(df64(t.z, t.w));
-        }
-    } else if constexpr (P == P_F64) {  // stored third row (9 chunks per link)
-        const double2* b = reinterpret_cast<const double2*>(base);
-#pragma unroll
-        for (int k = 6; k < 9; ++k) {
-            double2 t = __ldg(b + (size_t)k * Vh + s);
-            u[2 * k] = (Real)t.x;
-            u[2 * k + 1] = (Real)t.y;
+            const int4 t = __ldg(b + (size_t)k * Vh + s);
+            u[2 * k] = (Real)fix_to_link(Fix{t.x, t.y});
+            u[2 * k + 1] = (Real)fix_to_link(Fix{t.z, t.w});
         }
     } else {
         link_row2<Real>(u);

@@ -21,6 +21,7 @@ struct DslashArgs {
     double a, b;                 // core = a psi(n) + b * sum of hops
     double sy[3];
     float fa, fb, fsy[3];        // the same coefficients for FP32 arithmetic
+    float2 da, db, dsy[3];       // and as double-float pairs (hi, lo)
     int nrhs;
     int g5_core, g5_out;
     unsigned* err;               // set to 1 when a bounded wait of a staged variant times out
@@ -36,6 +37,7 @@ constexpr long long DSLASH_WAIT_POLLS = 1ll << 22;  // default first-wait limit 
 cudaError_t launch_dslash(const DslashArgs& A, int sp, int gp, int ny, int bx, int by, int var, cudaStream_t st);
 // the variant groups, one translation unit each (grid and block already derived from bx, by)
 cudaError_t launch_dslash_regs(const DslashArgs& A, int sp, int gp, int ny, int var, dim3 grid, dim3 block, cudaStream_t st);
+cudaError_t launch_dslash_split(const DslashArgs& A, int sp, int gp, int ny, int var, int bx, int by, cudaStream_t st);
 cudaError_t launch_dslash_staged(const DslashArgs& A, int sp, int gp, int ny, int var, dim3 grid, dim3 block,
                                  cudaStream_t st);
 cudaError_t launch_dslash_multi(const DslashArgs& A, int sp, int gp, int ny, int var, dim3 grid, dim3 block, cudaStream_t st);

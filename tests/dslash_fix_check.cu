@@ -1,0 +1,99 @@
+// Host-side check of the fixed-point hop (dslash_fix.cuh) against 80-bit sums: one row of the colour
+// multiply for random unit rows and half spinors over the exponent range, with zero components, with
+// every component at the bound, and the conversions to and from FP64 and double-float.  Prints "ok" or
+// the first failure.
+#include <cmath>
+#include <cstdio>
+#include <random>
+
+#include "dslash_fix.cuh"
+
+using namespace ov;
+
+static int fail(const char* what, double a, double b)
+{
+    std::printf("%s: %.17g %.17g\n", what, a, b);
+    return 1;
+}
+
+int main()
+{
+    std::mt19937_64 g(1);
+    std::normal_distribution<double> n;
+    for (int t = 0; t < 200000; ++t) {
+        double u[6], nn = 0, h[12], mx = 0;
+        for (double& x : u) {
+            x = t % 4 == 0 ? (g() % 2 ? 1.0 : -1.0) : n(g);  // every entry equal: the largest product sums
+            nn += x * x;
+        }
+        for (double& x : u) x /= std::sqrt(nn);
+        const double sc = std::ldexp(1.0, (int)(g() % 1600) - 800);
+        for (double& x : h) x = (t % 4 < 2 ? (g() % 2 ? 1.0 : -1.0) * (2.0 - 4e-16) : n(g)) * sc * (t % 3 == 0 && g() % 5 == 0 ? 0.0 : 1.0);
+        for (double x : h) mx = std::fmax(mx, std::fabs(x));
+        if (mx == 0) continue;
+        const uint32_t em = fix_range(h);
+        if (em == FIX_BAD) {
+            double mn = mx;
+            for (double x : h)
+                if (x != 0) mn = std::fmin(mn, std::fabs(x));
+            if (mn * 33554432.0 > mx) return fail("refused", mn, mx);
+            continue;
+        }
+        FixProd re{}, im{};
+        long double rr = 0, ri = 0;
+        for (int j = 0; j < 3; ++j) {
+            const Fix ur = link_to_fix(u[2 * j]), ui = link_to_fix(u[2 * j + 1]);
+            const Fix a = to_fix(h[2 * j], em), b = to_fix(h[2 * j + 1], em);
+            if (std::fabs(fix_to_link(ur) - u[2 * j]) > 1.2e-16 * std::fabs(u[2 * j]) + 2.2e-19) return fail("link", fix_to_link(ur), u[2 * j]);
+            fix_mac(re, ur, a);
+            fix_mac(re, ui, fix_neg(b));
+            fix_mac(im, ur, b);
+            fix_mac(im, ui, a);
+            rr += (long double)u[2 * j] * h[2 * j] - (long double)u[2 * j + 1] * h[2 * j + 1];
+            ri += (long double)u[2 * j] * h[2 * j + 1] + (long double)u[2 * j + 1] * h[2 * j];
+        }
+        // 2^-55 of the largest component: half an FP64 rounding of one product of that size
+        const int e = (int)(em >> 20);
+        for (int k = 0; k < 2; ++k) {
+            const long long v = fix_sum(k ? im : re);
+            const long double ex = ldexpl((long double)v, e - 1080), ref = k ? ri : rr;
+            if (fabsl(ex - ref) > ldexpl(mx, -55)) return fail("row", (double)ex, (double)ref);
+            if (fabsl(fix_to_f64(v, e) - ex) > ldexpl(fabsl(ex), -53)) return fail("to f64", fix_to_f64(v, e), (double)ex);
+            const int sh = (int)(g() % 32);
+            if (fix_sar((int)(v >> 32), (int)v, sh) != (v >> sh)) return fail("shift", (double)v, sh);
+            // double-float result: 47 significand bits, low word at most half a unit of the high one
+            float a, b;
+            const int ed = 80 + (int)(g() % 160);
+            fixd_from_fix(v, ed, a, b);
+            const long double tv = ldexpl((long double)v, ed - 184);
+            if (fabsl((long double)a + b - tv) > ldexpl(fabsl(tv), -47) || std::fabs(b) > std::ldexp(std::fabs(a), -24))
+                return fail("to df", a, (double)tv);
+        }
+        // double-float input
+        float hh[12], hl[12], m = 0;
+        for (int i = 0; i < 12; ++i) {
+            const double x = std::ldexp(h[i] / sc, (int)(t % 101) - 40);
+            hh[i] = (float)x;
+            hl[i] = (float)(x - hh[i]);
+            m = std::fmax(m, std::fabs(hh[i]));
+        }
+        const uint32_t ed = fixd_range(hh, hl);
+        if (ed == FIX_BAD) return fail("df refused", m, 0);
+        for (int i = 0; i < 12; ++i) {
+            const Fix f = fixd_to_fix(hh[i], hl[i], ed);
+            const long double val = ldexpl((long double)(f.h * 4294967296.0L + f.l), (int)(ed >> 23) - 186);
+            if (fabsl(val - ((long double)hh[i] + hl[i])) > ldexpl(m, -50)) return fail("from df", hh[i], (double)val);
+        }
+    }
+    double z[12] = {};
+    if (fix_range(z) != 0) return fail("zero", 0, 0);
+    z[3] = 5e-324;
+    if (fix_range(z) != FIX_BAD) return fail("subnormal", 0, 0);
+    z[3] = INFINITY;
+    if (fix_range(z) != FIX_BAD) return fail("inf", 0, 0);
+    z[3] = NAN;
+    if (fix_range(z) != FIX_BAD) return fail("nan", 0, 0);
+    if (fix_to_f64(0, 1000) != 0.0 || fix_to_f64(-1, 1080) != -1.0) return fail("to f64 ends", 0, 0);
+    std::printf("ok\n");
+    return 0;
+}

@@ -1,0 +1,105 @@
+"""The FP64 and double-float dslash at the edges of its fixed-point hop: fields whose neighbouring
+sites differ by many orders of magnitude, vanishing neighbours and components, infinities and NaN,
+scales near the ends of the exponent range, and every launch variant on ragged site groups."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from gpu_common import ABC, RHO, TOL, dev, host, need_gpu, rel, torch
+
+pytestmark = pytest.mark.gpu
+
+DIMS = (6, 4, 4, 6)
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    need_gpu()
+
+
+def apply(prec, U, psi, dims=DIMS):
+    from paper_1106_4964_gb300 import Context
+
+    ctx = Context(dims, ABC)
+    ctx.set_gauge(dev(U))
+    out = torch.empty_like(dev(psi))
+    ctx.apply_dslash(dev(psi), out, -RHO, prec=prec)
+    return host(out)
+
+
+def fields():
+    rng = np.random.default_rng(7)
+    base = synth.gaussian_spinor(DIMS, 2)
+    site = 2.0 ** rng.integers(-40, 41, base.shape[:5])[..., None, None]
+    comp = 2.0 ** rng.integers(-35, 36, base.shape)
+    colour0 = base.copy()
+    colour0[..., 1:] = 0  # zero components in every neighbour
+    sector = base.copy()
+    sector[..., 2:, :] = 0
+    return {"site_scales": base * site, "component_scales": base * comp, "one_colour": colour0,
+            "one_chirality": sector, "point": synth.point_sources(DIMS)[4:5], "zero": np.zeros_like(base)}
+
+
+@pytest.mark.parametrize("name", sorted(fields()))
+@pytest.mark.parametrize("prec", ["f64", "df64"])
+def test_uneven_fields(prec, name):
+    """Site by site: the error relative to the largest of the nine spinors a site reads."""
+    U = synth.gauge_field(DIMS, 1, 0.5)
+    psi = fields()[name]
+    got = apply(prec, U, psi)[0]
+    ref = oracle.dslash(DIMS, ABC, U, -RHO, psi).reshape(got.shape)
+    mag = np.abs(psi[0]).max(axis=(-2, -1))
+    near = mag.copy()
+    for ax in range(4):
+        near = np.maximum(near, np.maximum(np.roll(mag, 1, ax), np.roll(mag, -1, ax)))
+    err = np.abs(got - ref).max(axis=(-2, -1))
+    assert np.all(err <= TOL[prec] * near)
+    if name == "zero":
+        assert not got.any()
+
+
+@pytest.mark.parametrize("prec,scale", [("f64", 1e-290), ("f64", 1e-200), ("f64", 1e290), ("df64", 1e-20), ("df64", 1e30)])
+def test_scales(prec, scale):
+    U = synth.gauge_field(DIMS, 1, 0.5)
+    psi = synth.gaussian_spinor(DIMS, 2)
+    got = apply(prec, U, psi * scale) / scale
+    assert rel(got, oracle.dslash(DIMS, ABC, U, -RHO, psi)) <= TOL[prec]
+
+
+@pytest.mark.parametrize("prec", ["f64", "df64"])
+@pytest.mark.parametrize("value", [np.inf, np.nan])
+def test_non_finite(prec, value):
+    """One non-finite component: its site and the eight neighbours get non-finite components, every
+    other site its value."""
+    U = synth.gauge_field(DIMS, 1, 0.5)
+    psi = synth.gaussian_spinor(DIMS, 2)
+    ref = oracle.dslash(DIMS, ABC, U, -RHO, psi).reshape(psi.shape)[0]
+    psi[0, 2, 1, 3, 4, 1, 2] = value
+    got = apply(prec, U, psi)[0]
+    bad = ~np.isfinite(got).all(axis=(-2, -1))
+    want = np.zeros_like(bad)
+    want[2, 1, 3, 4] = True
+    for ax in range(4):
+        for st in (1, -1):
+            want |= np.roll((np.indices(want.shape) == np.array([2, 1, 3, 4]).reshape(4, 1, 1, 1, 1)).all(0), st, ax)
+    assert np.array_equal(bad, want)
+    assert rel(got[~bad], ref[~bad]) <= TOL[prec]
+
+
+@pytest.mark.parametrize("shape", [(32, 1, 0), (32, 3, 1), (64, 2, 2), (256, 1, 1)])
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (2, 6, 4, 10), (6, 4, 4, 6)])
+@pytest.mark.parametrize("prec", ["f64", "df64"])
+def test_launch_shapes(prec, dims, shape):
+    from paper_1106_4964_gb300 import Context
+
+    U = synth.gauge_field(dims, 5, 0.5)
+    psi = synth.gaussian_spinor(dims, 6, nrhs=4)
+    ctx = Context(dims, ABC)
+    ctx.set_gauge(dev(U))
+    ctx.set_dslash_shape(prec, 4, *shape)
+    out = torch.empty_like(dev(psi))
+    ctx.apply_dslash(dev(psi), out, -RHO, prec=prec)
+    got = host(out)
+    for r in range(4):
+        assert rel(got[r], oracle.dslash(dims, ABC, U, -RHO, psi[r])) <= TOL[prec]
