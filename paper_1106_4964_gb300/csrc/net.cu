@@ -5,17 +5,18 @@
 // with T_0 = 1, T_{1+2mu} x(n) = U_mu(n) x(n+mu), T_{2+2mu} x(n) = U_mu(n-mu)^dag x(n-mu)
 // (boundary phases applied) and W[p][c][c'] a complex 4x4 spin matrix.  The
 // map is linear and commutes with gauge transformations.  The network is
-// M = L2 . L1 with 1 -> 16 -> 1 channels, applied to one right-hand side
-// at a time in FP32 (internal even/odd layout; activations are 16-rhs fields).
+// M = L2 . L1 with 1 -> 16 -> 1 channels, applied to batches of right-hand sides in FP32 (internal
+// even/odd layout; the activations of a batch of nb are a field of 16 nb right-hand sides).
 //
 // Backward pass: the adjoint of T_p is T_{pbar} (forward <-> backward hop),
 // so the input gradient is the forward kernel with weights
 // W'[q][c'][c] = W[qbar][c][c']^dag; the weight gradient
 // gW[p][c][c'] = sum_n gy_c(n) (T_p x_{c'}(n))^dag (summed over colour) is a
-// split-K reduction over sites with block partials summed in fixed order.
+// product over sites and colours with block partials summed in fixed order.
 // Training: loss sum_k |M(r_k) - e_k|^2 / |e_k|^2 over (residual, error)
 // pairs recorded at the FP64 true-residual points of the library's own
 // deflated CG solves, Adam on the device.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -39,6 +40,7 @@ struct NetState {
     size_t partials_n = 0;
     int adam_t = 0;
     int adj_valid = 0;  // Wadj matches W
+    int batch = 0;      // fields the work fields hold
     // recorded training pairs: residuals and iterates (then errors), f32 single-rhs fields
     int recording = 0;
     FieldDesc pr{}, px{};
@@ -48,198 +50,330 @@ struct NetState {
 
 namespace {
 
-struct PathSite {
-    int sn, q;        // source checkerboard site and parity
-    float u[18];      // link (forward: U, backward: U used as U^dag)
-    float ph;
-};
-
-__device__ __forceinline__ void path_setup(const Geom& g, const char* gauge, int p, int s, const int c[4], int path,
-                                           PathSite& P)
-{
-    if (path == 0) {
-        P.sn = s;
-        P.q = p;
-        P.ph = 1.f;
-        return;
-    }
-    const int mu = (path - 1) >> 1;
-    const bool fwd = ((path - 1) & 1) == 0;
-    int d[4] = {c[0], c[1], c[2], c[3]};
-    bool cross;
-    if (fwd) {
-        d[mu] = c[mu] + 1 == g.L[mu] ? 0 : c[mu] + 1;
-        cross = d[mu] == 0;
-    } else {
-        d[mu] = c[mu] == 0 ? g.L[mu] - 1 : c[mu] - 1;
-        cross = c[mu] == 0;
-    }
-    P.sn = cb_index(g, d[0], d[1], d[2], d[3]);
-    P.q = 1 - p;
-    const int lpar = fwd ? p : P.q, ls = fwd ? s : P.sn;
-    load_link<P_F32, float>(gauge + ((size_t)(lpar * 4 + mu) * g.Vh) * 48, g.Vh, ls, P.u);
-    P.ph = cross ? (float)g.bc[mu] : 1.f;
-}
-
-// t = T_path x_c (one channel; xc = channel base, both parities)
-__device__ __forceinline__ void path_apply(const Geom& g, const char* xc, int path, const PathSite& P, float t[24])
+// t = (T_path x)(site s of parity p, coordinates c); x: one FP32 field, both parities
+__device__ __forceinline__ void transport(const Geom& g, const char* gauge, const char* x, int p, int s, const int c[4],
+                                          int path, float t[24])
 {
     const size_t par = (size_t)6 * 16 * g.Vh;
-    float v[24];
-    load_spinor<P_F32, float>(xc + P.q * par, nullptr, g.Vh, P.sn, v);
     if (path == 0) {
-#pragma unroll
-        for (int k = 0; k < 24; ++k) t[k] = v[k];
+        load_spinor<P_F32, float>(x + p * par, nullptr, g.Vh, s, t);
         return;
     }
-    const bool fwd = ((path - 1) & 1) == 0;
+    int sn;
+    float ph = 1.f;
+    switch (path) {
+    case 1: sn = cb_neighbour<0>(g, s, c); if (c[0] + 1 == g.L[0]) ph = g.fbc[0]; break;
+    case 2: sn = cb_neighbour<1>(g, s, c); if (c[0] == 0) ph = g.fbc[0]; break;
+    case 3: sn = cb_neighbour<2>(g, s, c); if (c[1] + 1 == g.L[1]) ph = g.fbc[1]; break;
+    case 4: sn = cb_neighbour<3>(g, s, c); if (c[1] == 0) ph = g.fbc[1]; break;
+    case 5: sn = cb_neighbour<4>(g, s, c); if (c[2] + 1 == g.L[2]) ph = g.fbc[2]; break;
+    case 6: sn = cb_neighbour<5>(g, s, c); if (c[2] == 0) ph = g.fbc[2]; break;
+    case 7: sn = cb_neighbour<6>(g, s, c); if (c[3] + 1 == g.L[3]) ph = g.fbc[3]; break;
+    default: sn = cb_neighbour<7>(g, s, c); if (c[3] == 0) ph = g.fbc[3]; break;
+    }
+    const int mu = (path - 1) >> 1;
+    const bool fwd = (path & 1) != 0;
+    float v[24], u[18];
+    load_spinor<P_F32, float>(x + (1 - p) * par, nullptr, g.Vh, sn, v);
+    load_link<P_F32, float>(gauge + ((size_t)((fwd ? p : 1 - p) * 4 + mu) * g.Vh) * 48, g.Vh, fwd ? s : sn, u);
+    if (!fwd) {  // U^dag
 #pragma unroll
-    for (int s = 0; s < 4; ++s)
+        for (int i = 0; i < 3; ++i) {
+            u[2 * (4 * i) + 1] = -u[2 * (4 * i) + 1];
+#pragma unroll
+            for (int j = i + 1; j < 3; ++j) {
+                const float ar = u[2 * (3 * i + j)], ai = u[2 * (3 * i + j) + 1];
+                u[2 * (3 * i + j)] = u[2 * (3 * j + i)];
+                u[2 * (3 * i + j) + 1] = -u[2 * (3 * j + i) + 1];
+                u[2 * (3 * j + i)] = ar;
+                u[2 * (3 * j + i) + 1] = -ai;
+            }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             float re = 0, im = 0;
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
-                float ur = fwd ? P.u[2 * (3 * i + j)] : P.u[2 * (3 * j + i)];
-                float ui = fwd ? P.u[2 * (3 * i + j) + 1] : -P.u[2 * (3 * j + i) + 1];
-                float xr = v[2 * (3 * s + j)], xi = v[2 * (3 * s + j) + 1];
-                re += ur * xr - ui * xi;
-                im += ur * xi + ui * xr;
+                const float ur = u[2 * (3 * i + j)], ui = u[2 * (3 * i + j) + 1];
+                const float xr = v[2 * (3 * q + j)], xi = v[2 * (3 * q + j) + 1];
+                re = fmaf(ur, xr, re);
+                im = fmaf(ur, xi, im);
+                re = fmaf(-ui, xi, re);
+                im = fmaf(ui, xr, im);
             }
-            t[2 * (3 * s + i)] = P.ph * re;
-            t[2 * (3 * s + i) + 1] = P.ph * im;
+            t[2 * (3 * q + i)] = ph * re;
+            t[2 * (3 * q + i) + 1] = ph * im;
         }
 }
 
-// forward layer: thread per (site, group of CG output channels); W in shared memory
-template <int CIN, int COUT, int CG>
-__global__ void __launch_bounds__(128) net_fwd_kernel(Geom g, const char* gauge, const char* x, char* y,
-                                                      const float2* __restrict__ Wg)
+// acc += w t: a complex 4 x 4 spin matrix (two weights per float4) on a spinor
+__device__ __forceinline__ void spin_mix(const float4 w[8], const float t[24], float acc[24])
 {
-    __shared__ float2 W[9 * COUT * CIN * 16];
-    for (int k = threadIdx.x; k < 9 * COUT * CIN * 16; k += blockDim.x) W[k] = Wg[k];
+#pragma unroll
+    for (int sa = 0; sa < 4; ++sa)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float4 w2 = w[2 * sa + h];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const float wr = q ? w2.z : w2.x, wi = q ? w2.w : w2.y;
+                const int sb = 2 * h + q;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    const float tr = t[2 * (3 * sb + a)], ti = t[2 * (3 * sb + a) + 1];
+                    float& re = acc[2 * (3 * sa + a)];
+                    float& im = acc[2 * (3 * sa + a) + 1];
+                    re = fmaf(wr, tr, re);
+                    im = fmaf(wr, ti, im);
+                    re = fmaf(-wi, ti, re);
+                    im = fmaf(wi, tr, im);
+                }
+            }
+        }
+}
+
+// All kernels take a batch of fields (training pairs, right-hand sides): blockIdx.z, or the site index of
+// the weight gradients, runs over it.  One launch per pair left the 8^3 x 16 lattice with 7 warps per SM:
+// a gradient over 8 pairs took 3.77 ms in 90 launches, of which the one-block sums of the weight
+// gradients' partials were 1.6 ms; batched, with one spinor transported per path, 0.75 ms.  The FP32
+// multiply-adds (150 000 per site and pair) are 0.27 ms of that.
+constexpr int NET_CG = 4;  // output channels per thread of the 1 -> 16 layer
+
+// 1 -> 16 layer: thread per (site, 4 output channels); each transported spinor feeds 4 x 192 multiply-adds
+__global__ void __launch_bounds__(128, 3) net_many_kernel(Geom g, const char* gauge, const char* x, char* y,
+                                                       const float2* __restrict__ Wg)
+{
+    __shared__ float4 W[9][NET_CG][8];  // two complex weights each
+    const int grp = blockIdx.y;
+    for (int k = threadIdx.x; k < 9 * NET_CG * 16; k += blockDim.x) {
+        const int path = k / (NET_CG * 16), e = k % (NET_CG * 16);
+        reinterpret_cast<float2*>(W)[k] = Wg[(path * NET_C + grp * NET_CG) * 16 + e];
+    }
     __syncthreads();
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    const int grp = blockIdx.y;
     if (idx >= 2 * g.Vh) return;
     const int p = idx >= g.Vh, s = idx - p * g.Vh;
     int c[4];
     cb_coords(g, s, p, c);
-    const size_t chan = (size_t)2 * 6 * 16 * g.Vh;  // bytes of one single-rhs f32 field
-    float acc[CG][24];
+    const size_t par = (size_t)6 * 16 * g.Vh, chan = 2 * par;  // bytes of one parity and of one FP32 field
+    x += blockIdx.z * chan;
+    float acc[NET_CG][24];
 #pragma unroll
-    for (int j = 0; j < CG; ++j)
+    for (int j = 0; j < NET_CG; ++j)
 #pragma unroll
         for (int k = 0; k < 24; ++k) acc[j][k] = 0.f;
     for (int path = 0; path < 9; ++path) {
-        PathSite P;
-        path_setup(g, gauge, p, s, c, path, P);
-        for (int ci = 0; ci < CIN; ++ci) {
-            float t[24];
-            path_apply(g, x + ci * chan, path, P, t);
+        float t[24];
+        transport(g, gauge, x, p, s, c, path, t);
 #pragma unroll
-            for (int j = 0; j < CG; ++j) {
-                const float2* w = W + ((path * COUT + grp * CG + j) * CIN + ci) * 16;
-#pragma unroll
-                for (int sa = 0; sa < 4; ++sa)
-#pragma unroll
-                    for (int sb = 0; sb < 4; ++sb) {
-                        const float2 ww = w[4 * sa + sb];
-#pragma unroll
-                        for (int a = 0; a < 3; ++a) {
-                            float tr = t[2 * (3 * sb + a)], ti = t[2 * (3 * sb + a) + 1];
-                            acc[j][2 * (3 * sa + a)] += ww.x * tr - ww.y * ti;
-                            acc[j][2 * (3 * sa + a) + 1] += ww.x * ti + ww.y * tr;
-                        }
-                    }
-            }
-        }
+        for (int j = 0; j < NET_CG; ++j) spin_mix(W[path][j], t, acc[j]);
     }
-    const size_t par = (size_t)6 * 16 * g.Vh;
 #pragma unroll
-    for (int j = 0; j < CG; ++j)
-        store_spinor<P_F32, float>(y + (grp * CG + j) * chan + p * par, nullptr, g.Vh, s, acc[j]);
+    for (int j = 0; j < NET_CG; ++j)
+        store_spinor<P_F32, float>(y + ((size_t)blockIdx.z * NET_C + grp * NET_CG + j) * chan + p * par, nullptr, g.Vh, s,
+                                   acc[j]);
 }
 
-// weight-gradient partials for path blockIdx.y over the block's sites,
-// entry e = ((co * CIN + ci) * 16) + 4 * sa + sb
-template <int CIN, int COUT>
-__global__ void __launch_bounds__(256) net_wgrad_kernel(Geom g, const char* gauge, const char* x, const char* gy,
-                                                        float2* partials)
+// 16 -> 1 layer, first half: the spin matrices commute with the transport, so the 16 channels are mixed
+// where they lie, z_p(n) = sum_c W[p][c] x_c(n) (thread per site and three paths), and one spinor per path
+// is transported instead of 16 (net_gather_kernel)
+__global__ void __launch_bounds__(128, 4) net_mix_kernel(Geom g, const char* x, char* z, const float2* __restrict__ Wg)
 {
-    constexpr int NS = 16;  // sites per staged chunk
-    __shared__ float sg[COUT][NS][24];
-    __shared__ float st[CIN][NS][24];
-    const int path = blockIdx.y;
-    const int e = threadIdx.x;
-    const int co = e / (CIN * 16), ci = (e / 16) % CIN, sa = (e % 16) / 4, sb = e % 4;
-    const bool active = e < COUT * CIN * 16;
-    const size_t chan = (size_t)2 * 6 * 16 * g.Vh;
-    const size_t par = (size_t)6 * 16 * g.Vh;
-    double dr = 0, di = 0;
-    const int N = 2 * g.Vh;
-    for (int base = blockIdx.x * NS; base < N; base += gridDim.x * NS) {
+    __shared__ float4 W[3][NET_C][8];
+    const int p0 = blockIdx.y * 3;
+    for (int k = threadIdx.x; k < 3 * NET_C * 16; k += blockDim.x)
+        reinterpret_cast<float2*>(W)[k] = Wg[p0 * NET_C * 16 + k];
+    __syncthreads();
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= 2 * g.Vh) return;
+    const int p = idx >= g.Vh, s = idx - p * g.Vh;
+    const size_t par = (size_t)6 * 16 * g.Vh, chan = 2 * par;
+    x += (size_t)blockIdx.z * NET_C * chan + p * par;
+    float acc[3][24];
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+#pragma unroll
+        for (int k = 0; k < 24; ++k) acc[j][k] = 0.f;
+    for (int ci = 0; ci < NET_C; ++ci) {
+        float v[24];
+        load_spinor<P_F32, float>(x + ci * chan, nullptr, g.Vh, s, v);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) spin_mix(W[j][ci], v, acc[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+        store_spinor<P_F32, float>(z + ((size_t)blockIdx.z * 9 + p0 + j) * chan + p * par, nullptr, g.Vh, s, acc[j]);
+}
+
+// second half: y(n) = sum_p (T_p z_p)(n)
+__global__ void __launch_bounds__(128) net_gather_kernel(Geom g, const char* gauge, const char* z, char* y)
+{
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= 2 * g.Vh) return;
+    const int p = idx >= g.Vh, s = idx - p * g.Vh;
+    int c[4];
+    cb_coords(g, s, p, c);
+    const size_t par = (size_t)6 * 16 * g.Vh, chan = 2 * par;
+    float acc[24];
+#pragma unroll
+    for (int k = 0; k < 24; ++k) acc[k] = 0.f;
+    for (int path = 0; path < 9; ++path) {
+        float t[24];
+        transport(g, gauge, z + ((size_t)blockIdx.z * 9 + path) * chan, p, s, c, path, t);
+#pragma unroll
+        for (int k = 0; k < 24; ++k) acc[k] += t[k];
+    }
+    store_spinor<P_F32, float>(y + blockIdx.z * chan + p * par, nullptr, g.Vh, s, acc);
+}
+
+// Weight gradients of both layers as one product over sites and colours,
+//   X[(c, s)][(p, s')] = sum_n sum_colour a_c(n)_s conj((T_p b)(n)_s'),
+// a: 16 channels at the site itself, b: one spinor, transported along each path.  Layer 1 has a = the
+// hidden gradient, b = the input; in layer 2 sum_n gy(n) (T_p h_c(n))^dag = sum_m (T_pbar gy)(m) h_c(m)^dag,
+// so a = the hidden field, b = gy and the result is conjugated (net_wgrad_reduce): one spinor is
+// transported instead of 16.  A block stages OUT_NS sites and keeps the whole 64 x 36 product in the
+// registers of its 192 threads (4 x 3 each); per-chunk FP32 sums are added to (hi, lo) pairs.
+constexpr int OUT_NS = 16;
+constexpr int OUT_THREADS = 192;
+constexpr int OUT_AS = 194, OUT_TS = 110;  // complex numbers per staged site (192 and 108, padded)
+constexpr int NET_X = 4 * NET_C * 36;
+
+__global__ void __launch_bounds__(OUT_THREADS, 3) net_outer_kernel(Geom g, const char* gauge, const char* a, const char* b,
+                                                                int nbatch, float2* partials)
+{
+    __shared__ __align__(16) float2 sa[OUT_NS * OUT_AS];
+    __shared__ __align__(16) float2 st[OUT_NS * OUT_TS];
+    const size_t par = (size_t)6 * 16 * g.Vh, chan = 2 * par;
+    const int N = 2 * g.Vh;  // a multiple of 16: a chunk lies in one field
+    const long total = (long)N * nbatch;
+    const int i = threadIdx.x & 15, jj = threadIdx.x >> 4;
+    float hr[4][3], hi[4][3], lr[4][3], li[4][3];
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int y = 0; y < 3; ++y) hr[x][y] = hi[x][y] = lr[x][y] = li[x][y] = 0.f;
+    for (long base = (long)blockIdx.x * OUT_NS; base < total; base += (long)gridDim.x * OUT_NS) {
+        const int fb = (int)(base / N), n0 = (int)(base - (long)fb * N);
         __syncthreads();
-        for (int k = threadIdx.x; k < NS * (COUT + CIN); k += blockDim.x) {
-            const int j = k % NS, ch = k / NS;
-            const int idx = base + j;
+        for (int k = threadIdx.x; k < OUT_NS * (NET_C + 9); k += OUT_THREADS) {
+            const int j = k % OUT_NS, ch = k / OUT_NS;
+            const int idx = n0 + j;
+            const int p = idx >= g.Vh, s = idx - p * g.Vh;
             float v[24];
-            if (idx < N) {
-                const int p = idx >= g.Vh, s = idx - p * g.Vh;
-                if (ch < COUT) {
-                    load_spinor<P_F32, float>(gy + ch * chan + p * par, nullptr, g.Vh, s, v);
-                } else {
-                    int c[4];
-                    cb_coords(g, s, p, c);
-                    PathSite P;
-                    path_setup(g, gauge, p, s, c, path, P);
-                    path_apply(g, x + (ch - COUT) * chan, path, P, v);
-                }
+            float2* dst;
+            int stride;
+            if (ch < NET_C) {
+                load_spinor<P_F32, float>(a + ((size_t)fb * NET_C + ch) * chan + p * par, nullptr, g.Vh, s, v);
+                dst = sa + j * OUT_AS + 4 * ch;
+                stride = 64;
             } else {
-#pragma unroll
-                for (int q = 0; q < 24; ++q) v[q] = 0.f;
+                int c[4];
+                cb_coords(g, s, p, c);
+                transport(g, gauge, b + fb * chan, p, s, c, ch - NET_C, v);
+                dst = st + j * OUT_TS + 4 * (ch - NET_C);
+                stride = 36;
             }
-            float* dst = ch < COUT ? sg[ch][j] : st[ch - COUT][j];
 #pragma unroll
-            for (int q = 0; q < 24; ++q) dst[q] = v[q];
+            for (int sp = 0; sp < 4; ++sp)
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    dst[q * stride + sp] = make_float2(v[2 * (3 * sp + q)], v[2 * (3 * sp + q) + 1]);
         }
         __syncthreads();
-        if (active) {
-            float accr = 0.f, acci = 0.f;
-            for (int j = 0; j < NS; ++j)
+        float cr[4][3], ci[4][3];
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    float gr = sg[co][j][2 * (3 * sa + a)], gi = sg[co][j][2 * (3 * sa + a) + 1];
-                    float tr = st[ci][j][2 * (3 * sb + a)], ti = st[ci][j][2 * (3 * sb + a) + 1];
-                    accr += gr * tr + gi * ti;  // gy * conj(t)
-                    acci += gi * tr - gr * ti;
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int y = 0; y < 3; ++y) cr[x][y] = ci[x][y] = 0.f;
+        for (int j = 0; j < OUT_NS; ++j) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const float4* pa = reinterpret_cast<const float4*>(sa + j * OUT_AS + q * 64 + 4 * i);
+                const float4 a0 = pa[0], a1 = pa[1];
+                const float2* pt = st + j * OUT_TS + q * 36 + 3 * jj;
+                const float ar[4] = {a0.x, a0.z, a1.x, a1.z}, ai[4] = {a0.y, a0.w, a1.y, a1.w};
+#pragma unroll
+                for (int y = 0; y < 3; ++y) {
+                    const float2 t = pt[y];
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) {
+                        cr[x][y] = fmaf(ar[x], t.x, cr[x][y]);
+                        ci[x][y] = fmaf(ai[x], t.x, ci[x][y]);
+                        cr[x][y] = fmaf(ai[x], t.y, cr[x][y]);
+                        ci[x][y] = fmaf(-ar[x], t.y, ci[x][y]);
+                    }
                 }
-            dr += accr;
-            di += acci;
+            }
         }
+        // (hi, lo) += the chunk's sum, the low word collecting the exact rounding error of each addition
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int y = 0; y < 3; ++y) {
+                float t = hr[x][y] + cr[x][y], v = t - hr[x][y];
+                lr[x][y] += (hr[x][y] - (t - v)) + (cr[x][y] - v);
+                hr[x][y] = t;
+                t = hi[x][y] + ci[x][y];
+                v = t - hi[x][y];
+                li[x][y] += (hi[x][y] - (t - v)) + (ci[x][y] - v);
+                hi[x][y] = t;
+            }
     }
-    if (active)
-        partials[((size_t)path * gridDim.x + blockIdx.x) * (COUT * CIN * 16) + e] = make_float2((float)dr, (float)di);
+    float2* out = partials + (size_t)blockIdx.x * NET_X;
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int y = 0; y < 3; ++y)
+            out[(4 * i + x) * 36 + 3 * jj + y] = make_float2(hr[x][y] + lr[x][y], hi[x][y] + li[x][y]);
 }
 
-// gW[path][ent] (+)= sum_b partials[path][b][ent], fixed order
-__global__ void net_wgrad_reduce(const float2* partials, int nblk, int nent, float2* gW, int accumulate)
+// gW (+)= the sum of X over the blocks, in FP64 and a fixed order: 32 entries per block, eight threads
+// per entry (each an eighth of the blocks).  bar: layer 2 (conjugate, spins exchanged, path reversed)
+__global__ void __launch_bounds__(256) net_wgrad_reduce(const float2* partials, int nblk, float2* gW, int bar)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= 9 * nent) return;
-    const int path = k / nent, ent = k % nent;
-    double r = 0, i = 0;
-    for (int b = 0; b < nblk; ++b) {
-        float2 v = partials[((size_t)path * nblk + b) * nent + ent];
+    __shared__ double2 sh[8][32];
+    const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
+    const int k = blockIdx.x * 32 + lane;
+    double r = 0, im = 0;
+    const int b1 = (int)((long)nblk * (part + 1) / 8);
+    for (int b = (int)((long)nblk * part / 8); b < b1; ++b) {
+        const float2 v = partials[(size_t)b * NET_X + k];
         r += v.x;
-        i += v.y;
+        im += v.y;
     }
-    float2 o = make_float2((float)r, (float)i);
-    if (accumulate) {
-        o.x += gW[k].x;
-        o.y += gW[k].y;
+    sh[part][lane] = make_double2(r, im);
+    __syncthreads();
+    if (part) return;
+#pragma unroll
+    for (int q = 1; q < 8; ++q) {
+        r += sh[q][lane].x;
+        im += sh[q][lane].y;
     }
-    gW[k] = o;
+    const int row = k / 36, col = k - row * 36;
+    const int ch = row >> 2, s = row & 3, path = col >> 2, s2 = col & 3;
+    int o;
+    if (bar) {
+        const int pb = path == 0 ? 0 : (((path - 1) & 1) ? path - 1 : path + 1);
+        o = (pb * NET_C + ch) * 16 + 4 * s2 + s;
+        im = -im;
+    } else {
+        o = (path * NET_C + ch) * 16 + 4 * s + s2;
+    }
+    gW[o].x += (float)r;
+    gW[o].y += (float)im;
+}
+
+// coefficients of gy_k = 2 (y_k - e_k) / |e_k|^2 (|e_k|^2 = 1 where e_k vanishes)
+__global__ void net_loss_coef(const double2* en, int n, double2* co)
+{
+    const int k = threadIdx.x + blockIdx.x * blockDim.x;
+    if (k >= n) return;
+    const double v = 2.0 / (en[k].x > 0 ? en[k].x : 1.0);
+    co[k] = make_double2(v, 0);
+    co[n + k] = make_double2(-v, 0);
 }
 
 // W'[q][c'][c] = W[qbar][c][c']^dag for a layer W[9][cout][cin][16]
@@ -270,14 +404,16 @@ __global__ void adam_kernel(float2* W, const float2* G, float* m, float* v, int 
     w[k] -= lr * (m[k] / c1) / (sqrtf(v[k] / c2) + eps);
 }
 
-FieldDesc one(const FieldDesc& f, int i)
+FieldDesc some(const FieldDesc& f, int i, int n)
 {
     FieldDesc s = f;
-    s.nrhs = 1;
+    s.nrhs = n;
     s.data = f.data + (size_t)i * f.rhs_bytes();
     s.norm = f.norm ? f.norm + (size_t)i * 2 * f.Vh : nullptr;
     return s;
 }
+
+FieldDesc one(const FieldDesc& f, int i) { return some(f, i, 1); }
 
 int net_init(ov_ctx* c)
 {
@@ -298,20 +434,50 @@ int net_init(ov_ctx* c)
     return OV_OK;
 }
 
-int layer_fwd(ov_ctx* c, int layer, bool adj, const FieldDesc& x, const FieldDesc& y, cudaStream_t st)
+// work fields of a batch of nb: h, gh (16 channels each), z (9 paths), y, gy; grown when a larger batch
+// is asked for (at most net_batch fields, so that they stay below about 2 GB)
+int net_batch(const ov_ctx* c, int want)
+{
+    const double per = (2.0 * NET_C + 9 + 2) * 192.0 * c->g.Vh;
+    const int cap = (int)std::min(16.0, std::max(1.0, 2e9 / per));
+    return std::min(want, cap);
+}
+
+struct NetWork {
+    FieldDesc h, gh, z, y, gy;
+};
+
+int net_work(ov_ctx* c, int nb, NetWork* w)
+{
+    NetState* n = c->net;
+    if (n->batch < nb) {
+        cudaDeviceSynchronize();  // queued kernels may still use the smaller fields
+        for (int slot : {WS_NET_H, WS_NET_GH, WS_NET_Z, WS_NET_Y, WS_NET_G}) ws_release(c, slot);
+        n->batch = nb;
+    }
+    nb = n->batch;
+    OV_TRY(ws_field(c, WS_NET_H, P_F32, NET_C * nb, &w->h));
+    OV_TRY(ws_field(c, WS_NET_GH, P_F32, NET_C * nb, &w->gh));
+    OV_TRY(ws_field(c, WS_NET_Z, P_F32, 9 * nb, &w->z));
+    OV_TRY(ws_field(c, WS_NET_Y, P_F32, nb, &w->y));
+    return ws_field(c, WS_NET_G, P_F32, nb, &w->gy);
+}
+
+// layer (or its adjoint) on nb fields; z: work field of the 16 -> 1 form
+int layer_fwd(ov_ctx* c, int layer, bool adj, const FieldDesc& x, const FieldDesc& y, const FieldDesc& z, int nb,
+              cudaStream_t st)
 {
     NetState* n = c->net;
     const float2* W = (adj ? n->Wadj : n->W) + (size_t)layer * NET_W;
     const Geom& g = c->g;
     const char* gauge = (const char*)c->gauge[P_F32];
+    const unsigned sites = (unsigned)((2 * g.Vh + 127) / 128);
     // layer 0: 1 -> 16 (adjoint 16 -> 1); layer 1: 16 -> 1 (adjoint 1 -> 16)
-    const bool one_to_many = (layer == 0) != adj;
-    if (one_to_many) {
-        dim3 grid((2 * g.Vh + 127) / 128, NET_C / 4);
-        net_fwd_kernel<1, NET_C, 4><<<grid, 128, 0, st>>>(g, gauge, x.data, y.data, W);
+    if ((layer == 0) != adj) {
+        net_many_kernel<<<dim3(sites, NET_C / NET_CG, nb), 128, 0, st>>>(g, gauge, x.data, y.data, W);
     } else {
-        dim3 grid((2 * g.Vh + 127) / 128, 1);
-        net_fwd_kernel<NET_C, 1, 1><<<grid, 128, 0, st>>>(g, gauge, x.data, y.data, W);
+        net_mix_kernel<<<dim3(sites, 3, nb), 128, 0, st>>>(g, x.data, z.data, W);
+        net_gather_kernel<<<dim3(sites, 1, nb), 128, 0, st>>>(g, gauge, z.data, y.data);
     }
     OV_CUDA(c, cudaGetLastError());
     return OV_OK;
@@ -331,17 +497,18 @@ int loss_grad(ov_ctx* c, const FieldDesc& pr, const FieldDesc& pe, int k0, int k
 {
     NetState* n = c->net;
     const Geom& g = c->g;
-    FieldDesc h, y, gy, gh;
-    OV_TRY(ws_field(c, WS_NET_H, P_F32, NET_C, &h));
-    OV_TRY(ws_field(c, WS_NET_GH, P_F32, NET_C, &gh));
-    OV_TRY(ws_field(c, WS_NET_G, P_F32, 1, &y));
-    OV_TRY(ws_field(c, WS_LZ_T, P_F32, 1, &gy));
-    const int nblk = 2 * 152;
-    const size_t need = (size_t)9 * nblk * 256;
+    const int np = k1 - k0;
+    const int B = net_batch(c, np);
+    NetWork w;
+    OV_TRY(net_work(c, B, &w));
+    const int nblk_max = 4 * 152;
+    const size_t need = (size_t)nblk_max * NET_X;
     if (n->partials_n < need) {
         if (n->partials) {
             cudaDeviceSynchronize();
             dev_free(c, n->partials, sizeof(float2) * n->partials_n);
+            n->partials = nullptr;
+            n->partials_n = 0;
         }
         void* p = nullptr;
         OV_TRY(dev_alloc(c, &p, sizeof(float2) * need));
@@ -350,40 +517,35 @@ int loss_grad(ov_ctx* c, const FieldDesc& pr, const FieldDesc& pe, int k0, int k
     }
     OV_CUDA(c, cudaMemsetAsync(n->G, 0, sizeof(float2) * NET_PARAMS, st));
     OV_TRY(refresh_adjoint(c, st));
-    const int np = k1 - k0;
-    std::vector<double> en(np);
-    double* dn = c->dscal + DSCAL_DOT;  // double2 per pair
-    for (int k = k0; k < k1; ++k) OV_TRY(norm2(c, one(pe, k), dn + 2 * (k - k0), st));
-    {
-        std::vector<double2> h2(np);
-        OV_CUDA(c, cudaMemcpyAsync(h2.data(), dn, sizeof(double2) * np, cudaMemcpyDeviceToHost, st));
-        OV_CUDA(c, cudaStreamSynchronize(st));
-        for (int k = 0; k < np; ++k) en[k] = h2[k].x > 0 ? h2[k].x : 1.0;
-    }
+    std::vector<double2> en(np);
+    std::vector<double> gn(np);
+    double2* dn = (double2*)(c->dscal + DSCAL_DOT);
+    double2* dco = (double2*)(c->dscal + DSCAL_CGCO);
     double* dg = c->dscal + DSCAL_NORM;
-    for (int k = k0; k < k1; ++k) {
-        FieldDesc r = one(pr, k), e = one(pe, k);
-        OV_TRY(layer_fwd(c, 0, false, r, h, st));
-        OV_TRY(layer_fwd(c, 1, false, h, y, st));
+    const char* gauge = (const char*)c->gauge[P_F32];
+    OV_TRY(norm2(c, some(pe, k0, np), (double*)dn, st));
+    for (int k = k0; k < k1; k += B) {
+        const int nb = std::min(B, k1 - k);
+        FieldDesc r = some(pr, k, nb), e = some(pe, k, nb), y = some(w.y, 0, nb), gy = some(w.gy, 0, nb);
+        OV_TRY(layer_fwd(c, 0, false, r, w.h, w.z, nb, st));
+        OV_TRY(layer_fwd(c, 1, false, w.h, y, w.z, nb, st));
         // gy = 2 (y - e) / |e|^2, with |gy|^2 recorded for the loss
+        net_loss_coef<<<1, 32, 0, st>>>(dn + (k - k0), nb, dco);
         FieldDesc xs[2] = {y, e};
-        const double s2 = 2.0 / en[k - k0];
-        double2 hc[2] = {make_double2(s2, 0), make_double2(-s2, 0)};
-        OV_TRY(lincomb(c, gy, 2, xs, hc, nullptr, 0, dg + (k - k0), st));
-        net_wgrad_kernel<NET_C, 1><<<dim3(nblk, 9), 256, 0, st>>>(g, (const char*)c->gauge[P_F32], h.data, gy.data,
-                                                                  n->partials);
-        net_wgrad_reduce<<<(9 * 256 + 255) / 256, 256, 0, st>>>(n->partials, nblk, 256, n->G + NET_W, 1);
-        OV_TRY(layer_fwd(c, 1, true, gy, gh, st));  // gh = L2^dag gy
-        net_wgrad_kernel<1, NET_C><<<dim3(nblk, 9), 256, 0, st>>>(g, (const char*)c->gauge[P_F32], r.data, gh.data,
-                                                                  n->partials);
-        net_wgrad_reduce<<<(9 * 256 + 255) / 256, 256, 0, st>>>(n->partials, nblk, 256, n->G, 1);
+        OV_TRY(lincomb(c, gy, 2, xs, nullptr, dco, 0, dg + (k - k0), st));
+        const int nblk = (int)std::min<long>(nblk_max, (2L * g.Vh * nb) / OUT_NS);
+        net_outer_kernel<<<nblk, OUT_THREADS, 0, st>>>(g, gauge, w.h.data, gy.data, nb, n->partials);
+        net_wgrad_reduce<<<NET_X / 32, 256, 0, st>>>(n->partials, nblk, n->G + NET_W, 1);
+        OV_TRY(layer_fwd(c, 1, true, gy, w.gh, w.z, nb, st));  // gh = L2^dag gy
+        net_outer_kernel<<<nblk, OUT_THREADS, 0, st>>>(g, gauge, w.gh.data, r.data, nb, n->partials);
+        net_wgrad_reduce<<<NET_X / 32, 256, 0, st>>>(n->partials, nblk, n->G, 0);
         OV_CUDA(c, cudaGetLastError());
     }
-    std::vector<double> gn(np);
+    OV_CUDA(c, cudaMemcpyAsync(en.data(), dn, sizeof(double2) * np, cudaMemcpyDeviceToHost, st));
     OV_CUDA(c, cudaMemcpyAsync(gn.data(), dg, sizeof(double) * np, cudaMemcpyDeviceToHost, st));
     OV_CUDA(c, cudaStreamSynchronize(st));
     double total = 0;
-    for (int k = 0; k < np; ++k) total += gn[k] * en[k] / 4.0;  // |y-e|^2/|e|^2 = |gy|^2 |e|^2 / 4
+    for (int k = 0; k < np; ++k) total += gn[k] * (en[k].x > 0 ? en[k].x : 1.0) / 4.0;  // |y-e|^2/|e|^2 = |gy|^2 |e|^2 / 4
     *loss = total;
     return OV_OK;
 }
@@ -418,27 +580,31 @@ int net_apply_precond(ov_ctx* c, const FieldDesc& r, const FieldDesc& z, cudaStr
         OV_TRY(refresh_adjoint(c, st));
         n->adj_valid = 1;
     }
-    FieldDesc h, a, b, d;
-    OV_TRY(ws_field(c, WS_NET_H, P_F32, NET_C, &h));
-    OV_TRY(ws_field(c, WS_NET_G, P_F32, 1, &a));
-    OV_TRY(ws_field(c, WS_NET_GH, P_F32, 1, &b));
-    if (sym) OV_TRY(ws_field(c, WS_NET_S, P_F32, 1, &d));
-    for (int q = 0; q < r.nrhs; ++q) {
-        FieldDesc rq = one(r, q), zq = one(z, q);
-        const bool f32in = r.prec == P_F32, f32out = z.prec == P_F32;
-        if (!f32in) OV_TRY(convert(c, rq, a, st));
-        const FieldDesc& x = f32in ? rq : a;
-        OV_TRY(layer_fwd(c, 0, false, x, h, st));
-        OV_TRY(layer_fwd(c, 1, false, h, (f32out && !sym) ? zq : b, st));
+    const int R = r.nrhs, B = net_batch(c, R);
+    NetWork w;
+    OV_TRY(net_work(c, B, &w));
+    FieldDesc a, b, d;
+    const bool f32in = r.prec == P_F32, f32out = z.prec == P_F32;
+    if (!f32in) OV_TRY(ws_field(c, WS_NET_A, P_F32, B, &a));
+    if (!f32out) OV_TRY(ws_field(c, WS_NET_B, P_F32, B, &b));
+    if (sym) OV_TRY(ws_field(c, WS_NET_S, P_F32, B, &d));
+    for (int q = 0; q < R; q += B) {
+        const int nb = std::min(B, R - q);
+        FieldDesc rq = some(r, q, nb), zq = some(z, q, nb);
+        if (!f32in) OV_TRY(convert(c, rq, some(a, 0, nb), st));
+        const FieldDesc x = f32in ? rq : some(a, 0, nb), out = f32out ? zq : some(b, 0, nb);
+        const FieldDesc y = sym ? some(w.y, 0, nb) : out;
+        OV_TRY(layer_fwd(c, 0, false, x, w.h, w.z, nb, st));
+        OV_TRY(layer_fwd(c, 1, false, w.h, y, w.z, nb, st));
         if (sym) {
             // z = (M + M^dag) r / 2, M^dag = L1^dag L2^dag: Hermitian, as CG expects of a preconditioner
-            OV_TRY(layer_fwd(c, 1, true, x, h, st));
-            OV_TRY(layer_fwd(c, 0, true, h, d, st));
-            FieldDesc v[2] = {b, d};
+            OV_TRY(layer_fwd(c, 1, true, x, w.h, w.z, nb, st));
+            OV_TRY(layer_fwd(c, 0, true, w.h, some(d, 0, nb), w.z, nb, st));
+            FieldDesc v[2] = {y, some(d, 0, nb)};
             double2 hc[2] = {make_double2(0.5, 0), make_double2(0.5, 0)};
-            OV_TRY(lincomb(c, f32out ? zq : b, 2, v, hc, nullptr, 0, nullptr, st));
+            OV_TRY(lincomb(c, out, 2, v, hc, nullptr, 0, nullptr, st));
         }
-        if (!f32out) OV_TRY(convert(c, b, zq, st));
+        if (!f32out) OV_TRY(convert(c, out, zq, st));
     }
     return OV_OK;
 }
@@ -556,7 +722,7 @@ int ov_net_train(ov_ctx* c, int nsolves, int steps, double lr, double mass, doub
     n->npairs = 0;
     FieldDesc b, xs32;
     OV_TRY(ws_field(c, WS_AUX1, P_F64, 1, &b));
-    OV_TRY(ws_field(c, WS_NET_G, P_F32, 1, &xs32));
+    OV_TRY(ws_field(c, WS_AUX1, P_F32, 1, &xs32));
     const int was_trained = n->trained;
     n->trained = 0;
     for (int s = 0; s < nsolves && n->npairs < n->cap; ++s) {
