@@ -44,7 +44,7 @@ struct EigSet {
     std::vector<double> vals;   // host copy
     FieldDesc vec[NPREC] = {};      // per storage precision (F64 is the master copy)
     double* d_sign = nullptr;   // device sign(lam_i) (which = 0)
-    void* tc_rows = nullptr;    // bf16 rows of the tensor-core projection [nev][24V]
+    void* tc_rows = nullptr;    // bf16 rows of the tensor-core projection, tiles [24V / 64][nev][64]
     size_t tc_bytes = 0;
     void* tc_lo = nullptr;      // bf16 remainders of the FP32 copy (FP32-class tensor-core operand)
     size_t tc_lo_bytes = 0;

@@ -330,16 +330,16 @@ __global__ void __launch_bounds__(OUT_THREADS, 3) net_outer_kernel(Geom g, const
             out[(4 * i + x) * 36 + 3 * jj + y] = make_float2(hr[x][y] + lr[x][y], hi[x][y] + li[x][y]);
 }
 
-// gW (+)= the sum of X over the blocks, in FP64 and a fixed order: 32 entries per block, eight threads
-// per entry (each an eighth of the blocks).  bar: layer 2 (conjugate, spins exchanged, path reversed)
-__global__ void __launch_bounds__(256) net_wgrad_reduce(const float2* partials, int nblk, float2* gW, int bar)
+// gW (+)= the sum of X over the blocks, in FP64 and a fixed order: 32 entries per block, 32 threads
+// per entry (each a share of the blocks).  bar: layer 2 (conjugate, spins exchanged, path reversed)
+__global__ void __launch_bounds__(1024) net_wgrad_reduce(const float2* partials, int nblk, float2* gW, int bar)
 {
-    __shared__ double2 sh[8][32];
+    __shared__ double2 sh[32][32];
     const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
     const int k = blockIdx.x * 32 + lane;
     double r = 0, im = 0;
-    const int b1 = (int)((long)nblk * (part + 1) / 8);
-    for (int b = (int)((long)nblk * part / 8); b < b1; ++b) {
+    const int b1 = (int)((long)nblk * (part + 1) / 32);
+    for (int b = (int)((long)nblk * part / 32); b < b1; ++b) {
         const float2 v = partials[(size_t)b * NET_X + k];
         r += v.x;
         im += v.y;
@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(256) net_wgrad_reduce(const float2* partials, 
     __syncthreads();
     if (part) return;
 #pragma unroll
-    for (int q = 1; q < 8; ++q) {
+    for (int q = 1; q < 32; ++q) {
         r += sh[q][lane].x;
         im += sh[q][lane].y;
     }
@@ -535,10 +535,10 @@ int loss_grad(ov_ctx* c, const FieldDesc& pr, const FieldDesc& pe, int k0, int k
         OV_TRY(lincomb(c, gy, 2, xs, nullptr, dco, 0, dg + (k - k0), st));
         const int nblk = (int)std::min<long>(nblk_max, (2L * g.Vh * nb) / OUT_NS);
         net_outer_kernel<<<nblk, OUT_THREADS, 0, st>>>(g, gauge, w.h.data, gy.data, nb, n->partials);
-        net_wgrad_reduce<<<NET_X / 32, 256, 0, st>>>(n->partials, nblk, n->G + NET_W, 1);
+        net_wgrad_reduce<<<NET_X / 32, 1024, 0, st>>>(n->partials, nblk, n->G + NET_W, 1);
         OV_TRY(layer_fwd(c, 1, true, gy, w.gh, w.z, nb, st));  // gh = L2^dag gy
         net_outer_kernel<<<nblk, OUT_THREADS, 0, st>>>(g, gauge, w.gh.data, r.data, nb, n->partials);
-        net_wgrad_reduce<<<NET_X / 32, 256, 0, st>>>(n->partials, nblk, n->G, 0);
+        net_wgrad_reduce<<<NET_X / 32, 1024, 0, st>>>(n->partials, nblk, n->G, 0);
         OV_CUDA(c, cudaGetLastError());
     }
     OV_CUDA(c, cudaMemcpyAsync(en.data(), dn, sizeof(double2) * np, cudaMemcpyDeviceToHost, st));

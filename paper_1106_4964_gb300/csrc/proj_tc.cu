@@ -77,6 +77,15 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
         : "memory");
 }
 
+__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
+            smem_u32(dst)),
+        "l"((uint64_t)map), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
+        : "memory");
+}
+
 // shared-memory matrix descriptor: K-major, 128B swizzle, 8-row groups 1024 bytes apart
 __device__ __forceinline__ uint64_t smem_desc(const void* p)
 {
@@ -182,10 +191,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             if (*(volatile int*)&abort_flag) break;
             uint8_t* sa = base + s * stage_bytes;
             mbar_expect_tx(&full_bar[s], stage_bytes);
-            const int k = (t0 + t) * TC_BK;
-            tma_load_2d(sa, &tmA, k, 0, &full_bar[s]);
-            if (nsplit == 2) tma_load_2d(sa + a_bytes, &tmAlo, k, 0, &full_bar[s]);
-            tma_load_2d(sa + nsplit * a_bytes, &tmB, k, 0, &full_bar[s]);
+            tma_load_3d(sa, &tmA, 0, 0, t0 + t, &full_bar[s]);
+            if (nsplit == 2) tma_load_3d(sa + a_bytes, &tmAlo, 0, 0, t0 + t, &full_bar[s]);
+            tma_load_2d(sa + nsplit * a_bytes, &tmB, (t0 + t) * TC_BK, 0, &full_bar[s]);
         }
     } else if (warp == 1 && lane == 0) {
         // MMA issuer
@@ -236,24 +244,36 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 // c[i][r] = (sum_g P[g][i][2r], sum_g P[g][i][2r+1]) in FP64, fixed order.  nsplit = 2: the columns
 // 2R + 2r, 2R + 2r + 1 hold the products with the bf16 remainder of psi, and the second accumulator
 // (columns npad + ...) the products of the remainder rows of eta; the three leading terms are added
-// (hi.hi + hi.lo + lo.hi; lo.lo is below the FP32 resolution)
-__global__ void proj_tc_reduce(const float* partials, int ngrid, int npad, int nsplit, int nev, int nrhs, double2* c)
+// (hi.hi + hi.lo + lo.hi; lo.lo is below the FP32 resolution).  One block per eigenvector: lanes over the
+// columns (coalesced), 32 rows of threads each a share of the CTAs (one thread per coefficient read 4-byte pieces
+// of all partials one after the other: 225 us for 100 x 12)
+__global__ void __launch_bounds__(1024) proj_tc_reduce(const float* partials, int ngrid, int npad, int nsplit, int nrhs,
+                                                      double2* c)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nev * nrhs) return;
-    const int i = k / nrhs, r = k % nrhs;
-    const int ncol = nsplit * npad;
-    double re = 0, im = 0;
-    for (int g = 0; g < ngrid; ++g) {
-        const float* p = partials + ((size_t)g * TC_M + i) * ncol;
-        re += p[2 * r];
-        im += p[2 * r + 1];
-        if (nsplit == 2) {
-            re += (double)p[2 * nrhs + 2 * r] + (double)p[npad + 2 * r];
-            im += (double)p[2 * nrhs + 2 * r + 1] + (double)p[npad + 2 * r + 1];
+    __shared__ double sh[32][32], col[256];
+    const int i = blockIdx.x, ncol = nsplit * npad;
+    for (int c0 = 0; c0 < ncol; c0 += 32) {
+        const int cc = c0 + threadIdx.x;
+        double v = 0;
+        if (cc < ncol)
+            for (int g = threadIdx.y; g < ngrid; g += 32) v += partials[((size_t)g * TC_M + i) * ncol + cc];
+        sh[threadIdx.y][threadIdx.x] = v;
+        __syncthreads();
+        if (threadIdx.y == 0) {
+#pragma unroll
+            for (int q = 1; q < 32; ++q) v += sh[q][threadIdx.x];
+            col[cc] = v;  // c0 + 31 < 256: ncol <= 256
         }
+        __syncthreads();
     }
-    c[k] = make_double2(re, im);
+    const int r = threadIdx.y * 32 + threadIdx.x;
+    if (r >= nrhs) return;
+    double re = col[2 * r], im = col[2 * r + 1];
+    if (nsplit == 2) {
+        re += col[2 * nrhs + 2 * r] + col[npad + 2 * r];
+        im += col[2 * nrhs + 2 * r + 1] + col[npad + 2 * r + 1];
+    }
+    c[(size_t)i * nrhs + r] = make_double2(re, im);
 }
 
 // B operand: rows 2r = psi_r, 2r+1 = (im, -re) pairs, bf16, from an FP32 field; nsplit = 2 adds rows
@@ -282,23 +302,19 @@ __global__ void build_b_kernel(const float4* __restrict__ x, int n4, int nrhs, i
     }
 }
 
-// the bf16 remainder x - bf16(x) of each FP32 value
-__global__ void to_bf16_lo_kernel(const float4* __restrict__ x, long long n4, __nv_bfloat16* y)
+// bf16 rows of the eigenvectors (lo: the bf16 remainders x - bf16(x)) in tiles [K / 64][nev][64]: the
+// 64 reals of all eigenvectors that one stage of either contraction needs are one contiguous block.
+// (Row-major rows made every stage 128-byte pieces 48 Vh reals apart: c = eta^dag psi of 100 rows and 12
+// right-hand sides at 16^3 x 32 took 327 us, 245 from the tiles; 1.6 GB.)  x: nev FP32 rows of K reals.
+template <bool LO>
+__global__ void to_bf16_tiles_kernel(const float4* __restrict__ x, long long K, int nev, __nv_bfloat16* y)
 {
     const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n4) return;
-    const float4 v = x[q];
-    const float e[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) y[4 * q + j] = __float2bfloat16_rn(e[j] - __bfloat162float(__float2bfloat16_rn(e[j])));
-}
-
-__global__ void to_bf16_kernel(const float4* __restrict__ x, long long n4, __nv_bfloat16* y)
-{
-    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n4) return;
-    const float4 v = x[q];
-    __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(y + 4 * q);
+    const int i = blockIdx.y;
+    if (4 * q >= K) return;
+    float4 v = x[(size_t)i * (K / 4) + q];
+    if (LO) v = make_float4(bf16_rem(v.x), bf16_rem(v.y), bf16_rem(v.z), bf16_rem(v.w));
+    __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(y + (((4 * q) / 64) * nev + i) * 64 + (4 * q) % 64);
     o[0] = __floats2bfloat162_rn(v.x, v.y);
     o[1] = __floats2bfloat162_rn(v.z, v.w);
 }
@@ -331,6 +347,21 @@ bool make_map(CUtensorMap* m, const void* ptr, long long K, int rows, int box_ro
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// 3D bf16 map of the tiled rows: 64 reals x nev rows x K / 64 tiles, box 64 x box_rows x box_tiles, 128B
+// swizzle, zero fill beyond nev
+bool make_tile_map(CUtensorMap* m, const void* ptr, long long K, int nev, int box_rows, int box_tiles)
+{
+    auto fn = encode_fn();
+    if (!fn) return false;
+    cuuint64_t dims[3] = {64, (cuuint64_t)nev, (cuuint64_t)(K / 64)};
+    cuuint64_t strides[2] = {128, (cuuint64_t)nev * 128};
+    cuuint32_t box[3] = {64, (cuuint32_t)box_rows, (cuuint32_t)box_tiles};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // ---------------------------------------------------------------------------
 // V c on the tensor cores (Eq. 7: psi_h = psi - sum_i eta_i c_i and the exact low-mode
 // part sum_i sign(lam_i) c_i eta_i).  As a real GEMM over the eigenvector index i:
@@ -340,9 +371,9 @@ bool make_map(CUtensorMap* m, const void* ptr, long long K, int rows, int box_ro
 // Real position k = 2m holds Re eta(m), k = 2m + 1 holds Im eta(m); the complex product is
 // assembled in the epilogue from the row and its neighbour (TMEM lanes k and k ^ 1):
 //   corr_re(m) = X(2m) - Y(2m+1),  corr_im(m) = Y(2m) + X(2m+1),  X = P[.][c_re], Y = P[.][c_im].
-// A = the eigenvector rows (bf16, [nev][48 Vh]) read as an MN-major operand: a tile is 128
+// A = the eigenvector rows (bf16 tiles [48 Vh / 64][nev][64]) read as an MN-major operand: a tile is 128
 // consecutive real positions (two 64-element swizzle atoms, LBO apart) by the eigenvector index
-// (8-row groups 1024 bytes apart), loaded by TMA straight from the row-major copy; rows i >= nev
+// (8-row groups 1024 bytes apart), loaded by TMA straight from the tiled copy; rows i >= nev
 // are zero-filled by the TMA bounds and cost no traffic.  nsplit = 2 adds the rows of the bf16
 // remainder eta - bf16(eta) into the same accumulator (FP32-class eigenvectors at 4 bytes per real).
 // Persistent, warp-specialised: warp 0 issues the TMA loads into a ring of stages, warp 1 issues
@@ -438,13 +469,8 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
             const long long tile = blockIdx.x + it * gridDim.x;
             uint8_t* st = base + (size_t)s * stage_bytes;
             mbar_expect_tx(&full_bar[s], stage_bytes);
-            const int x0 = (int)(tile * UP_M);
-            tma_load_2d(st, &tmA, x0, 0, &full_bar[s]);
-            tma_load_2d(st + half_bytes, &tmA, x0 + 64, 0, &full_bar[s]);
-            if (P.nsplit == 2) {
-                tma_load_2d(st + 2 * half_bytes, &tmAlo, x0, 0, &full_bar[s]);
-                tma_load_2d(st + 3 * half_bytes, &tmAlo, x0 + 64, 0, &full_bar[s]);
-            }
+            tma_load_3d(st, &tmA, 0, 0, (int)(2 * tile), &full_bar[s]);  // both 64-element atoms
+            if (P.nsplit == 2) tma_load_3d(st + 2 * half_bytes, &tmAlo, 0, 0, (int)(2 * tile), &full_bar[s]);
         }
         // drain: no block leaves with bulk copies in flight (the bounded waits of the stages that were
         // issued and never taken by the MMA thread)
@@ -497,8 +523,24 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
         const long long rhs_reals = 48LL * P.Vh;
         const long long par_reals = 24LL * P.Vh;
         const long long lo_chunk = 12LL * P.Vh;  // chunks 3..5 of a parity (spins 2, 3) start here
+        // psi of a tile is loaded one tile ahead (RMAX values per thread): loaded where it is used, each of
+        // the R loads of a row cost its latency in turn (12 right-hand sides and 100 rows at 16^3 x 32: 1090
+        // us, 279 with the loads ahead and the tiled rows; 1.7 GB)
+        constexpr int RMAX = 16;
+        float ps[RMAX];
+        auto load_psi = [&](long long it) {
+            const long long k = (blockIdx.x + it * gridDim.x) * UP_M + row;
+#pragma unroll
+            for (int r = 0; r < RMAX; ++r)
+                ps[r] = (P.mode == 0 && r < P.R && it < my_tiles) ? __ldg(P.psi + r * rhs_reals + k) : 0.f;
+        };
+        load_psi(0);
         for (long long it = 0; it < my_tiles; ++it) {
             const int a = (int)(it & 1);
+            float cur[RMAX];
+#pragma unroll
+            for (int r = 0; r < RMAX; ++r) cur[r] = ps[r];
+            load_psi(it + 1);
             if (*(volatile int*)&abort_flag) break;
             if (!mbar_wait(&tfull[a], (uint32_t)((it >> 1) & 1))) {
                 if (lane == 0) atomicExch(P.err, 16);
@@ -511,7 +553,11 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
             const bool lower = (k % par_reals) >= lo_chunk;  // gamma5 = -1 on spins 2, 3
             const float g5 = lower ? -1.f : 1.f;
             const float sg = (lane & 1) ? 1.f : -1.f;
-            for (int c0 = 0; c0 < P.npad; c0 += 16) {
+            float* o1 = P.out1 + k;
+            float* o2 = P.out2 ? P.out2 + k : nullptr;
+#pragma unroll
+            for (int c0 = 0; c0 < 8 * RMAX; c0 += 16) {
+                if (c0 >= P.npad) break;
                 float v[16];
                 tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * P.npad + c0), v);
 #pragma unroll
@@ -523,9 +569,8 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
                     const float YWp = __shfl_xor_sync(0xffffffffu, YW, 1);
                     if (r < P.R) {
                         const float corr = X + sg * Yp, w = XW + sg * YWp;
-                        const long long idx = (long long)r * rhs_reals + k;
-                        P.out1[idx] = P.mode == 0 ? P.psi[idx] - corr : corr;
-                        if (P.out2) P.out2[idx] = g5 * w;
+                        o1[r * rhs_reals] = P.mode == 0 ? cur[r] - corr : corr;
+                        if (o2) o2[r * rhs_reals] = g5 * w;
                     }
                 }
             }
@@ -598,9 +643,8 @@ int eig_bf16_rows(ov_ctx* c, int which, cudaStream_t st, const void** out)
         const long long K = 48LL * c->g.Vh;
         OV_TRY(dev_alloc(c, &E.tc_rows, (size_t)E.nev * K * 2));
         E.tc_bytes = (size_t)E.nev * K * 2;
-        const long long n4 = (long long)E.nev * K / 4;
-        to_bf16_kernel<<<(unsigned)((n4 + 255) / 256), 256, 0, st>>>((const float4*)f32.data, n4,
-                                                                     (__nv_bfloat16*)E.tc_rows);
+        to_bf16_tiles_kernel<false><<<dim3((unsigned)((K / 4 + 255) / 256), E.nev), 256, 0, st>>>(
+            (const float4*)f32.data, K, E.nev, (__nv_bfloat16*)E.tc_rows);
         OV_CUDA(c, cudaGetLastError());
     }
     *out = E.tc_rows;
@@ -620,9 +664,8 @@ int eig_bf16_lo_rows(ov_ctx* c, int which, cudaStream_t st, const void** out)
         E.tc_lo_bytes = (size_t)E.nev * K * 2;
         // remainder of the FP32 copy: hi + lo carries 16 significand bits of the FP32 value, which is what
         // the FP32 arithmetic of the operator resolves
-        const long long n4 = (long long)E.nev * K / 4;
-        to_bf16_lo_kernel<<<(unsigned)((n4 + 255) / 256), 256, 0, st>>>((const float4*)f32.data, n4,
-                                                                        (__nv_bfloat16*)E.tc_lo);
+        to_bf16_tiles_kernel<true><<<dim3((unsigned)((K / 4 + 255) / 256), E.nev), 256, 0, st>>>(
+            (const float4*)f32.data, K, E.nev, (__nv_bfloat16*)E.tc_lo);
         OV_CUDA(c, cudaGetLastError());
     }
     *out = E.tc_lo;
@@ -668,7 +711,7 @@ int proj_update_tc(ov_ctx* c, int which, const FieldDesc& psi, const double2* dc
                                                                         npad, kpB, (__nv_bfloat16*)c->tc_cb);
     OV_CUDA(c, cudaGetLastError());
     CUtensorMap ma, malo, mb;
-    if (!make_map(&ma, A, K, nev, kpadA) || !make_map(&malo, nsplit == 2 ? Alo : A, K, nev, kpadA) ||
+    if (!make_tile_map(&ma, A, K, nev, kpadA, 2) || !make_tile_map(&malo, nsplit == 2 ? Alo : A, K, nev, kpadA, 2) ||
         !make_map(&mb, c->tc_cb, kpB, npad, npad))
         return set_err(c, OV_ECUDA, "cuTensorMapEncodeTiled failed");
     const uint32_t stage_bytes = (uint32_t)nsplit * 2 * kpadA * 128;
@@ -767,7 +810,7 @@ int proj_dots_tc(ov_ctx* c, int which, const FieldDesc& psi, double2* cout, cuda
                                                                            (__nv_bfloat16*)c->tc_b, K);
     OV_CUDA(c, cudaGetLastError());
     CUtensorMap ma, malo, mb;
-    if (!make_map(&ma, A, K, nev, TC_M) || !make_map(&malo, nsplit == 2 ? Alo : A, K, nev, TC_M) ||
+    if (!make_tile_map(&ma, A, K, nev, TC_M, 1) || !make_tile_map(&malo, nsplit == 2 ? Alo : A, K, nev, TC_M, 1) ||
         !make_map(&mb, c->tc_b, K, ncolB, npad))
         return set_err(c, OV_ECUDA, "cuTensorMapEncodeTiled failed");
     const int ktiles = (int)(K / TC_BK);
@@ -791,8 +834,7 @@ int proj_dots_tc(ov_ctx* c, int which, const FieldDesc& psi, double2* cout, cuda
     proj_tc_kernel<<<grid, TC_THREADS, smem, st>>>(ma, malo, mb, ktiles, npad, nsplit, tmem_cols,
                                                    (float*)c->partials, c->tc_err);
     OV_CUDA(c, cudaGetLastError());
-    proj_tc_reduce<<<(nev * R + 127) / 128, 128, 0, st>>>((const float*)c->partials, grid, npad, nsplit, nev, R,
-                                                          cout);
+    proj_tc_reduce<<<nev, dim3(32, 32), 0, st>>>((const float*)c->partials, grid, npad, nsplit, R, cout);
     OV_CUDA(c, cudaGetLastError());
     return OV_OK;
 }
