@@ -256,6 +256,7 @@ int dslash_apply(ov_ctx* c, const FieldDesc& in, const FieldDesc& out, double a,
     A.da = split2(a);
     A.db = split2(b);
     A.nrhs = in.nrhs;
+    A.pdl = c->pdl;
     A.g5_core = g5_core;
     A.g5_out = g5_out;
     auto it = c->shape.find({in.prec, in.nrhs});
@@ -543,7 +544,9 @@ static int with_graph(ov_ctx* c, int kind, const FieldDesc& in, const FieldDesc&
     }
     const long long before = c->dslash_launches;
     OV_CUDA(c, cudaStreamBeginCapture(gs, cudaStreamCaptureModeThreadLocal));
+    c->pdl = true;
     int s = body(gs);
+    c->pdl = false;
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(gs, &g);
     const long long n = c->dslash_launches - before;

@@ -99,6 +99,7 @@ struct ov_ctx {
     std::map<std::tuple<int, const void*, const void*, int, int, double, int>, std::pair<cudaGraphExec_t, long long>>
         graphs;
     bool use_graphs = true;
+    bool pdl = false;  // set while a graph of this context is captured: dslash launches may overlap their start
     long long graph_captures = 0, graph_replays = 0;  // instrumentation (ov_graph_stats)
     // library-owned stream (and its two ordering events) on which graphs run for callers that pass the
     // legacy default stream, which cannot be captured

@@ -220,6 +220,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, MINB) dslash_split_kernel(const
     using W = Wide<SP>;
     __shared__ int4 sh[8][6][32];
     __shared__ uint32_t she[8][32];
+    pdl_begin();
     const Geom& g = A.g;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const BlockWork bw = block_work((A.nrhs + nby - 1) / nby);
@@ -247,6 +248,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, MINB) dslash_split_kernel(const
         const bool fwd = (w & 1) == 0;
         const int ls = fwd ? s : sn;
         const char* lb = A.gauge + (size_t)((fwd ? p : q) * 4 + (w >> 1)) * g.Vh * 144;
+        pdl_wait();
         for (int r = bw.grp * nby; r < r1; ++r) {
             const char* in_q = A.in + ((size_t)r * 2 + q) * par_bytes;
             {
@@ -324,13 +326,12 @@ cudaError_t launch_ny(const DslashArgs& A, int ny, int ngrp, int by, cudaStream_
 {
     const dim3 grid = block_grid(A.g.Vh, 32 * ngrp, (A.nrhs + by - 1) / by);
     switch (ny) {
-    case 0: dslash_split_kernel<SP, 0, MINB><<<grid, SPLIT_THREADS, 0, st>>>(A, ngrp, by); break;
-    case 1: dslash_split_kernel<SP, 1, MINB><<<grid, SPLIT_THREADS, 0, st>>>(A, ngrp, by); break;
-    case 2: dslash_split_kernel<SP, 2, MINB><<<grid, SPLIT_THREADS, 0, st>>>(A, ngrp, by); break;
-    case 3: dslash_split_kernel<SP, 3, MINB><<<grid, SPLIT_THREADS, 0, st>>>(A, ngrp, by); break;
-    default: return cudaErrorInvalidValue;
+    case 0: return launch_kernel(dslash_split_kernel<SP, 0, MINB>, grid, dim3(SPLIT_THREADS), st, A.pdl, A, ngrp, by);
+    case 1: return launch_kernel(dslash_split_kernel<SP, 1, MINB>, grid, dim3(SPLIT_THREADS), st, A.pdl, A, ngrp, by);
+    case 2: return launch_kernel(dslash_split_kernel<SP, 2, MINB>, grid, dim3(SPLIT_THREADS), st, A.pdl, A, ngrp, by);
+    case 3: return launch_kernel(dslash_split_kernel<SP, 3, MINB>, grid, dim3(SPLIT_THREADS), st, A.pdl, A, ngrp, by);
     }
-    return cudaGetLastError();
+    return cudaErrorInvalidValue;
 }
 
 template <int SP>

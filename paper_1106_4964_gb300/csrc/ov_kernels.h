@@ -24,6 +24,7 @@ struct DslashArgs {
     float2 da, db, dsy[3];       // and as double-float pairs (hi, lo)
     int nrhs;
     int g5_core, g5_out;
+    int pdl;                     // launch with programmatic stream serialization (launch_kernel)
     unsigned* err;               // set to 1 when a bounded wait of a staged variant times out
     long long wait_polls;        // limit of the bulk-copy variants' first mbarrier wait (polls)
 };
