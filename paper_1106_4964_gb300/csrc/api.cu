@@ -186,9 +186,13 @@ bool verbose()
     return v;
 }
 
-// Flags set by kernels whose bounded waits ran out (derr[2]); read and cleared.
+// Flags set by kernels whose bounded waits ran out (derr[2]); read and cleared.  Only the bulk-copy dslash
+// variants wait: with none launched since the last look the call stays asynchronous (the read and its
+// synchronisation were 25 of the 39 us of an H_w application at 4^4).
 int check_kernel_flags(ov_ctx* c, cudaStream_t st)
 {
+    if (!c->wait_pending) return OV_OK;
+    c->wait_pending = false;
     unsigned f = 0;
     OV_CUDA(c, cudaMemcpyAsync(&f, c->derr + 2, sizeof f, cudaMemcpyDeviceToHost, st));
     OV_CUDA(c, cudaStreamSynchronize(st));
@@ -262,6 +266,10 @@ int dslash_apply(ov_ctx* c, const FieldDesc& in, const FieldDesc& out, double a,
     auto it = c->shape.find({in.prec, in.nrhs});
     std::tuple<int, int, int> sh = it != c->shape.end() ? it->second : default_shape(in.prec, in.nrhs);
     OV_CUDA(c, launch_dslash(A, in.prec, gprec, ny, std::get<0>(sh), std::get<1>(sh), std::get<2>(sh), st));
+    if (std::get<2>(sh) == 4 || std::get<2>(sh) == 5) {
+        c->wait_pending = true;
+        if (c->pdl) c->wait_in_graphs = true;
+    }
     c->dslash_launches++;
     return OV_OK;
 }
@@ -492,6 +500,7 @@ void graphs_clear(ov_ctx* c)
     cudaDeviceSynchronize();
     for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second.first);
     c->graphs.clear();
+    c->wait_in_graphs = false;
 }
 
 // Run `body(s)` (a fixed sequence of kernel launches on stream s) through a
@@ -531,6 +540,7 @@ static int with_graph(ov_ctx* c, int kind, const FieldDesc& in, const FieldDesc&
     auto it = c->graphs.find(key);
     if (it != c->graphs.end()) {
         OV_CUDA(c, cudaGraphLaunch(it->second.first, gs));
+        if (c->wait_in_graphs) c->wait_pending = true;
         c->dslash_launches += it->second.second;
         c->graph_replays++;
         return join();
@@ -923,7 +933,7 @@ static int apply_canonical(ov_ctx* c, const void* in, void* out, double m, int n
     FieldDesc fi, fo;
     OV_TRY(ws_field(c, WS_IN, prec, nrhs, &fi));
     OV_TRY(ws_field(c, WS_OUT, prec, nrhs, &fo));
-    OV_CUDA(c, launch_pack(c->g, din, fi, 0, st));
+    OV_CUDA(c, launch_pack(c->g, din, fi, st));
     if (kind == 2) {
         OV_TRY(overlap_apply(c, fi, fo, m, st));
     } else if (kind == 3) {
@@ -934,7 +944,7 @@ static int apply_canonical(ov_ctx* c, const void* in, void* out, double m, int n
     } else {
         OV_TRY(dslash_apply(c, fi, fo, 4.0 + m, -0.5, kind == 1, 0, 0, nullptr, nullptr, st));
     }
-    OV_CUDA(c, launch_unpack(c->g, fo, dout, 0, st));
+    OV_CUDA(c, launch_unpack(c->g, fo, dout, st));
     OV_TRY(stage_out_finish(c, out, dout, bytes, st));
     return check_kernel_flags(c, st);
 }
@@ -1056,7 +1066,7 @@ int ov_set_eigenpairs(ov_ctx* c, int which, int nev, const double* vals, const v
         FieldDesc sub = E.vec[P_F64];
         sub.nrhs = n;
         sub.data = E.vec[P_F64].data + (size_t)i0 * E.vec[P_F64].rhs_bytes();
-        OV_CUDA(c, launch_pack(c->g, src, sub, 0, st));
+        OV_CUDA(c, launch_pack(c->g, src, sub, st));
         OV_CUDA(c, cudaStreamSynchronize(st));
     }
     E.nev = nev;
@@ -1089,7 +1099,7 @@ int ov_get_eigenpairs(ov_ctx* c, int which, int* nev, double* vals, void* vecs, 
             FieldDesc sub = E.vec[P_F64];
             sub.nrhs = n;
             sub.data = E.vec[P_F64].data + (size_t)i0 * E.vec[P_F64].rhs_bytes();
-            OV_CUDA(c, launch_unpack(c->g, sub, dst, 0, st));
+            OV_CUDA(c, launch_unpack(c->g, sub, dst, st));
             OV_TRY(stage_out_finish(c, hdst, dst, one * n, st));
         }
         OV_CUDA(c, cudaStreamSynchronize(st));
@@ -1127,10 +1137,10 @@ int ov_cg_solve(ov_ctx* c, const void* b, void* x, int nrhs, double mass, double
     FieldDesc fb, fx;
     OV_TRY(ws_field(c, WS_CG_B, P_F64, nrhs, &fb));
     OV_TRY(ws_field(c, WS_CG_X, P_F64, nrhs, &fx));
-    OV_CUDA(c, launch_pack(c->g, db, fb, 0, st));
+    OV_CUDA(c, launch_pack(c->g, db, fb, st));
     int s = cg_impl(c, fb, fx, mass, tol, max_iter, precond, inner_prec, info, st);
     if (s != OV_OK && s != OV_ENOTCONV && s != OV_ESTALL) return s;
-    OV_CUDA(c, launch_unpack(c->g, fx, dx, 0, st));
+    OV_CUDA(c, launch_unpack(c->g, fx, dx, st));
     OV_TRY(stage_out_finish(c, x, dx, bytes, st));
     return s;
 }
@@ -1154,7 +1164,7 @@ int ov_cg_solve_multimass(ov_ctx* c, const void* b, void* x, int nrhs, int nmass
     OV_TRY(stage_in(c, 0, b, one, st, &db));
     FieldDesc fb;
     OV_TRY(ws_field(c, WS_CG_B, P_F64, nrhs, &fb));
-    OV_CUDA(c, launch_pack(c->g, db, fb, 0, st));
+    OV_CUDA(c, launch_pack(c->g, db, fb, st));
     // one accurate-precision solution field per mass (device memory for the duration of the call)
     std::vector<FieldDesc> fx(nmass);
     int s = OV_OK;
@@ -1168,7 +1178,7 @@ int ov_cg_solve_multimass(ov_ctx* c, const void* b, void* x, int nrhs, int nmass
             void* hx = (char*)x + one * k;
             s2 = stage_out_buffer(c, 1, hx, one, &dx);
             if (s2 == OV_OK) s2 = convert(c, fx[k], f64, st);
-            if (s2 == OV_OK && launch_unpack(c->g, f64, dx, 0, st) != cudaSuccess)
+            if (s2 == OV_OK && launch_unpack(c->g, f64, dx, st) != cudaSuccess)
                 s2 = set_err(c, OV_ECUDA, "multimass: unpack failed");
             if (s2 == OV_OK) s2 = stage_out_finish(c, hx, dx, one, st);
         }
@@ -1211,7 +1221,7 @@ int ov_field_import(ov_ctx* c, ov_field* f, const void* canonical, void* stream)
     const size_t bytes = (size_t)f->d.nrhs * 2 * c->g.Vh * 12 * 16;
     const double* src = nullptr;
     OV_TRY(stage_in(c, 0, canonical, bytes, st, &src));
-    OV_CUDA(c, launch_pack(c->g, src, f->d, 0, st));
+    OV_CUDA(c, launch_pack(c->g, src, f->d, st));
     return OV_OK;
 }
 
@@ -1222,7 +1232,7 @@ int ov_field_export(ov_ctx* c, const ov_field* f, void* canonical, void* stream)
     const size_t bytes = (size_t)f->d.nrhs * 2 * c->g.Vh * 12 * 16;
     double* dst = nullptr;
     OV_TRY(stage_out_buffer(c, 1, canonical, bytes, &dst));
-    OV_CUDA(c, launch_unpack(c->g, f->d, dst, 0, st));
+    OV_CUDA(c, launch_unpack(c->g, f->d, dst, st));
     return stage_out_finish(c, canonical, dst, bytes, st);
 }
 
@@ -1514,6 +1524,7 @@ int ov_tune_dslash(ov_ctx* c, int prec, int nrhs, int* bx, int* by, int* variant
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    OV_TRY(check_kernel_flags(c, st));
     c->shape[{prec, nrhs}] = bsh;
     if (bx) *bx = std::get<0>(bsh);
     if (by) *by = std::get<1>(bsh);

@@ -106,6 +106,10 @@ struct ov_ctx {
     cudaStream_t gstream = nullptr;
     cudaEvent_t gev[2] = {nullptr, nullptr};
 
+    // bounded waits: launches of the bulk-copy dslash variants (the only ones that wait) whose timeout flag
+    // has not been read yet, and whether a captured graph holds such launches
+    bool wait_pending = false, wait_in_graphs = false;
+
     // instrumentation: number of dslash launches issued through this context
     long long dslash_launches = 0;
 

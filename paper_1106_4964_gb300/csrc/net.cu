@@ -670,9 +670,9 @@ int ov_net_apply(ov_ctx* c, const void* in, void* out, int nrhs, void* stream)
     FieldDesc fi, fo;
     OV_TRY(ws_field(c, WS_IN, P_F32, nrhs, &fi));
     OV_TRY(ws_field(c, WS_OUT, P_F32, nrhs, &fo));
-    OV_CUDA(c, launch_pack(c->g, din, fi, 0, st));
+    OV_CUDA(c, launch_pack(c->g, din, fi, st));
     OV_TRY(net_apply_precond(c, fi, fo, st));
-    OV_CUDA(c, launch_unpack(c->g, fo, dout, 0, st));
+    OV_CUDA(c, launch_unpack(c->g, fo, dout, st));
     return stage_out_finish(c, out, dout, bytes, st);
 }
 
@@ -689,9 +689,9 @@ int ov_net_loss_grad(ov_ctx* c, const void* r, const void* e, int npairs, double
     OV_TRY(ws_field(c, WS_CG_R, P_F32, npairs, &fr));
     OV_TRY(ws_field(c, WS_CG_T, P_F32, npairs, &fe));
     OV_TRY(stage_in(c, 0, r, bytes, st, &dr));
-    OV_CUDA(c, launch_pack(c->g, dr, fr, 0, st));
+    OV_CUDA(c, launch_pack(c->g, dr, fr, st));
     OV_TRY(stage_in(c, 1, e, bytes, st, &de));
-    OV_CUDA(c, launch_pack(c->g, de, fe, 0, st));
+    OV_CUDA(c, launch_pack(c->g, de, fe, st));
     OV_TRY(loss_grad(c, fr, fe, 0, npairs, loss, st));
     if (grad) {
         std::vector<float2> h(NET_PARAMS);

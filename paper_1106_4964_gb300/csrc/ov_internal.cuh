@@ -283,6 +283,48 @@ __device__ __forceinline__ df64 to_df(R v)
         return df64(v);
 }
 
+// FP64 <-> FP32 with integer instructions (GB300 converts 2 values per clock and SM on its FP64 pipe): normal
+// numbers and zeros; the rest (subnormals, infinities, NaN, overflow) by the conversion instruction
+__device__ __forceinline__ float f64_to_f32(double x)
+{
+    const uint32_t hi = f64_hi(x), lo = f64_lo(x), a = hi & 0x7fffffffu;
+    // round to nearest even at bit 29 of the low word; a carry moves into the exponent
+    uint32_t f = __funnelshift_l(lo, a - (896u << 20), 3);
+    f += (lo & 0x1fffffffu) + (f & 1u) > 0x10000000u;
+    if (a - (897u << 20) < (254u << 20)) return __uint_as_float(f | (hi & 0x80000000u));
+    if ((a | lo) == 0) return __uint_as_float(hi);
+    return (float)x;
+}
+__device__ __forceinline__ double f32_to_f64(float x)
+{
+    const uint32_t b = __float_as_uint(x), a = b & 0x7fffffffu;
+    if (a - 0x00800000u < 0x7f000000u) return f64_bits(((a >> 3) + (896u << 20)) | (b & 0x80000000u), b << 29);
+    if (a == 0) return f64_bits(b, 0u);
+    return (double)x;
+}
+template <typename R>
+__device__ __forceinline__ R from_f64(double x)
+{
+    if constexpr (std::is_same<R, double>::value) {
+        return x;
+    } else if constexpr (std::is_same<R, float>::value) {
+        return f64_to_f32(x);
+    } else {
+        const float h = f64_to_f32(x);
+        return df64(h, f64_to_f32(x - f32_to_f64(h)));
+    }
+}
+template <typename R>
+__device__ __forceinline__ double to_f64(R x)
+{
+    if constexpr (std::is_same<R, double>::value)
+        return x;
+    else if constexpr (std::is_same<R, float>::value)
+        return f32_to_f64(x);
+    else
+        return f32_to_f64(x.hi) + f32_to_f64(x.lo);
+}
+
 template <int P, typename Real>
 __device__ __forceinline__ void load_spinor(const char* __restrict__ base, const float* __restrict__ nrm,
                                             int Vh, int s, Real v[24])

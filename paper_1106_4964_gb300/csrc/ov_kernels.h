@@ -49,8 +49,8 @@ constexpr int DSLASH_VARIANTS = 12;
 
 // ---------------------------------------------------------------- layout conversion
 // canonical complex128 [nrhs][V][12] (device) <-> internal field
-cudaError_t launch_pack(const Geom& g, const double* canon, const FieldDesc& f, int gamma5, cudaStream_t st);
-cudaError_t launch_unpack(const Geom& g, const FieldDesc& f, double* canon, int gamma5, cudaStream_t st);
+cudaError_t launch_pack(const Geom& g, const double* canon, const FieldDesc& f, cudaStream_t st);
+cudaError_t launch_unpack(const Geom& g, const FieldDesc& f, double* canon, cudaStream_t st);
 // canonical complex128 gauge [V][4][3][3] (device) -> reconstruct-12 links in `prec`;
 // *dev_err receives max |U U^dag - 1| and max |row2 - conj(row0 x row1)| (as float bits, atomicMax)
 cudaError_t launch_pack_gauge(const Geom& g, const double* canon, void* out, int prec, unsigned* dev_err,

@@ -922,12 +922,19 @@ int cg_impl(ov_ctx* c, const FieldDesc& b_in, const FieldDesc& x_out, double mas
         OV_CUDA(c, launch_proj_update(c->g, xi64, nd, (const double2*)c->dscal, nullptr, v, v, none, st));
         return OV_OK;
     };
+    bool x_zero = !warm;
     auto refresh = [&](bool& all_done) -> int {
-        if (nzero) OV_TRY(drop_zero_modes(x));
-        OV_TRY(normal_apply(c, x, t, mass, st));
-        FieldDesc v2[2] = {b, t};
-        double2 h2[2] = {make_double2(1, 0), make_double2(-1, 0)};
-        OV_TRY(lincomb(c, r, 2, v2, h2, nullptr, 0, dnr, st));
+        if (x_zero) {  // the first residual of a cold start is b: no application to a vanishing x
+            double2 h1[1] = {make_double2(1, 0)};
+            OV_TRY(lincomb(c, r, 1, &b, h1, nullptr, 0, dnr, st));
+            x_zero = false;
+        } else {
+            if (nzero) OV_TRY(drop_zero_modes(x));
+            OV_TRY(normal_apply(c, x, t, mass, st));
+            FieldDesc v2[2] = {b, t};
+            double2 h2[2] = {make_double2(1, 0), make_double2(-1, 0)};
+            OV_TRY(lincomb(c, r, 2, v2, h2, nullptr, 0, dnr, st));
+        }
         std::vector<double> nr(R);
         if (nzero) {
             OV_TRY(drop_zero_modes(r));
