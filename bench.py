@@ -58,7 +58,8 @@ def peaks():
 
 VARIANT_UNIT = {0: "dslash_regs.cu", 1: "dslash_regs.cu", 2: "dslash_regs.cu", 3: "dslash_staged.cu",
                 4: "dslash_staged.cu", 5: "dslash_staged.cu", 6: "dslash_multi.cu", 7: "dslash_multi.cu",
-                8: "dslash_batched.cu", 9: "dslash_batched.cu", 10: "dslash_pair.cu", 11: "dslash_pair.cu"}
+                8: "dslash_batched.cu", 9: "dslash_batched.cu", 10: "dslash_pair.cu", 11: "dslash_pair.cu",
+                12: "dslash_hop32.cu"}
 
 
 WIDE_UNIT = "dslash_split.cu"  # FP64 and double-float, every variant
@@ -100,6 +101,8 @@ def kernel_name(prec: str, var: int, nrhs: int = 1) -> str:
         return f"dslash_batched_kernel<{prec},{prec},hops_batched={4 if var == 8 else 8}>"
     if var in (10, 11):
         return f"dslash_pair_kernel<{prec},{prec},rhs_pairs_per_thread={1 if var == 10 else 2}>"
+    if var == 12:
+        return f"dslash_hop_kernel<{prec},{prec}>"
     return f"dslash_kernel<{prec},{prec},variant={var}>"
 
 

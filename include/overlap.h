@@ -387,7 +387,8 @@ int ov_get_option(const ov_ctx* ctx, const char* name, double* value);
  * loads of four or eight hops issued before their arithmetic (by = 1); 10, 11
  * two or four right-hand sides per thread as pairs on the packed FP32 pipe
  * (for 6, 7, 10, 11 `by` counts groups of right-hand sides and bx * by <=
- * 128).  Variants 3-11 take FP32 arithmetic (FP32 and 16-bit storage) only.
+ * 128); 12 one warp per hop of 32 sites (bx = 32, by = 1), for small lattices.
+ * Variants 3-12 take FP32 arithmetic (FP32 and 16-bit storage) only.
  * ov_tune_dslash times every candidate on `stream` and keeps the fastest
  * (the autotuner). */
 int ov_set_dslash_shape(ov_ctx* ctx, int prec, int nrhs, int bx, int by, int variant);

@@ -215,14 +215,20 @@ int eig_vectors(ov_ctx* c, int which, int prec, cudaStream_t st, FieldDesc* out)
     return OV_OK;
 }
 
-static std::tuple<int, int, int> default_shape(int prec, int nrhs)
+static std::tuple<int, int, int> default_shape(const Geom& g, int prec, int nrhs)
 {
     // FP64, double-float: one block of eight warps per 32 sites and right-hand side, with the registers each
     // form needs.  us per launch, 32 x 1 / 64 x 1 / 128 x 1: FP64 8^3 x 16 10.3 / 12.4 / 20; 24^3 x 64 488 / 498 /
     // 505; 12 rhs at 8^4 30.8 / 34.8 / 41; double-float 24^3 x 64 665 / 686 / 687
     if (wide(prec)) return {32, 1, prec == P_F64 ? 1 : 0};
-    if (nrhs == 1) return {128, 1, 0};
-    return {32, nrhs > 16 ? 16 : nrhs, 0};
+    // FP32 arithmetic by sites x right-hand sides.  One warp per hop while one site per thread would leave most
+    // of the chip idle (us, against 64 x 1 variant 0: 4^4 2.2 / 2.8, 8^4 2.3 / 3.0, FP16 8^3 x 16 3.1 / 3.5, two
+    // sources at 8^4 3.1 / 3.3; three 3.9 / 3.6 in BF16, 12^4 4.4 / 4.3); then unbounded registers while the
+    // blocks fit at once, and more resident warps beyond (variant 1 against 0: 12 sources at 8^3 x 16 9.1 / 9.0,
+    // two at 16^3 x 32 20.0 / 20.3, 12 there 101.7 / 107.5; blocks of 32 sites x 12 sources 157)
+    const long n = 2L * g.Vh * nrhs;
+    if (n <= 9000) return {32, 1, 12};
+    return {64, 1, n <= 200000 ? 0 : 1};
 }
 
 // a double as an unevaluated sum of two FP32 numbers
@@ -264,7 +270,7 @@ int dslash_apply(ov_ctx* c, const FieldDesc& in, const FieldDesc& out, double a,
     A.g5_core = g5_core;
     A.g5_out = g5_out;
     auto it = c->shape.find({in.prec, in.nrhs});
-    std::tuple<int, int, int> sh = it != c->shape.end() ? it->second : default_shape(in.prec, in.nrhs);
+    std::tuple<int, int, int> sh = it != c->shape.end() ? it->second : default_shape(c->g, in.prec, in.nrhs);
     OV_CUDA(c, launch_dslash(A, in.prec, gprec, ny, std::get<0>(sh), std::get<1>(sh), std::get<2>(sh), st));
     if (std::get<2>(sh) == 4 || std::get<2>(sh) == 5) {
         c->wait_pending = true;
@@ -1445,6 +1451,7 @@ int ov_set_dslash_shape(ov_ctx* c, int prec, int nrhs, int bx, int by, int varia
         ((variant == 3 || variant == 4 || variant == 5) && by != 1))
         return set_err(c, OV_EINVAL, "bad variant %d for this precision / shape", variant);
     const int maxt = variant == 0 ? (wide(prec) ? 256 : 512) : (variant == 3 || variant >= 6 ? 128 : 256);
+    if (variant == 12 && (bx != 32 || by != 1)) return set_err(c, OV_EINVAL, "variant 12: bx = 32, by = 1");
     if ((variant == 8 || variant == 9) && by != 1) return set_err(c, OV_EINVAL, "variants 8, 9: by must be 1");
     if (bx < 1 || by < 1 || bx * by > maxt || bx % 32) return set_err(c, OV_EINVAL, "bad shape %d x %d", bx, by);
     c->shape[{prec, nrhs}] = std::make_tuple(bx, by, variant);
@@ -1469,6 +1476,10 @@ int ov_tune_dslash(ov_ctx* c, int prec, int nrhs, int* bx, int* by, int* variant
         if (v >= 3 && wide(prec)) continue;  // staged variants: FP32 arithmetic only
         if (v == 4 || v == 5) {              // bulk-copy staging: fixed 128-site blocks
             cand.push_back(std::make_tuple(128, 1, v));
+            continue;
+        }
+        if (v == 12) {                       // one warp per hop
+            cand.push_back(std::make_tuple(32, 1, v));
             continue;
         }
         if (v == 8 || v == 9) {              // batched hop loads: 128-thread blocks, one rhs per block row
@@ -1499,7 +1510,7 @@ int ov_tune_dslash(ov_ctx* c, int prec, int nrhs, int* bx, int* by, int* variant
                 cand.push_back(std::make_tuple(x, y, v));
             }
     }
-    if (cand.empty()) cand.push_back(default_shape(prec, nrhs));
+    if (cand.empty()) cand.push_back(default_shape(c->g, prec, nrhs));
     cudaEvent_t e0, e1;
     OV_CUDA(c, cudaEventCreate(&e0));
     OV_CUDA(c, cudaEventCreate(&e1));

@@ -17,6 +17,7 @@ cudaError_t launch_dslash(const DslashArgs& A, int sp, int gp, int ny, int bx, i
     if (var == 6 || var == 7) return launch_dslash_multi(A, sp, gp, ny, var, grid, block, st);
     if (var == 8 || var == 9) return launch_dslash_batched(A, sp, gp, ny, var, grid, block, st);
     if (var == 10 || var == 11) return launch_dslash_pair(A, sp, gp, ny, var, grid, block, st);
+    if (var == 12) return launch_dslash_hop32(A, sp, gp, ny, var, grid, block, st);
     return cudaErrorInvalidValue;
 }
 

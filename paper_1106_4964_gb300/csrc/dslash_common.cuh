@@ -213,6 +213,10 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 template <class... P, class... Args>
 cudaError_t launch_kernel(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t st, bool pdl, const Args&... args)
 {
+    if (!pdl) {
+        k<<<grid, block, 0, st>>>(P(args)...);
+        return cudaGetLastError();
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -221,7 +225,7 @@ cudaError_t launch_kernel(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t s
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
-    cfg.numAttrs = pdl ? 1 : 0;
+    cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k, P(args)...);
 }
 
@@ -311,6 +315,80 @@ __device__ __forceinline__ void epilogue(const DslashArgs& A, int r, int p, int 
         for (int i = 12; i < 24; ++i) o[i] = -o[i];
     }
     store_spinor<SP, Real>(A.out + off, A.out_n ? A.out_n + noff : nullptr, g.Vh, s, o);
+}
+
+// Neighbour index and boundary flag of hop w (+x, -x, ... -t; warp-uniform)
+__device__ __forceinline__ void hop_neighbour(const Geom& g, int w, int s, const int c[4], int& sn, bool& cross)
+{
+    switch (w) {
+    case 0: sn = cb_neighbour<0>(g, s, c); cross = c[0] + 1 == g.L[0]; break;
+    case 1: sn = cb_neighbour<1>(g, s, c); cross = c[0] == 0; break;
+    case 2: sn = cb_neighbour<2>(g, s, c); cross = c[1] + 1 == g.L[1]; break;
+    case 3: sn = cb_neighbour<3>(g, s, c); cross = c[1] == 0; break;
+    case 4: sn = cb_neighbour<4>(g, s, c); cross = c[2] + 1 == g.L[2]; break;
+    case 5: sn = cb_neighbour<5>(g, s, c); cross = c[2] == 0; break;
+    case 6: sn = cb_neighbour<6>(g, s, c); cross = c[3] + 1 == g.L[3]; break;
+    default: sn = cb_neighbour<7>(g, s, c); cross = c[3] == 0; break;
+    }
+}
+
+template <typename Real>
+__device__ __forceinline__ void project_hop(int w, const Real v[24], Real h[12])
+{
+    switch (w) {
+    case 0: project<0, +1, Real>(v, h); break;
+    case 1: project<0, -1, Real>(v, h); break;
+    case 2: project<1, +1, Real>(v, h); break;
+    case 3: project<1, -1, Real>(v, h); break;
+    case 4: project<2, +1, Real>(v, h); break;
+    case 5: project<2, -1, Real>(v, h); break;
+    case 6: project<3, +1, Real>(v, h); break;
+    default: project<3, -1, Real>(v, h); break;
+    }
+}
+
+// Complex component (spin sp, warp-uniform; one colour) of the hop sum: the upper spins add the hops'
+// results, the lower ones subtract S A_mu^dag of them (accumulate() of dslash_common.cuh, hop by hop in
+// the same order).  ld(hop, a, re, im): result of spin a.
+template <class V, class L>
+__device__ __forceinline__ void sum_hops(int sp, L ld, V& re, V& im)
+{
+    V x, y;
+    re = im = V(0);
+    if (sp < 2) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            ld(k, sp, x, y);
+            re += x;
+            im += y;
+        }
+        return;
+    }
+    const int b = sp - 2;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int mu = k >> 1;
+        ld(k, mu < 2 ? 1 - b : b, x, y);
+        // A_mu^dag chi: rows (i x1, i x0), (x1, -x0), (i x0, -i x1), (x0, x1)
+        const bool neg = ((k & 1) == 0) != ((mu == 1 || mu == 2) && b == 1);
+        if (mu == 0 || mu == 2) {
+            if (neg) {
+                re += y;
+                im -= x;
+            } else {
+                re -= y;
+                im += x;
+            }
+        } else {
+            if (neg) {
+                re -= x;
+                im -= y;
+            } else {
+                re += x;
+                im += y;
+            }
+        }
+    }
 }
 
 // Host side of block_work: the one-dimensional grid of a launch with site blocks of bx sites

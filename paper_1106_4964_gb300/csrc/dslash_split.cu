@@ -93,16 +93,7 @@ __device__ __forceinline__ void load_half(const DslashArgs& A, const char* in_q,
     using Real = real_t<SP>;
     Real v[24];
     load_spinor<SP, Real>(in_q, nullptr, A.g.Vh, sn, v);
-    switch (w) {
-    case 0: project<0, +1, Real>(v, h); break;
-    case 1: project<0, -1, Real>(v, h); break;
-    case 2: project<1, +1, Real>(v, h); break;
-    case 3: project<1, -1, Real>(v, h); break;
-    case 4: project<2, +1, Real>(v, h); break;
-    case 5: project<2, -1, Real>(v, h); break;
-    case 6: project<3, +1, Real>(v, h); break;
-    default: project<3, -1, Real>(v, h); break;
-    }
+    project_hop<Real>(w, v, h);
     if (cross && A.g.fbc[w >> 1] != 1.f) {
         const Real f = (Real)A.g.bc[w >> 1];
 #pragma unroll
@@ -169,50 +160,6 @@ __device__ __noinline__ void hop_real(const DslashArgs& A, const char* in_q, con
     for (int k = 0; k < 6; ++k) out[k * 32] = Wide<SP>::put(chi[2 * k], chi[2 * k + 1]);
 }
 
-// Complex component (spin sp, warp-uniform; one colour) of the hop sum: the upper spins add the hops'
-// results, the lower ones subtract S A_mu^dag of them (accumulate() of dslash_common.cuh, hop by hop in
-// the same order).  ld(hop, a, re, im): result of spin a.
-template <class V, class L>
-__device__ __forceinline__ void sum_hops(int sp, L ld, V& re, V& im)
-{
-    V x, y;
-    re = im = V(0);
-    if (sp < 2) {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            ld(k, sp, x, y);
-            re += x;
-            im += y;
-        }
-        return;
-    }
-    const int b = sp - 2;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const int mu = k >> 1;
-        ld(k, mu < 2 ? 1 - b : b, x, y);
-        // A_mu^dag chi: rows (i x1, i x0), (x1, -x0), (i x0, -i x1), (x0, x1)
-        const bool neg = ((k & 1) == 0) != ((mu == 1 || mu == 2) && b == 1);
-        if (mu == 0 || mu == 2) {
-            if (neg) {
-                re += y;
-                im -= x;
-            } else {
-                re -= y;
-                im += x;
-            }
-        } else {
-            if (neg) {
-                re -= x;
-                im -= y;
-            } else {
-                re += x;
-                im += y;
-            }
-        }
-    }
-}
-
 template <int SP, int NY, int MINB>
 __global__ void __launch_bounds__(SPLIT_THREADS, MINB) dslash_split_kernel(const __grid_constant__ DslashArgs A, int ngrp, int nby)
 {
@@ -235,16 +182,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, MINB) dslash_split_kernel(const
         int c[4], sn;
         bool cross;
         cb_coords(g, s, p, c);
-        switch (w) {
-        case 0: sn = cb_neighbour<0>(g, s, c); cross = c[0] + 1 == g.L[0]; break;
-        case 1: sn = cb_neighbour<1>(g, s, c); cross = c[0] == 0; break;
-        case 2: sn = cb_neighbour<2>(g, s, c); cross = c[1] + 1 == g.L[1]; break;
-        case 3: sn = cb_neighbour<3>(g, s, c); cross = c[1] == 0; break;
-        case 4: sn = cb_neighbour<4>(g, s, c); cross = c[2] + 1 == g.L[2]; break;
-        case 5: sn = cb_neighbour<5>(g, s, c); cross = c[2] == 0; break;
-        case 6: sn = cb_neighbour<6>(g, s, c); cross = c[3] + 1 == g.L[3]; break;
-        default: sn = cb_neighbour<7>(g, s, c); cross = c[3] == 0; break;
-        }
+        hop_neighbour(g, w, s, c, sn, cross);
         const bool fwd = (w & 1) == 0;
         const int ls = fwd ? s : sn;
         const char* lb = A.gauge + (size_t)((fwd ? p : q) * 4 + (w >> 1)) * g.Vh * 144;

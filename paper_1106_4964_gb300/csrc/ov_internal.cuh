@@ -397,6 +397,18 @@ __device__ __forceinline__ float load_spinor_unscaled(const char* __restrict__ b
     return __ldg(nrm + s);
 }
 
+// eight 16-bit values x[0..7] * inv
+template <int P>
+__device__ __forceinline__ uint4 half_chunk(const float* x, float inv)
+{
+    uint4 t;
+    t.x = Half<P>::from2(x[0] * inv, x[1] * inv);
+    t.y = Half<P>::from2(x[2] * inv, x[3] * inv);
+    t.z = Half<P>::from2(x[4] * inv, x[5] * inv);
+    t.w = Half<P>::from2(x[6] * inv, x[7] * inv);
+    return t;
+}
+
 template <int P, typename Real>
 __device__ __forceinline__ void store_spinor(char* __restrict__ base, float* __restrict__ nrm, int Vh, int s,
                                              const Real v[24])
@@ -419,22 +431,34 @@ __device__ __forceinline__ void store_spinor(char* __restrict__ base, float* __r
             b[(size_t)k * Vh + s] =
                 make_float4((float)v[4 * k], (float)v[4 * k + 1], (float)v[4 * k + 2], (float)v[4 * k + 3]);
     } else {
-        float m = 0.f;
+        float f[24], m = 0.f;
 #pragma unroll
-        for (int i = 0; i < 24; ++i) m = fmaxf(m, fabsf((float)v[i]));
+        for (int i = 0; i < 24; ++i) {
+            f[i] = (float)v[i];
+            m = fmaxf(m, fabsf(f[i]));
+        }
         float inv = m > 0.f ? 1.0f / m : 0.f;
         uint4* b = reinterpret_cast<uint4*>(base);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            uint4 t;
-            t.x = Half<P>::from2((float)v[8 * k + 0] * inv, (float)v[8 * k + 1] * inv);
-            t.y = Half<P>::from2((float)v[8 * k + 2] * inv, (float)v[8 * k + 3] * inv);
-            t.z = Half<P>::from2((float)v[8 * k + 4] * inv, (float)v[8 * k + 5] * inv);
-            t.w = Half<P>::from2((float)v[8 * k + 6] * inv, (float)v[8 * k + 7] * inv);
-            b[(size_t)k * Vh + s] = t;
-        }
+        for (int k = 0; k < 3; ++k) b[(size_t)k * Vh + s] = half_chunk<P>(f + 8 * k, inv);
         nrm[s] = m;
     }
+}
+
+// chunk w (0..2, warp-uniform) of a 16-bit store_spinor; chunk 0 writes the scale
+template <int P>
+__device__ __forceinline__ void store_spinor_chunk(char* __restrict__ base, float* __restrict__ nrm, int Vh, int s,
+                                                   const float v[24], int w)
+{
+    float m = 0.f;
+#pragma unroll
+    for (int i = 0; i < 24; ++i) m = fmaxf(m, fabsf(v[i]));
+    const float inv = m > 0.f ? 1.0f / m : 0.f;
+    uint4* b = reinterpret_cast<uint4*>(base);
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        if (k == w) b[(size_t)k * Vh + s] = half_chunk<P>(v + 8 * k, inv);
+    if (w == 0) nrm[s] = m;
 }
 
 // ---------------------------------------------------------------------------
