@@ -389,8 +389,9 @@ int ov_get_option(const ov_ctx* ctx, const char* name, double* value);
  * (for 6, 7, 10, 11 `by` counts groups of right-hand sides and bx * by <=
  * 128); 12 one warp per hop of 32 sites (bx = 32, by = 1), for small lattices.
  * Variants 3-12 take FP32 arithmetic (FP32 and 16-bit storage) only.
- * ov_tune_dslash times every candidate on `stream` and keeps the fastest
- * (the autotuner). */
+ * ov_tune_dslash times every candidate on `stream` and keeps the fastest, or
+ * the default launch when no candidate is faster by more than the timing
+ * scatters (the autotuner). */
 int ov_set_dslash_shape(ov_ctx* ctx, int prec, int nrhs, int bx, int by, int variant);
 int ov_tune_dslash(ov_ctx* ctx, int prec, int nrhs, int* bx, int* by, int* variant, void* stream);
 

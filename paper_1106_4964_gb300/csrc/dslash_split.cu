@@ -9,10 +9,10 @@
 // the multiply in the instruction cache instead of eight (the straight-line double-float kernel was
 // 14 000 instructions and stalled on instruction fetch for three quarters of its time).
 //
-// us per launch at 24^3 x 64 / 12 right-hand sides at 8^3 x 16 / one at 4^4: FP64 488 / 57 / 7.9 (one
-// thread per site and FP64 multiply-adds: 1583 / 190 / 35), double-float 665 / 80 / 7.7 (973 / 209 / 30).
-// FP64: integer and FP64 pipes each 42 % busy, half of the issue slots used; double-float: integer
-// pipe 57 % (the conversions from and to pairs), the rest latency between dependent operations.
+// us per launch at 24^3 x 64 / 12 right-hand sides at 8^3 x 16 / one at 4^4: FP64 423 / 54 / 5.9 (one thread
+// per site and FP64 multiply-adds: 1583 / 190 / 33), double-float 592 / 70 / 6.0 (973 / 209 / 28).  The integer
+// multiply pipe is 57 %, the integer and FP64 pipes 42 % busy (FP64); half of the issue slots are used, the
+// rest waits on dependent operations and the block's barriers.
 //
 // A block walks over bx / 32 groups of sites and `by` right-hand sides (the innermost, so that a site
 // group's links are re-read from L1).  Sites that the fixed-point format does not hold send their
@@ -102,44 +102,43 @@ __device__ __forceinline__ void load_half(const DslashArgs& A, const char* in_q,
 }
 
 // U h (forward) or U^dag h in fixed point: out[(3 a + i) * 32] = spin a, colour i.  One code for both
-// directions (half the instructions to fetch): the backward hop reads the link's transpose and negates
-// its imaginary parts.
+// directions and both spins (a quarter of the instructions to fetch, half the live registers: the link is
+// read again for the second spin, from L1): the backward hop reads the link's transpose and negates its
+// imaginary parts.  h is overwritten.
 template <int SP>
-__device__ __forceinline__ void colour_fix(const int4* lb, int Vh, bool fwd, const real_t<SP> h[12], uint32_t emax,
-                                           int4* out)
+__device__ __forceinline__ void colour_fix(const int4* lb, int Vh, bool fwd, real_t<SP> h[12], uint32_t emax, int4* out)
 {
-    Fix f[12], n[6];  // n = -Im h
-#pragma unroll
-    for (int i = 0; i < 12; ++i) f[i] = Wide<SP>::fix(h[i], emax);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) n[i] = fix_neg(f[2 * i + 1]);
     const int m = fwd ? 0 : -1;
-    if (emax == 0) {  // a vanishing hop contributes exactly nothing
-#pragma unroll
-        for (int i = 0; i < 6; ++i) n[i].l = 0;
-    }
     const size_t si = (size_t)(fwd ? 3 : 1) * Vh, sj = (size_t)(fwd ? 1 : 3) * Vh;
+#pragma unroll 1
+    for (int a = 0; a < 2; ++a) {
+        Fix f[6], n[3];  // n = -Im h
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        FixProd re[2] = {}, im[2] = {};
+        for (int i = 0; i < 6; ++i) f[i] = Wide<SP>::fix(h[i], emax);
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            const int4 t = __ldg(lb + i * si + j * sj);
-            const Fix ur{t.x, t.y}, ui{(t.z ^ m) - m, t.w ^ m};
+        for (int i = 0; i < 3; ++i) n[i] = fix_neg(f[2 * i + 1]);
+        if (emax == 0) {  // a vanishing hop contributes exactly nothing
 #pragma unroll
-            for (int a = 0; a < 2; ++a) {
-                const int k = 3 * a + j;
-                fix_mac(re[a], ur, f[2 * k]);
-                fix_mac(re[a], ui, n[k]);
-                fix_mac(im[a], ur, f[2 * k + 1]);
-                fix_mac(im[a], ui, f[2 * k]);
+            for (int i = 0; i < 3; ++i) n[i].l = 0;
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            FixProd re = {}, im = {};
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const int4 t = __ldg(lb + i * si + j * sj);
+                const Fix ur{t.x, t.y}, ui{(t.z ^ m) - m, t.w ^ m};
+                fix_mac(re, ur, f[2 * j]);
+                fix_mac(re, ui, n[j]);
+                fix_mac(im, ur, f[2 * j + 1]);
+                fix_mac(im, ui, f[2 * j]);
             }
+            const long long x = fix_sum(re), y = fix_sum(im);
+            out[i * 32] = make_int4((int)x, (int)(x >> 32), (int)y, (int)(y >> 32));
         }
+        out += 3 * 32;
 #pragma unroll
-        for (int a = 0; a < 2; ++a) {
-            const long long x = fix_sum(re[a]), y = fix_sum(im[a]);
-            out[(3 * a + i) * 32] = make_int4((int)x, (int)(x >> 32), (int)y, (int)(y >> 32));
-        }
+        for (int i = 0; i < 6; ++i) h[i] = h[i + 6];
     }
 }
 
