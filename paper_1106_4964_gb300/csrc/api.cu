@@ -1499,8 +1499,8 @@ int ov_tune_dslash(ov_ctx* c, int prec, int nrhs, int* bx, int* by, int* variant
         }
         if (wide(prec)) {                    // a block walks over x / 32 site groups and y right-hand sides
             for (int x : {32, 64, 128})
-                for (int y = 1; y <= nrhs && y <= 4; ++y)
-                    if (nrhs % y == 0) cand.push_back(std::make_tuple(x, y, v));
+                for (int y = 1; y <= nrhs && x * y <= 256; ++y)  // the limit of launch_dslash
+                    if (y <= 4 && nrhs % y == 0) cand.push_back(std::make_tuple(x, y, v));
             continue;
         }
         const int maxt = v == 0 ? 512 : (v == 3 ? 128 : 256);

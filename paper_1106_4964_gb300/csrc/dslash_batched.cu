@@ -161,19 +161,15 @@ __global__ void __launch_bounds__(128) dslash_batched_kernel(DslashArgs A)
 template <int SP, int GP, int NB>
 cudaError_t launch_batched(const DslashArgs& A, int ny, dim3 grid, dim3 block, cudaStream_t st)
 {
-    if constexpr (wide_dev<SP>) {
-        return cudaErrorInvalidValue;
-    } else {
-        if ((int)(block.x * block.y) > 128) return cudaErrorInvalidValue;
-        switch (ny) {
-        case 0: dslash_batched_kernel<SP, GP, 0, NB><<<grid, block, 0, st>>>(A); break;
-        case 1: dslash_batched_kernel<SP, GP, 1, NB><<<grid, block, 0, st>>>(A); break;
-        case 2: dslash_batched_kernel<SP, GP, 2, NB><<<grid, block, 0, st>>>(A); break;
-        case 3: dslash_batched_kernel<SP, GP, 3, NB><<<grid, block, 0, st>>>(A); break;
-        default: return cudaErrorInvalidValue;
-        }
-        return cudaGetLastError();
+    if ((int)(block.x * block.y) > 128) return cudaErrorInvalidValue;
+    switch (ny) {
+    case 0: dslash_batched_kernel<SP, GP, 0, NB><<<grid, block, 0, st>>>(A); break;
+    case 1: dslash_batched_kernel<SP, GP, 1, NB><<<grid, block, 0, st>>>(A); break;
+    case 2: dslash_batched_kernel<SP, GP, 2, NB><<<grid, block, 0, st>>>(A); break;
+    case 3: dslash_batched_kernel<SP, GP, 3, NB><<<grid, block, 0, st>>>(A); break;
+    default: return cudaErrorInvalidValue;
     }
+    return cudaGetLastError();
 }
 
 struct Batched {

@@ -25,8 +25,9 @@
 // which gives D_w (a = 4+m, b = -1/2), H_w (g5_core), and the fused
 // Clenshaw step b_k = c_k psi_h + alpha H_w t + beta b_{k+1} - b_{k+2}.
 //
-// The kernels are split over translation units by launch variant (dslash_regs.cu: 0-2,
-// dslash_staged.cu: 3-5, dslash_multi.cu: 6-7, dslash_batched.cu: 8-9, dslash_pair.cu: 10-11), so that
+// The kernels are split over translation units by launch variant (FP32 arithmetic: dslash_regs.cu: 0-2,
+// dslash_staged.cu: 3-5, dslash_multi.cu: 6-7, dslash_batched.cu: 8-9, dslash_pair.cu: 10-11, dslash_hop32.cu:
+// 12; FP64 and double-float: dslash_split.cu), so that
 // they compile in parallel; this header holds what they share.
 #pragma once
 
@@ -41,8 +42,6 @@ namespace {
 
 template <int SP>
 using real_t = typename std::conditional<SP == P_F64, double, typename std::conditional<SP == P_DF64, df64, float>::type>::type;
-template <int SP>
-constexpr bool wide_dev = SP == P_F64 || SP == P_DF64;
 
 template <int MU, int S, typename Real>
 __device__ __forceinline__ void project(const Real v[24], Real h[12])
@@ -213,8 +212,8 @@ __device__ __forceinline__ void epilogue(const DslashArgs& A, int r, int p, int 
 // the registers so that more warps are resident to hide load latency.
 template <int SP, int VAR>
 struct Bounds {
-    static constexpr int maxt = VAR == 0 ? (wide_dev<SP> ? 256 : 512) : 256;
-    static constexpr int minb = VAR == 0 ? 1 : (wide_dev<SP> ? VAR + 1 : VAR + 2);
+    static constexpr int maxt = VAR == 0 ? 512 : 256;
+    static constexpr int minb = VAR == 0 ? 1 : VAR + 2;
 };
 
 // Programmatic dependent launch: a kernel lets its successor's blocks start as soon as all of its own have

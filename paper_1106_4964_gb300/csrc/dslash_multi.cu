@@ -84,21 +84,17 @@ __global__ void __launch_bounds__(128) dslash_multi_kernel(DslashArgs A)
 template <int SP, int GP, int RB>
 cudaError_t launch_multi(const DslashArgs& A, int ny, dim3 block, cudaStream_t st)
 {
-    if constexpr (wide_dev<SP>) {
-        return cudaErrorInvalidValue;
-    } else {
-        if ((int)(block.x * block.y) > 128) return cudaErrorInvalidValue;
-        const int groups = (A.nrhs + RB - 1) / RB;
-        const dim3 grid = block_grid(A.g.Vh, block.x, (groups + block.y - 1) / block.y);
-        switch (ny) {
-        case 0: dslash_multi_kernel<SP, GP, 0, RB><<<grid, block, 0, st>>>(A); break;
-        case 1: dslash_multi_kernel<SP, GP, 1, RB><<<grid, block, 0, st>>>(A); break;
-        case 2: dslash_multi_kernel<SP, GP, 2, RB><<<grid, block, 0, st>>>(A); break;
-        case 3: dslash_multi_kernel<SP, GP, 3, RB><<<grid, block, 0, st>>>(A); break;
-        default: return cudaErrorInvalidValue;
-        }
-        return cudaGetLastError();
+    if ((int)(block.x * block.y) > 128) return cudaErrorInvalidValue;
+    const int groups = (A.nrhs + RB - 1) / RB;
+    const dim3 grid = block_grid(A.g.Vh, block.x, (groups + block.y - 1) / block.y);
+    switch (ny) {
+    case 0: dslash_multi_kernel<SP, GP, 0, RB><<<grid, block, 0, st>>>(A); break;
+    case 1: dslash_multi_kernel<SP, GP, 1, RB><<<grid, block, 0, st>>>(A); break;
+    case 2: dslash_multi_kernel<SP, GP, 2, RB><<<grid, block, 0, st>>>(A); break;
+    case 3: dslash_multi_kernel<SP, GP, 3, RB><<<grid, block, 0, st>>>(A); break;
+    default: return cudaErrorInvalidValue;
     }
+    return cudaGetLastError();
 }
 
 struct Multi {

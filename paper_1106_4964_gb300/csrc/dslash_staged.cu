@@ -180,34 +180,30 @@ __global__ void __launch_bounds__(128) dslash_staged_kernel(DslashArgs A)
 template <int SP, int GP>
 cudaError_t launch_staged(const DslashArgs& A, int ny, dim3 grid, dim3 block, cudaStream_t st)
 {
-    if constexpr (wide_dev<SP>) {
-        return cudaErrorInvalidValue;
-    } else {
-        if (block.y != 1 || block.x > 128) return cudaErrorInvalidValue;
-        const size_t shm = (size_t)block.x * AsyncLayout<SP, GP>::PER_THREAD;
-        static bool attr_set[4] = {false, false, false, false};
-        if (!attr_set[ny]) {
-            cudaError_t e = cudaSuccess;
-            switch (ny) {
-            case 0: e = cudaFuncSetAttribute(dslash_staged_kernel<SP, GP, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024); break;
-            case 1: e = cudaFuncSetAttribute(dslash_staged_kernel<SP, GP, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024); break;
-            case 2: e = cudaFuncSetAttribute(dslash_staged_kernel<SP, GP, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024); break;
-            case 3: e = cudaFuncSetAttribute(dslash_staged_kernel<SP, GP, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024); break;
-            default: return cudaErrorInvalidValue;
-            }
-            if (e != cudaSuccess) return e;
-            attr_set[ny] = true;
-        }
-        const dim3 g2 = block_grid(A.g.Vh, block.x, A.nrhs);
+    if (block.y != 1 || block.x > 128) return cudaErrorInvalidValue;
+    const size_t shm = (size_t)block.x * AsyncLayout<SP, GP>::PER_THREAD;
+    static bool attr_set[4] = {false, false, false, false};
+    if (!attr_set[ny]) {
+        cudaError_t e = cudaSuccess;
         switch (ny) {
-        case 0: dslash_staged_kernel<SP, GP, 0><<<g2, block, shm, st>>>(A); break;
-        case 1: dslash_staged_kernel<SP, GP, 1><<<g2, block, shm, st>>>(A); break;
-        case 2: dslash_staged_kernel<SP, GP, 2><<<g2, block, shm, st>>>(A); break;
-        case 3: dslash_staged_kernel<SP, GP, 3><<<g2, block, shm, st>>>(A); break;
+        case 0: e = cudaFuncSetAttribute(dslash_staged_kernel<SP, GP, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024); break;
+        case 1: e = cudaFuncSetAttribute(dslash_staged_kernel<SP, GP, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024); break;
+        case 2: e = cudaFuncSetAttribute(dslash_staged_kernel<SP, GP, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024); break;
+        case 3: e = cudaFuncSetAttribute(dslash_staged_kernel<SP, GP, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024); break;
         default: return cudaErrorInvalidValue;
         }
-        return cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        attr_set[ny] = true;
     }
+    const dim3 g2 = block_grid(A.g.Vh, block.x, A.nrhs);
+    switch (ny) {
+    case 0: dslash_staged_kernel<SP, GP, 0><<<g2, block, shm, st>>>(A); break;
+    case 1: dslash_staged_kernel<SP, GP, 1><<<g2, block, shm, st>>>(A); break;
+    case 2: dslash_staged_kernel<SP, GP, 2><<<g2, block, shm, st>>>(A); break;
+    case 3: dslash_staged_kernel<SP, GP, 3><<<g2, block, shm, st>>>(A); break;
+    default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -465,38 +461,34 @@ __global__ void __launch_bounds__(TMA_TB, PRE ? 3 : 1) dslash_tma_kernel(DslashA
 template <int SP, int GP, bool PRE>
 cudaError_t launch_tma(const DslashArgs& A, int ny, cudaStream_t st)
 {
-    if constexpr (wide_dev<SP>) {
-        return cudaErrorInvalidValue;
-    } else {
-        constexpr bool NRM = SP == P_F16 || SP == P_BF16;
-        const TmaPlan P = tma_plan(A.g.Lxh, nchunk_dev<SP>(), NRM);
-        if (P.bytes > 200 * 1024) return cudaErrorInvalidValue;
-        static bool attr_set[4] = {false, false, false, false};
-        if (!attr_set[ny]) {
-            cudaError_t e = cudaSuccess;
-            const int lim = 200 * 1024;
-            switch (ny) {
-            case 0: e = cudaFuncSetAttribute(dslash_tma_kernel<SP, GP, 0, PRE>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); break;
-            case 1: e = cudaFuncSetAttribute(dslash_tma_kernel<SP, GP, 1, PRE>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); break;
-            case 2: e = cudaFuncSetAttribute(dslash_tma_kernel<SP, GP, 2, PRE>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); break;
-            case 3: e = cudaFuncSetAttribute(dslash_tma_kernel<SP, GP, 3, PRE>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); break;
-            default: return cudaErrorInvalidValue;
-            }
-            if (e != cudaSuccess) return e;
-            attr_set[ny] = true;
-        }
-        const long long nb = 2LL * ((A.g.Vh + TMA_TB - 1) / TMA_TB) * A.nrhs;
-        if (nb > 0x7fffffffLL) return cudaErrorInvalidValue;
-        const dim3 grid((unsigned)nb);
+    constexpr bool NRM = SP == P_F16 || SP == P_BF16;
+    const TmaPlan P = tma_plan(A.g.Lxh, nchunk_dev<SP>(), NRM);
+    if (P.bytes > 200 * 1024) return cudaErrorInvalidValue;
+    static bool attr_set[4] = {false, false, false, false};
+    if (!attr_set[ny]) {
+        cudaError_t e = cudaSuccess;
+        const int lim = 200 * 1024;
         switch (ny) {
-        case 0: dslash_tma_kernel<SP, GP, 0, PRE><<<grid, TMA_TB, P.bytes, st>>>(A); break;
-        case 1: dslash_tma_kernel<SP, GP, 1, PRE><<<grid, TMA_TB, P.bytes, st>>>(A); break;
-        case 2: dslash_tma_kernel<SP, GP, 2, PRE><<<grid, TMA_TB, P.bytes, st>>>(A); break;
-        case 3: dslash_tma_kernel<SP, GP, 3, PRE><<<grid, TMA_TB, P.bytes, st>>>(A); break;
+        case 0: e = cudaFuncSetAttribute(dslash_tma_kernel<SP, GP, 0, PRE>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); break;
+        case 1: e = cudaFuncSetAttribute(dslash_tma_kernel<SP, GP, 1, PRE>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); break;
+        case 2: e = cudaFuncSetAttribute(dslash_tma_kernel<SP, GP, 2, PRE>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); break;
+        case 3: e = cudaFuncSetAttribute(dslash_tma_kernel<SP, GP, 3, PRE>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); break;
         default: return cudaErrorInvalidValue;
         }
-        return cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        attr_set[ny] = true;
     }
+    const long long nb = 2LL * ((A.g.Vh + TMA_TB - 1) / TMA_TB) * A.nrhs;
+    if (nb > 0x7fffffffLL) return cudaErrorInvalidValue;
+    const dim3 grid((unsigned)nb);
+    switch (ny) {
+    case 0: dslash_tma_kernel<SP, GP, 0, PRE><<<grid, TMA_TB, P.bytes, st>>>(A); break;
+    case 1: dslash_tma_kernel<SP, GP, 1, PRE><<<grid, TMA_TB, P.bytes, st>>>(A); break;
+    case 2: dslash_tma_kernel<SP, GP, 2, PRE><<<grid, TMA_TB, P.bytes, st>>>(A); break;
+    case 3: dslash_tma_kernel<SP, GP, 3, PRE><<<grid, TMA_TB, P.bytes, st>>>(A); break;
+    default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
 }
 
 struct Staged {

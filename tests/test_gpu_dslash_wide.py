@@ -103,3 +103,22 @@ def test_launch_shapes(prec, dims, shape):
     got = host(out)
     for r in range(4):
         assert rel(got[r], oracle.dslash(dims, ABC, U, -RHO, psi[r])) <= TOL[prec]
+
+
+@pytest.mark.parametrize("nrhs", [3, 12])
+@pytest.mark.parametrize("prec", ["f64", "df64"])
+def test_autotuner_candidates(prec, nrhs):
+    """Every candidate the autotuner times for several right-hand sides is a launch the library takes."""
+    from paper_1106_4964_gb300 import Context
+
+    U = synth.gauge_field(DIMS, 5, 0.5)
+    psi = synth.gaussian_spinor(DIMS, 6, nrhs=nrhs)
+    ctx = Context(DIMS, ABC)
+    ctx.set_gauge(dev(U))
+    shape = ctx.tune_dslash(prec, nrhs)
+    ctx.set_dslash_shape(prec, nrhs, *shape)
+    out = torch.empty_like(dev(psi))
+    ctx.apply_dslash(dev(psi), out, -RHO, prec=prec)
+    got = host(out)
+    for r in range(nrhs):
+        assert rel(got[r], oracle.dslash(DIMS, ABC, U, -RHO, psi[r])) <= TOL[prec]
