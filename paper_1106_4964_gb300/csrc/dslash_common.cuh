@@ -179,13 +179,13 @@ __device__ __forceinline__ void hop(const DslashArgs& A, const char* in_q, const
     if constexpr (SP == P_F16 || SP == P_BF16) {
         // 16-bit storage: project the unscaled values and apply the site's scale (and the boundary
         // phase) to the 12 projected reals instead of the 24 loaded ones
-        float n = load_spinor_unscaled<SP>(in_q, inn_q, A.g.Vh, sn, v);
+        float n = load_spinor_unscaled<SP, false>(in_q, inn_q, A.g.Vh, sn, v);
         project<MU, S, Real>(v, h);
         if (cross) n *= A.g.fbc[MU];
 #pragma unroll
         for (int i = 0; i < 12; ++i) h[i] *= n;
     } else {
-        load_spinor<SP, Real>(in_q, inn_q, A.g.Vh, sn, v);
+        load_spinor<SP, Real, false>(in_q, inn_q, A.g.Vh, sn, v);
         project<MU, S, Real>(v, h);
         // a phase of 1 is skipped for the whole launch: nearly every warp holds boundary sites of the x rows
         if (A.g.fbc[MU] != 1.f && cross) {
@@ -217,7 +217,8 @@ struct Bounds {
 };
 
 // Programmatic dependent launch: a kernel lets its successor's blocks start as soon as all of its own have
-// started, and waits for its predecessor to complete before it touches memory, so that inside a captured
+// started, and waits for its predecessor to complete before it touches memory (fields by ordinary loads, see
+// ld_field; only the links, which no launch of a graph writes, by read-only ones), so that inside a captured
 // graph the launch and the index arithmetic of one launch run under the tail of the one before (FP64 overlap
 // at 4^4, 201 launches: 1307 -> 1191 us; 12-source CG at 8^4 361 -> 347 ms; nothing at 16^3 x 32 and above).
 __device__ __forceinline__ void pdl_begin()
@@ -307,7 +308,7 @@ __device__ __forceinline__ void epilogue(const DslashArgs& A, int r, int p, int 
     Real o[24];
     {
         Real self[24];
-        load_spinor<SP, Real>(A.in + off, A.in_n ? A.in_n + noff : nullptr, g.Vh, s, self);
+        load_spinor<SP, Real, false>(A.in + off, A.in_n ? A.in_n + noff : nullptr, g.Vh, s, self);
         const Real a = coef<Real>(A.a, A.fa), b = coef<Real>(A.b, A.fb);
 #pragma unroll
         for (int i = 0; i < 24; ++i) o[i] = a * self[i] + b * acc[i];
@@ -319,7 +320,7 @@ __device__ __forceinline__ void epilogue(const DslashArgs& A, int r, int p, int 
 #pragma unroll
     for (int j = 0; j < NY; ++j) {
         Real w[24];
-        load_spinor<SP, Real>(A.y[j] + off, A.y_n[j] ? A.y_n[j] + noff : nullptr, g.Vh, s, w);
+        load_spinor<SP, Real, false>(A.y[j] + off, A.y_n[j] ? A.y_n[j] + noff : nullptr, g.Vh, s, w);
         const Real sj = coef<Real>(A.sy[j], A.fsy[j]);
 #pragma unroll
         for (int i = 0; i < 24; ++i) o[i] += sj * w[i];

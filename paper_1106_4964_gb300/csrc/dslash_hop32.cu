@@ -43,9 +43,9 @@ __global__ void __launch_bounds__(HOP_THREADS) dslash_hop_kernel(const __grid_co
         float v[24], h[12], u[18], chi[12];
         float ph = cross ? A.g.fbc[w >> 1] : 1.f;
         if constexpr (H16)
-            ph *= load_spinor_unscaled<SP>(in_q, inn_q, g.Vh, sn, v);
+            ph *= load_spinor_unscaled<SP, false>(in_q, inn_q, g.Vh, sn, v);
         else
-            load_spinor<SP, float>(in_q, inn_q, g.Vh, sn, v);
+            load_spinor<SP, float, false>(in_q, inn_q, g.Vh, sn, v);
         const bool fwd = (w & 1) == 0;
         load_link<GP, float>(A.gauge + (size_t)((fwd ? p : q) * 4 + (w >> 1)) * g.Vh * gauge_link_bytes_dev<GP>(), g.Vh,
                              fwd ? s : sn, u);
@@ -81,15 +81,15 @@ __global__ void __launch_bounds__(HOP_THREADS) dslash_hop_kernel(const __grid_co
         }
         auto field4 = [&](const char* base, const float* nrm, float x[4]) {
             if constexpr (H16) {
-                const uint2 t = __ldg(reinterpret_cast<const uint2*>(base + off) + 2 * ((size_t)(w >> 1) * g.Vh + s) + (w & 1));
-                const float n = __ldg(nrm + noff + s);
+                const uint2 t = ld_field<false>(reinterpret_cast<const uint2*>(base + off) + 2 * ((size_t)(w >> 1) * g.Vh + s) + (w & 1));
+                const float n = ld_field<false>(nrm + noff + s);
                 const float2 a = Half<SP>::to2(t.x), b = Half<SP>::to2(t.y);
                 x[0] = a.x * n;
                 x[1] = a.y * n;
                 x[2] = b.x * n;
                 x[3] = b.y * n;
             } else {
-                const float4 t = __ldg(reinterpret_cast<const float4*>(base + off) + (size_t)w * g.Vh + s);
+                const float4 t = ld_field<false>(reinterpret_cast<const float4*>(base + off) + (size_t)w * g.Vh + s);
                 x[0] = t.x;
                 x[1] = t.y;
                 x[2] = t.z;

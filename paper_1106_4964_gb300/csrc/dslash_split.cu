@@ -92,7 +92,7 @@ __device__ __forceinline__ void load_half(const DslashArgs& A, const char* in_q,
 {
     using Real = real_t<SP>;
     Real v[24];
-    load_spinor<SP, Real>(in_q, nullptr, A.g.Vh, sn, v);
+    load_spinor<SP, Real, false>(in_q, nullptr, A.g.Vh, sn, v);
     project_hop<Real>(w, v, h);
     if (cross && A.g.fbc[w >> 1] != 1.f) {
         const Real f = (Real)A.g.bc[w >> 1];
@@ -242,12 +242,12 @@ __global__ void __launch_bounds__(SPLIT_THREADS, MINB) dslash_split_kernel(const
                 const Real a = W::flip(W::coef(A.a, A.da), low && (A.g5_core ^ A.g5_out));
                 const Real b = W::flip(W::coef(A.b, A.db), low && (A.g5_core ^ A.g5_out));
                 Real xr, xi;
-                W::get(__ldg(reinterpret_cast<const int4*>(A.in + off)), xr, xi);
+                W::get(ld_field<false>(reinterpret_cast<const int4*>(A.in + off)), xr, xi);
                 Real o0 = a * xr + b * re, o1 = a * xi + b * im;
 #pragma unroll
                 for (int j = 0; j < NY; ++j) {
                     const Real sj = W::flip(W::coef(A.sy[j], A.dsy[j]), low && A.g5_out);
-                    W::get(__ldg(reinterpret_cast<const int4*>(A.y[j] + off)), xr, xi);
+                    W::get(ld_field<false>(reinterpret_cast<const int4*>(A.y[j] + off)), xr, xi);
                     o0 += sj * xr;
                     o1 += sj * xi;
                 }

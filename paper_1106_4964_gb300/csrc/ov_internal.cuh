@@ -325,15 +325,26 @@ __device__ __forceinline__ double to_f64(R x)
         return f32_to_f64(x.hi) + f32_to_f64(x.lo);
 }
 
-template <int P, typename Real>
-__device__ __forceinline__ void load_spinor(const char* __restrict__ base, const float* __restrict__ nrm,
-                                            int Vh, int s, Real v[24])
+// RO: the field is written by no kernel that may run beside this one, and is read through the read-only path
+// (ld.global.nc).  A kernel that starts before its predecessor has ended (programmatic launches) reads what
+// that one writes: its loads are ordinary ones, which stay behind griddepcontrol.wait.
+template <bool RO, typename T>
+__device__ __forceinline__ T ld_field(const T* p)
+{
+    if constexpr (RO)
+        return __ldg(p);
+    else
+        return *p;
+}
+
+template <int P, typename Real, bool RO = true>
+__device__ __forceinline__ void load_spinor(const char* base, const float* nrm, int Vh, int s, Real v[24])
 {
     if constexpr (P == P_DF64) {
         const float4* b = reinterpret_cast<const float4*>(base);
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
-            float4 t = __ldg(b + (size_t)k * Vh + s);
+            float4 t = ld_field<RO>(b + (size_t)k * Vh + s);
             v[2 * k] = from_df<Real>(df64(t.x, t.y));
             v[2 * k + 1] = from_df<Real>(df64(t.z, t.w));
         }
@@ -341,7 +352,7 @@ __device__ __forceinline__ void load_spinor(const char* __restrict__ base, const
         const double2* b = reinterpret_cast<const double2*>(base);
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
-            double2 t = __ldg(b + (size_t)k * Vh + s);
+            double2 t = ld_field<RO>(b + (size_t)k * Vh + s);
             v[2 * k] = (Real)t.x;
             v[2 * k + 1] = (Real)t.y;
         }
@@ -349,7 +360,7 @@ __device__ __forceinline__ void load_spinor(const char* __restrict__ base, const
         const float4* b = reinterpret_cast<const float4*>(base);
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            float4 t = __ldg(b + (size_t)k * Vh + s);
+            float4 t = ld_field<RO>(b + (size_t)k * Vh + s);
             v[4 * k] = t.x;
             v[4 * k + 1] = t.y;
             v[4 * k + 2] = t.z;
@@ -357,10 +368,10 @@ __device__ __forceinline__ void load_spinor(const char* __restrict__ base, const
         }
     } else {
         const uint4* b = reinterpret_cast<const uint4*>(base);
-        float n = __ldg(nrm + s);
+        float n = ld_field<RO>(nrm + s);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            uint4 t = __ldg(b + (size_t)k * Vh + s);
+            uint4 t = ld_field<RO>(b + (size_t)k * Vh + s);
             float2 a0 = Half<P>::to2(t.x), a1 = Half<P>::to2(t.y), a2 = Half<P>::to2(t.z),
                    a3 = Half<P>::to2(t.w);
             v[8 * k + 0] = a0.x * n;
@@ -376,14 +387,13 @@ __device__ __forceinline__ void load_spinor(const char* __restrict__ base, const
 }
 
 // 16-bit storage: the 24 stored values without their site scale, which is returned
-template <int P>
-__device__ __forceinline__ float load_spinor_unscaled(const char* __restrict__ base, const float* __restrict__ nrm,
-                                                      int Vh, int s, float v[24])
+template <int P, bool RO = true>
+__device__ __forceinline__ float load_spinor_unscaled(const char* base, const float* nrm, int Vh, int s, float v[24])
 {
     const uint4* b = reinterpret_cast<const uint4*>(base);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        uint4 t = __ldg(b + (size_t)k * Vh + s);
+        uint4 t = ld_field<RO>(b + (size_t)k * Vh + s);
         const float2 a0 = Half<P>::to2(t.x), a1 = Half<P>::to2(t.y), a2 = Half<P>::to2(t.z), a3 = Half<P>::to2(t.w);
         v[8 * k + 0] = a0.x;
         v[8 * k + 1] = a0.y;
@@ -394,7 +404,7 @@ __device__ __forceinline__ float load_spinor_unscaled(const char* __restrict__ b
         v[8 * k + 6] = a3.x;
         v[8 * k + 7] = a3.y;
     }
-    return __ldg(nrm + s);
+    return ld_field<RO>(nrm + s);
 }
 
 // eight 16-bit values x[0..7] * inv
