@@ -22,6 +22,28 @@ int set_err(ov_ctx* c, int code, const char* fmt, ...)
     return code;
 }
 
+// st is being captured into a graph of the caller
+static bool capturing(cudaStream_t st)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    return st != nullptr && (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone);
+}
+
+int CallScope::finish(int s)
+{
+    if (done_) return s;
+    done_ = true;
+    if (c_->staged) {
+        c_->staged = false;
+        // (a captured import runs, and reads its host buffer, when the caller's graph does)
+        if (!capturing(st_)) {
+            const cudaError_t e = cudaStreamSynchronize(st_);
+            if (e != cudaSuccess && s == OV_OK) s = set_err(c_, OV_ECUDA, "waiting for a host buffer: %s", cudaGetErrorString(e));
+        }
+    }
+    return s;
+}
+
 int dev_alloc(ov_ctx* c, void** p, size_t bytes)
 {
     *p = nullptr;
@@ -151,6 +173,7 @@ int stage_in(ov_ctx* c, int which, const void* src, size_t bytes, cudaStream_t s
         return OV_OK;
     }
     OV_TRY(ensure_stage(c, which, bytes));
+    c->staged = true;
     OV_CUDA(c, cudaMemcpyAsync(c->stage[which], src, bytes, cudaMemcpyHostToDevice, st));
     *dev = (const double*)c->stage[which];
     return OV_OK;
@@ -523,9 +546,7 @@ static int with_graph(ov_ctx* c, int kind, const FieldDesc& in, const FieldDesc&
 {
     // the rational sign is a host-driven iteration (convergence tests between launches): never captured
     if (!c->use_graphs || c->sign_backend == 1) return body(st);
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (st != nullptr && (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone))
-        return body(st);  // the caller is capturing: record the launches into its graph
+    if (capturing(st)) return body(st);  // the caller is capturing: record the launches into its graph
     cudaStream_t gs = st;
     if (st == nullptr) {
         if (!c->gstream) {
@@ -894,6 +915,7 @@ int ov_set_gauge(ov_ctx* c, const void* U, void* stream)
 {
     if (!c || !U) return c ? set_err(c, OV_EINVAL, "set_gauge: null pointer") : OV_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
+    CallScope call(c, st);
     const size_t bytes = (size_t)2 * c->g.Vh * 4 * 9 * 16;
     const double* dU = nullptr;
     OV_TRY(stage_in(c, 0, U, bytes, st, &dU));
@@ -933,6 +955,7 @@ static int apply_canonical(ov_ctx* c, const void* in, void* out, double m, int n
     if (nrhs < 1 || nrhs > 16) return set_err(c, OV_EINVAL, "nrhs = %d out of range 1..16", nrhs);
     if (!c->have_gauge) return set_err(c, OV_ESTATE, "no gauge field (call ov_set_gauge)");
     cudaStream_t st = (cudaStream_t)stream;
+    CallScope call(c, st);
     const size_t bytes = (size_t)nrhs * 2 * c->g.Vh * 12 * 16;
     const double* din = nullptr;
     double* dout = nullptr;
@@ -954,7 +977,7 @@ static int apply_canonical(ov_ctx* c, const void* in, void* out, double m, int n
     }
     OV_CUDA(c, launch_unpack(c->g, fo, dout, st));
     OV_TRY(stage_out_finish(c, out, dout, bytes, st));
-    return check_kernel_flags(c, st);
+    return call.finish(check_kernel_flags(c, st));
 }
 
 int ov_apply_dslash(ov_ctx* c, const void* in, void* out, double m, int nrhs, int prec, void* stream)
@@ -1059,6 +1082,7 @@ int ov_set_eigenpairs(ov_ctx* c, int which, int nev, const double* vals, const v
     if (nev < 0 || nev > 2048) return set_err(c, OV_EINVAL, "nev = %d out of range 0..2048", nev);
     if (nev > 0 && (!vals || !vecs)) return set_err(c, OV_EINVAL, "null eigenpair buffers");
     cudaStream_t st = (cudaStream_t)stream;
+    CallScope call(c, st);
     EigSet& E = c->eig[which];
     OV_CUDA(c, cudaStreamSynchronize(st));
     graphs_clear(c);
@@ -1137,6 +1161,7 @@ int ov_cg_solve(ov_ctx* c, const void* b, void* x, int nrhs, double mass, double
     OV_TRY(check_prec(c, inner_prec));
     if (!c->have_gauge || !c->have_poly) return set_err(c, OV_ESTATE, "cg: needs gauge field and sign polynomial");
     cudaStream_t st = (cudaStream_t)stream;
+    CallScope call(c, st);
     const size_t bytes = (size_t)nrhs * 2 * c->g.Vh * 12 * 16;
     const double* db = nullptr;
     double* dx = nullptr;
@@ -1150,7 +1175,7 @@ int ov_cg_solve(ov_ctx* c, const void* b, void* x, int nrhs, double mass, double
     if (s != OV_OK && s != OV_ENOTCONV && s != OV_ESTALL) return s;
     OV_CUDA(c, launch_unpack(c->g, fx, dx, st));
     OV_TRY(stage_out_finish(c, x, dx, bytes, st));
-    return s;
+    return call.finish(s);
 }
 
 int ov_cg_solve_multimass(ov_ctx* c, const void* b, void* x, int nrhs, int nmass, const double* masses, double tol,
@@ -1167,6 +1192,7 @@ int ov_cg_solve_multimass(ov_ctx* c, const void* b, void* x, int nrhs, int nmass
     OV_TRY(check_prec(c, inner_prec));
     if (!c->have_gauge || !c->have_poly) return set_err(c, OV_ESTATE, "multimass: needs gauge field and sign polynomial");
     cudaStream_t st = (cudaStream_t)stream;
+    CallScope call(c, st);
     const size_t one = (size_t)nrhs * 2 * c->g.Vh * 12 * 16;
     const double* db = nullptr;
     OV_TRY(stage_in(c, 0, b, one, st, &db));
@@ -1226,11 +1252,12 @@ int ov_field_import(ov_ctx* c, ov_field* f, const void* canonical, void* stream)
 {
     if (!c || !f || !canonical) return c ? set_err(c, OV_EINVAL, "null pointer") : OV_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
+    CallScope call(c, st);
     const size_t bytes = (size_t)f->d.nrhs * 2 * c->g.Vh * 12 * 16;
     const double* src = nullptr;
     OV_TRY(stage_in(c, 0, canonical, bytes, st, &src));
     OV_CUDA(c, launch_pack(c->g, src, f->d, st));
-    return OV_OK;
+    return call.finish(OV_OK);
 }
 
 int ov_field_export(ov_ctx* c, const ov_field* f, void* canonical, void* stream)

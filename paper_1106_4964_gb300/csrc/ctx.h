@@ -88,6 +88,7 @@ struct ov_ctx {
     double* dscal = nullptr;  // device scalar scratch, DSCAL_DOUBLES doubles
     void* stage[2] = {nullptr, nullptr};
     size_t stage_bytes[2] = {0, 0};
+    bool staged = false;  // the call in progress copies from a host buffer of the caller (CallScope)
     unsigned* derr = nullptr;
 
     std::map<std::pair<int, int>, std::tuple<int, int, int>> shape;  // (prec, nrhs) -> (bx, by, variant)
@@ -152,6 +153,22 @@ int set_err(ov_ctx* c, int code, const char* fmt, ...);
         int s_ = (x);             \
         if (s_ != OV_OK) return s_; \
     } while (0)
+
+// One call of the C ABI that works on stream st.  A call that copied from a host buffer waits for st before
+// it returns, on every path out: the caller may reuse a pinned buffer at once.
+class CallScope {
+public:
+    CallScope(ov_ctx* c, cudaStream_t st) : c_(c), st_(st) {}
+    ~CallScope() { finish(OV_OK); }
+    CallScope(const CallScope&) = delete;
+    // s, or the error of the wait
+    int finish(int s);
+
+private:
+    ov_ctx* c_;
+    cudaStream_t st_;
+    bool done_ = false;
+};
 
 int dev_alloc(ov_ctx* c, void** p, size_t bytes);
 void graphs_clear(ov_ctx* c);

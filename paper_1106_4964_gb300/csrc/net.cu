@@ -662,6 +662,7 @@ int ov_net_apply(ov_ctx* c, const void* in, void* out, int nrhs, void* stream)
     if (!c->have_gauge) return set_err(c, OV_ESTATE, "no gauge field");
     if (!c->net) return set_err(c, OV_ESTATE, "no network weights");
     cudaStream_t st = (cudaStream_t)stream;
+    CallScope call(c, st);
     const size_t bytes = (size_t)nrhs * 2 * c->g.Vh * 12 * 16;
     const double* din = nullptr;
     double* dout = nullptr;
@@ -673,7 +674,7 @@ int ov_net_apply(ov_ctx* c, const void* in, void* out, int nrhs, void* stream)
     OV_CUDA(c, launch_pack(c->g, din, fi, st));
     OV_TRY(net_apply_precond(c, fi, fo, st));
     OV_CUDA(c, launch_unpack(c->g, fo, dout, st));
-    return stage_out_finish(c, out, dout, bytes, st);
+    return call.finish(stage_out_finish(c, out, dout, bytes, st));
 }
 
 int ov_net_loss_grad(ov_ctx* c, const void* r, const void* e, int npairs, double* loss, double* grad, void* stream)
@@ -683,6 +684,7 @@ int ov_net_loss_grad(ov_ctx* c, const void* r, const void* e, int npairs, double
     if (!c->have_gauge) return set_err(c, OV_ESTATE, "no gauge field");
     if (!c->net) return set_err(c, OV_ESTATE, "no network weights");
     cudaStream_t st = (cudaStream_t)stream;
+    CallScope call(c, st);
     const size_t bytes = (size_t)npairs * 2 * c->g.Vh * 12 * 16;
     const double *dr = nullptr, *de = nullptr;
     FieldDesc fr, fe;
