@@ -28,7 +28,13 @@
  *    buffers are staged through library-owned device memory and the call
  *    synchronises `stream` before returning.  Device buffers are used in
  *    place and the call is stream-ordered on `stream` (a cudaStream_t passed
- *    as void*; NULL = the legacy default stream).  The caller owns every
+ *    as void*; NULL = the legacy default stream).  The calls of one context
+ *    take turns in the order in which they were made, whatever their streams:
+ *    a call on another stream waits on the device for the one before.
+ *    (ov_dslash_field, ov_field_import and ov_field_export use no shared
+ *    buffer and are ordered by their stream alone; launches that the caller
+ *    captured into its own graph are the caller's to order.)  One host thread
+ *    at a time uses a context.  The caller owns every
  *    buffer it passes; the library owns the packed gauge field, the
  *    eigenpairs, all workspaces and the network weights.
  *  - Every call returns OV_OK (0) or a negative ov_status; on error no

@@ -29,18 +29,36 @@ static bool capturing(cudaStream_t st)
     return st != nullptr && (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone);
 }
 
+int CallScope::begin()
+{
+    if (capturing(st_)) return OV_OK;
+    OV_CUDA(c_, cudaStreamGetId(st_, &id_));
+    if (!c_->order_ev) OV_CUDA(c_, cudaEventCreateWithFlags(&c_->order_ev, cudaEventDisableTiming));
+    if (c_->order_set && c_->order_id != id_) OV_CUDA(c_, cudaStreamWaitEvent(st_, c_->order_ev, 0));
+    ordered_ = true;
+    return OV_OK;
+}
+
 int CallScope::finish(int s)
 {
     if (done_) return s;
     done_ = true;
+    cudaError_t e = cudaSuccess;
+    if (ordered_) {
+        e = cudaEventRecord(c_->order_ev, st_);
+        c_->order_id = id_;
+        c_->order_set = e == cudaSuccess;
+        if (e != cudaSuccess) cudaStreamSynchronize(st_);  // no event to wait for: nothing left in flight
+    }
     if (c_->staged) {
         c_->staged = false;
         // (a captured import runs, and reads its host buffer, when the caller's graph does)
         if (!capturing(st_)) {
-            const cudaError_t e = cudaStreamSynchronize(st_);
-            if (e != cudaSuccess && s == OV_OK) s = set_err(c_, OV_ECUDA, "waiting for a host buffer: %s", cudaGetErrorString(e));
+            const cudaError_t w = cudaStreamSynchronize(st_);
+            if (e == cudaSuccess) e = w;
         }
     }
+    if (e != cudaSuccess && s == OV_OK) s = set_err(c_, OV_ECUDA, "end of call: %s", cudaGetErrorString(e));
     return s;
 }
 
@@ -901,6 +919,7 @@ int ov_destroy(ov_ctx* c)
     if (c->gstream) cudaStreamDestroy(c->gstream);
     for (auto& e : c->gev)
         if (e) cudaEventDestroy(e);
+    if (c->order_ev) cudaEventDestroy(c->order_ev);
     delete c;
     return OV_OK;
 }
@@ -916,8 +935,10 @@ int ov_set_gauge(ov_ctx* c, const void* U, void* stream)
     if (!c || !U) return c ? set_err(c, OV_EINVAL, "set_gauge: null pointer") : OV_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
     CallScope call(c, st);
+    OV_TRY(call.begin());
     const size_t bytes = (size_t)2 * c->g.Vh * 4 * 9 * 16;
     const double* dU = nullptr;
+    if (c->gauge[0]) OV_CUDA(c, cudaDeviceSynchronize());  // ov_dslash_field launches, on any stream, read the links
     OV_TRY(stage_in(c, 0, U, bytes, st, &dU));
     for (int p = 0; p < NPREC; ++p) {
         if (!c->gauge[p] && p != P_DF64) OV_TRY(dev_alloc(c, &c->gauge[p], (size_t)8 * c->g.Vh * gauge_link_bytes(p)));
@@ -943,7 +964,7 @@ int ov_set_gauge(ov_ctx* c, const void* U, void* stream)
     graphs_clear(c);
     // eigenpairs of a previous gauge field no longer apply
     for (auto& e : c->eig) eig_clear(c, e);
-    return OV_OK;
+    return call.finish(OV_OK);
 }
 
 static int apply_canonical(ov_ctx* c, const void* in, void* out, double m, int nrhs, int prec, void* stream, int kind)
@@ -956,6 +977,7 @@ static int apply_canonical(ov_ctx* c, const void* in, void* out, double m, int n
     if (!c->have_gauge) return set_err(c, OV_ESTATE, "no gauge field (call ov_set_gauge)");
     cudaStream_t st = (cudaStream_t)stream;
     CallScope call(c, st);
+    OV_TRY(call.begin());
     const size_t bytes = (size_t)nrhs * 2 * c->g.Vh * 12 * 16;
     const double* din = nullptr;
     double* dout = nullptr;
@@ -1023,6 +1045,8 @@ int ov_set_sign_poly(ov_ctx* c, double rho, double eps, int degree, double lambd
     } else {
         if (!c->have_gauge) return set_err(c, OV_ESTATE, "lambda_max estimate needs the gauge field");
         double l = 0;
+        CallScope call(c, (cudaStream_t)0);
+        OV_TRY(call.begin());
         OV_TRY(estimate_lambda_max(c, 50, &l, (cudaStream_t)0));
         c->lmax = 1.01 * l;
     }
@@ -1039,6 +1063,8 @@ int ov_set_sign_rational(ov_ctx* c, double rho, double eps, int npoles, double l
     double l = lambda_max;
     if (!(l > 0)) {
         if (!c->have_gauge) return set_err(c, OV_ESTATE, "lambda_max estimate needs the gauge field");
+        CallScope call(c, (cudaStream_t)0);
+        OV_TRY(call.begin());
         OV_TRY(estimate_lambda_max(c, 50, &l, (cudaStream_t)0));
         l *= 1.01;
     }
@@ -1083,6 +1109,7 @@ int ov_set_eigenpairs(ov_ctx* c, int which, int nev, const double* vals, const v
     if (nev > 0 && (!vals || !vecs)) return set_err(c, OV_EINVAL, "null eigenpair buffers");
     cudaStream_t st = (cudaStream_t)stream;
     CallScope call(c, st);
+    OV_TRY(call.begin());
     EigSet& E = c->eig[which];
     OV_CUDA(c, cudaStreamSynchronize(st));
     graphs_clear(c);
@@ -1122,6 +1149,8 @@ int ov_get_eigenpairs(ov_ctx* c, int which, int* nev, double* vals, void* vecs, 
     if (vals)
         for (int i = 0; i < E.nev; ++i) vals[i] = E.vals[i];
     if (vecs && E.nev) {
+        CallScope call(c, st);
+        OV_TRY(call.begin());
         const size_t one = (size_t)2 * c->g.Vh * 12 * 16;
         for (int i0 = 0; i0 < E.nev; i0 += 16) {
             int n = E.nev - i0 < 16 ? E.nev - i0 : 16;
@@ -1147,7 +1176,9 @@ int ov_deflate(ov_ctx* c, int which, int nev, double tol, void* stream)
     if (!(tol > 0)) return set_err(c, OV_EINVAL, "tol must be positive");
     if (!c->have_gauge) return set_err(c, OV_ESTATE, "deflate: no gauge field");
     if (which == 1 && !c->have_poly) return set_err(c, OV_ESTATE, "deflate(which=1): no sign polynomial");
-    return deflate_impl(c, which, nev, tol, (cudaStream_t)stream);
+    CallScope call(c, (cudaStream_t)stream);
+    OV_TRY(call.begin());
+    return call.finish(deflate_impl(c, which, nev, tol, (cudaStream_t)stream));
 }
 
 int ov_cg_solve(ov_ctx* c, const void* b, void* x, int nrhs, double mass, double tol, int max_iter, int precond,
@@ -1162,6 +1193,7 @@ int ov_cg_solve(ov_ctx* c, const void* b, void* x, int nrhs, double mass, double
     if (!c->have_gauge || !c->have_poly) return set_err(c, OV_ESTATE, "cg: needs gauge field and sign polynomial");
     cudaStream_t st = (cudaStream_t)stream;
     CallScope call(c, st);
+    OV_TRY(call.begin());
     const size_t bytes = (size_t)nrhs * 2 * c->g.Vh * 12 * 16;
     const double* db = nullptr;
     double* dx = nullptr;
@@ -1193,6 +1225,7 @@ int ov_cg_solve_multimass(ov_ctx* c, const void* b, void* x, int nrhs, int nmass
     if (!c->have_gauge || !c->have_poly) return set_err(c, OV_ESTATE, "multimass: needs gauge field and sign polynomial");
     cudaStream_t st = (cudaStream_t)stream;
     CallScope call(c, st);
+    OV_TRY(call.begin());
     const size_t one = (size_t)nrhs * 2 * c->g.Vh * 12 * 16;
     const double* db = nullptr;
     OV_TRY(stage_in(c, 0, b, one, st, &db));
@@ -1288,7 +1321,9 @@ int ov_overlap_field(ov_ctx* c, const ov_field* in, ov_field* out, double mass, 
     if (in == out) return set_err(c, OV_EINVAL, "in and out must differ");
     if (in->d.prec != out->d.prec || in->d.nrhs != out->d.nrhs)
         return set_err(c, OV_EINVAL, "fields differ in precision or nrhs");
-    return overlap_apply(c, in->d, out->d, mass, (cudaStream_t)stream);
+    CallScope call(c, (cudaStream_t)stream);
+    OV_TRY(call.begin());
+    return call.finish(overlap_apply(c, in->d, out->d, mass, (cudaStream_t)stream));
 }
 
 int ov_field_dot(ov_ctx* c, const ov_field* x, const ov_field* y, double* out, void* stream)
@@ -1297,6 +1332,8 @@ int ov_field_dot(ov_ctx* c, const ov_field* x, const ov_field* y, double* out, v
     if (x->d.prec != y->d.prec || x->d.nrhs != y->d.nrhs)
         return set_err(c, OV_EINVAL, "fields differ in precision or nrhs");
     cudaStream_t st = (cudaStream_t)stream;
+    CallScope call(c, st);
+    OV_TRY(call.begin());
     double* dev = nullptr;
     if (is_device_ptr(out)) {
         dev = out;
@@ -1309,7 +1346,7 @@ int ov_field_dot(ov_ctx* c, const ov_field* x, const ov_field* y, double* out, v
         OV_CUDA(c, cudaMemcpyAsync(out, dev, sizeof(double) * 2 * x->d.nrhs, cudaMemcpyDeviceToHost, st));
         OV_CUDA(c, cudaStreamSynchronize(st));
     }
-    return OV_OK;
+    return call.finish(OV_OK);
 }
 
 int ov_project_lowmodes(ov_ctx* c, int which, const ov_field* psi, int engine, double* out, void* stream)
@@ -1319,6 +1356,8 @@ int ov_project_lowmodes(ov_ctx* c, int which, const ov_field* psi, int engine, d
     EigSet& E = c->eig[which];
     if (!E.nev) return set_err(c, OV_ESTATE, "no eigenpairs stored (which=%d)", which);
     cudaStream_t st = (cudaStream_t)stream;
+    CallScope call(c, st);
+    OV_TRY(call.begin());
     const int R = psi->d.nrhs;
     const size_t ncoef = (size_t)E.nev * R;
     if (ncoef * 2 > (size_t)DSCAL_COEF) return set_err(c, OV_EINVAL, "nev * nrhs = %zu too large", ncoef);
@@ -1356,6 +1395,8 @@ int ov_lowmode_update(ov_ctx* c, int which, const ov_field* psi, const double* c
             return set_err(c, OV_EINVAL, "fields differ in precision or nrhs");
     if (out1 == psi || out2 == psi || out1 == out2) return set_err(c, OV_EINVAL, "fields must differ");
     cudaStream_t st = (cudaStream_t)stream;
+    CallScope call(c, st);
+    OV_TRY(call.begin());
     const size_t ncoef = (size_t)E.nev * pd.nrhs;
     if (ncoef * 2 > (size_t)DSCAL_COEF) return set_err(c, OV_EINVAL, "nev * nrhs = %zu too large", ncoef);
     double2* dev = (double2*)c->dscal;
@@ -1494,6 +1535,8 @@ int ov_tune_dslash(ov_ctx* c, int prec, int nrhs, int* bx, int* by, int* variant
     if (nrhs < 1 || nrhs > 16) return set_err(c, OV_EINVAL, "nrhs out of range");
     if (!c->have_gauge) return set_err(c, OV_ESTATE, "no gauge field");
     cudaStream_t st = (cudaStream_t)stream;
+    CallScope call(c, st);
+    OV_TRY(call.begin());
     FieldDesc fi, fo;
     OV_TRY(ws_field(c, WS_IN, prec, nrhs, &fi));
     OV_TRY(ws_field(c, WS_OUT, prec, nrhs, &fo));

@@ -88,6 +88,10 @@ struct ov_ctx {
     double* dscal = nullptr;  // device scalar scratch, DSCAL_DOUBLES doubles
     void* stage[2] = {nullptr, nullptr};
     size_t stage_bytes[2] = {0, 0};
+    // end of the last call that used the context's buffers, and the stream it ran on (CallScope)
+    cudaEvent_t order_ev = nullptr;
+    unsigned long long order_id = 0;
+    bool order_set = false;
     bool staged = false;  // the call in progress copies from a host buffer of the caller (CallScope)
     unsigned* derr = nullptr;
 
@@ -154,20 +158,26 @@ int set_err(ov_ctx* c, int code, const char* fmt, ...);
         if (s_ != OV_OK) return s_; \
     } while (0)
 
-// One call of the C ABI that works on stream st.  A call that copied from a host buffer waits for st before
-// it returns, on every path out: the caller may reuse a pinned buffer at once.
+// One call of the C ABI that works on stream st.
+//  - The context's work fields, scalars and buffers are shared by all its calls: begin() makes st wait for the
+//    last call if that ran on another stream (calls on one stream pay only the event's record).  A stream that
+//    the caller is capturing takes no part: the caller orders the replays of its own graph.
+//  - A call that copied from a host buffer waits for st before it returns, on every path out: the caller may
+//    reuse a pinned buffer at once.
 class CallScope {
 public:
     CallScope(ov_ctx* c, cudaStream_t st) : c_(c), st_(st) {}
     ~CallScope() { finish(OV_OK); }
     CallScope(const CallScope&) = delete;
-    // s, or the error of the wait
+    int begin();
+    // s, or the error of the wait or the record
     int finish(int s);
 
 private:
     ov_ctx* c_;
     cudaStream_t st_;
-    bool done_ = false;
+    unsigned long long id_ = 0;  // of the stream: a handle may be that of a destroyed one
+    bool ordered_ = false, done_ = false;
 };
 
 int dev_alloc(ov_ctx* c, void** p, size_t bytes);

@@ -631,6 +631,8 @@ int ov_net_set_weights(ov_ctx* c, const double* w, int n)
 {
     if (!c) return OV_EINVAL;
     if (!w || n != 2 * NET_PARAMS) return set_err(c, OV_EINVAL, "weights: expected %d doubles", 2 * NET_PARAMS);
+    CallScope call(c, (cudaStream_t)0);
+    OV_TRY(call.begin());
     OV_TRY(net_init(c));
     std::vector<float2> h(NET_PARAMS);
     for (int i = 0; i < NET_PARAMS; ++i) h[i] = make_float2((float)w[2 * i], (float)w[2 * i + 1]);
@@ -645,6 +647,8 @@ int ov_net_get_weights(ov_ctx* c, double* w, int n)
     if (!c) return OV_EINVAL;
     if (!w || n != 2 * NET_PARAMS) return set_err(c, OV_EINVAL, "weights: expected %d doubles", 2 * NET_PARAMS);
     if (!c->net) return set_err(c, OV_ESTATE, "no network weights");
+    CallScope call(c, (cudaStream_t)0);
+    OV_TRY(call.begin());
     std::vector<float2> h(NET_PARAMS);
     OV_CUDA(c, cudaMemcpy(h.data(), c->net->W, sizeof(float2) * NET_PARAMS, cudaMemcpyDeviceToHost));
     for (int i = 0; i < NET_PARAMS; ++i) {
@@ -663,6 +667,7 @@ int ov_net_apply(ov_ctx* c, const void* in, void* out, int nrhs, void* stream)
     if (!c->net) return set_err(c, OV_ESTATE, "no network weights");
     cudaStream_t st = (cudaStream_t)stream;
     CallScope call(c, st);
+    OV_TRY(call.begin());
     const size_t bytes = (size_t)nrhs * 2 * c->g.Vh * 12 * 16;
     const double* din = nullptr;
     double* dout = nullptr;
@@ -685,6 +690,7 @@ int ov_net_loss_grad(ov_ctx* c, const void* r, const void* e, int npairs, double
     if (!c->net) return set_err(c, OV_ESTATE, "no network weights");
     cudaStream_t st = (cudaStream_t)stream;
     CallScope call(c, st);
+    OV_TRY(call.begin());
     const size_t bytes = (size_t)npairs * 2 * c->g.Vh * 12 * 16;
     const double *dr = nullptr, *de = nullptr;
     FieldDesc fr, fe;
@@ -713,6 +719,8 @@ int ov_net_train(ov_ctx* c, int nsolves, int steps, double lr, double mass, doub
     if (nsolves < 1 || nsolves > 64 || steps < 0 || !(lr > 0)) return set_err(c, OV_EINVAL, "bad training arguments");
     if (!c->have_gauge || !c->have_poly) return set_err(c, OV_ESTATE, "training needs gauge field and sign polynomial");
     cudaStream_t st = (cudaStream_t)stream;
+    CallScope call(c, st);
+    OV_TRY(call.begin());
     OV_TRY(net_init(c));
     NetState* n = c->net;
     // ---- record (residual, iterate) pairs from deflated mixed-precision CG solves of random sources

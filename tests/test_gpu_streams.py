@@ -1,4 +1,5 @@
-"""Stream behaviour of the calls: a host buffer belongs to its caller again when the call returns."""
+"""Stream behaviour of the calls: a host buffer belongs to its caller again when the call returns, and the
+calls of one context, which share its work fields, take turns across streams."""
 import pytest
 
 import synth
@@ -75,3 +76,58 @@ def test_host_input_may_be_reused(name, busy):
     CALLS[name](ctx, x, out)
     x.zero_()
     assert (host(out) == host(ref)).all()
+
+
+@pytest.mark.parametrize("second", ["null", "other"])
+@pytest.mark.parametrize("name", ["Hw", "overlap", "normal", "net"])
+def test_calls_on_two_streams_take_turns(name, second, busy):
+    """The first call sits behind other work of its stream when the second, on an idle stream, is made."""
+    ctx = make()
+    xs = [dev(synth.gaussian_spinor(DIMS, k, nrhs=2)) for k in range(4)]
+    refs = [torch.empty_like(x) for x in xs]
+    for x, ref in zip(xs, refs):
+        CALLS[name](ctx, x, ref)
+    outs = [torch.zeros_like(x) for x in xs]
+    s1 = torch.cuda.Stream()
+    s2 = torch.cuda.Stream() if second == "other" else torch.cuda.default_stream()
+    for s in (s1, s2):  # each stream's graph exists
+        with torch.cuda.stream(s):
+            CALLS[name](ctx, xs[0], outs[0])
+    outs[0].zero_()
+    torch.cuda.synchronize()
+    for k, s in enumerate((s1, s2, s1, s2)):
+        with torch.cuda.stream(s):
+            if s is s1:
+                busy(1)
+            CALLS[name](ctx, xs[k], outs[k])
+    for ref, out in zip(refs, outs):
+        assert (host(out) == host(ref)).all()
+
+
+def test_set_gauge_waits_for_calls_on_other_streams(busy):
+    ctx = make()
+    x = dev(synth.gaussian_spinor(DIMS, 1, nrhs=2))
+    u2 = dev(synth.gauge_field(DIMS, 9, 0.5))
+    f = [ctx.field(2, "f64") for _ in range(2)]
+    f[0].load(x)
+    outs = [torch.zeros_like(x) for _ in range(2)]
+    refs = [torch.zeros_like(x) for _ in range(2)]
+    s1 = torch.cuda.Stream()
+
+    def go(res):
+        with torch.cuda.stream(s1):
+            ctx.apply_Hw(x, res[0], -RHO, prec="f64")
+            ctx.dslash_field(f[0], f[1], -RHO)
+
+    go(refs)
+    f[1].store(refs[1], stream=s1)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s1):
+        busy()
+    go(outs)
+    ctx.set_gauge(u2, stream=torch.cuda.Stream())
+    f[1].store(outs[1], stream=s1)
+    for ref, out in zip(refs, outs):
+        assert (host(out) == host(ref)).all()
+    for a in f:
+        a.close()
