@@ -153,6 +153,21 @@ def _stream(stream):
     return int(stream)
 
 
+def _lend(stream, *bufs):
+    """Tell torch's allocator that device tensors are used on `stream` when that is not the current one: the calls
+    return before their work is done, and a tensor that its owner drops would be handed out again."""
+    bufs = [b for b in bufs if getattr(b, "is_cuda", False)]
+    if stream is None or not bufs:
+        return
+    import torch
+
+    if _stream(stream) == torch.cuda.current_stream().cuda_stream:
+        return
+    s = stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(_stream(stream))
+    for b in bufs:
+        b.record_stream(s)
+
+
 def _prec(p):
     return PREC[p] if isinstance(p, str) else int(p)
 
@@ -175,9 +190,11 @@ class Field:
         self.h = h
 
     def load(self, x, stream=None):
+        _lend(stream, x)
         self.ctx._check(self.ctx.lib.ov_field_import(self.ctx.h, self.h, _ptr(x), _stream(stream)))
 
     def store(self, x, stream=None):
+        _lend(stream, x)
         self.ctx._check(self.ctx.lib.ov_field_export(self.ctx.h, self.h, _ptr(x), _stream(stream)))
 
     def close(self):
@@ -234,11 +251,13 @@ class Context:
         self._check(self.lib.ov_set_gauge(self.h, _ptr(U), _stream(stream)))
 
     def apply_dslash(self, x, out, m, prec="f64", stream=None):
+        _lend(stream, x, out)
         self._check(self.lib.ov_apply_dslash(self.h, _ptr(x), _ptr(out), float(m), self._nrhs(x), _prec(prec),
                                              _stream(stream)))
         return out
 
     def apply_Hw(self, x, out, m, prec="f64", stream=None):
+        _lend(stream, x, out)
         self._check(self.lib.ov_apply_Hw(self.h, _ptr(x), _ptr(out), float(m), self._nrhs(x), _prec(prec),
                                          _stream(stream)))
         return out
@@ -265,11 +284,13 @@ class Context:
         return b, c, d.value
 
     def apply_overlap(self, x, out, mass=0.0, prec="f64", stream=None):
+        _lend(stream, x, out)
         self._check(self.lib.ov_apply_overlap(self.h, _ptr(x), _ptr(out), float(mass), self._nrhs(x), _prec(prec),
                                               _stream(stream)))
         return out
 
     def apply_normal(self, x, out, mass=0.0, prec="f64", chiral=0, stream=None):
+        _lend(stream, x, out)
         self._check(self.lib.ov_apply_normal(self.h, _ptr(x), _ptr(out), float(mass), self._nrhs(x), _prec(prec),
                                              int(chiral), _stream(stream)))
         return out
@@ -295,6 +316,7 @@ class Context:
     def cg_solve(self, b, x, mass=0.0, tol=1e-10, max_iter=1000, precond=0, inner_prec="f64", stream=None,
                  check=True):
         info = SolveInfo()
+        _lend(stream, b, x)
         st = self.lib.ov_cg_solve(self.h, _ptr(b), _ptr(x), self._nrhs(b), float(mass), float(tol), int(max_iter),
                                   int(precond), _prec(inner_prec), ctypes.byref(info), _stream(stream))
         if check:
@@ -310,6 +332,7 @@ class Context:
         if _nbytes(x) != len(m) * _nbytes(b):
             raise ValueError("x must hold len(masses) x nrhs fields")
         infos = (SolveInfo * len(m))()
+        _lend(stream, b, x)
         st = self.lib.ov_cg_solve_multimass(self.h, _ptr(b), _ptr(x), nrhs, len(m), _ptr(m), float(tol),
                                             int(max_iter), _prec(inner_prec), int(output), infos, _stream(stream))
         if check:
@@ -335,6 +358,7 @@ class Context:
         self._check(self.lib.ov_net_set_weights(self.h, _ptr(w), self.NET_DOUBLES))
 
     def net_apply(self, x, out, stream=None):
+        _lend(stream, x, out)
         self._check(self.lib.ov_net_apply(self.h, _ptr(x), _ptr(out), self._nrhs(x), _stream(stream)))
         return out
 
@@ -390,6 +414,7 @@ class Context:
         """ov_field_dot_noalloc: out is a host numpy array (default) or a device tensor of 2*nrhs doubles."""
         if out is None:
             out = np.empty(2 * x.nrhs)
+        _lend(stream, out)
         st = self.lib.ov_field_dot_noalloc(x.h, y.h, _ptr(out), _stream(stream))
         if st != 0:
             raise OverlapError(st, "ov_field_dot_noalloc failed")

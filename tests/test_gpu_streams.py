@@ -131,3 +131,27 @@ def test_set_gauge_waits_for_calls_on_other_streams(busy):
         assert (host(out) == host(ref)).all()
     for a in f:
         a.close()
+
+
+@pytest.mark.parametrize("name", ["Hw", "net"])
+def test_input_tensor_dropped_after_the_call(name, busy):
+    """A call on a side stream returns before its work has begun; its input's memory is not handed out again to
+    the current stream until that work is done."""
+    ctx = make()
+    psi = synth.gaussian_spinor(DIMS, 1, nrhs=2)
+    ref, out = torch.empty_like(dev(psi)), torch.empty_like(dev(psi))
+    s1 = torch.cuda.Stream()
+    run = {"Hw": lambda x, o: ctx.apply_Hw(x, o, -RHO, prec="f32", stream=s1),
+           "net": lambda x, o: ctx.net_apply(x, o, stream=s1)}[name]
+    run(dev(psi), ref)
+    torch.cuda.synchronize()
+    x = dev(psi)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s1):
+        busy()
+    run(x, out)
+    shape, kind = x.shape, x.dtype
+    del x
+    refill = [torch.zeros(shape, dtype=kind, device="cuda") for _ in range(8)]
+    assert (host(out) == host(ref)).all()
+    del refill
