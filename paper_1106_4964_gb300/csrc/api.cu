@@ -976,6 +976,8 @@ static int apply_canonical(ov_ctx* c, const void* in, void* out, double m, int n
     if (nrhs < 1 || nrhs > 16) return set_err(c, OV_EINVAL, "nrhs = %d out of range 1..16", nrhs);
     if (!c->have_gauge) return set_err(c, OV_ESTATE, "no gauge field (call ov_set_gauge)");
     cudaStream_t st = (cudaStream_t)stream;
+    // a replay of the caller's graph would use the context's fields without taking its turn
+    if (capturing(st)) return set_err(c, OV_ECUDA, "not on a stream that is being captured (use fields)");
     CallScope call(c, st);
     OV_TRY(call.begin());
     const size_t bytes = (size_t)nrhs * 2 * c->g.Vh * 12 * 16;

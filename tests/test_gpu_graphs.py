@@ -142,3 +142,30 @@ def test_many_replays_equal_the_eager_result(cfg1, prec):
     assert int(bad) == 0 and ctx.graph_stats()[1] == 199
     fi.close()
     fo.close()
+
+
+def test_canonical_calls_are_refused_under_capture(cfg1):
+    """They share the context's fields with every other call: a capturing stream gets OV_ECUDA, nothing is
+    recorded, the capture stays valid and the context works."""
+    from paper_1106_4964_gb300 import OverlapError
+
+    psi = dev(synth.gaussian_spinor(cfg1["dims"], 15))
+    ctx = make_ctx(cfg1)
+    out, ref = torch.empty_like(psi), torch.empty_like(psi)
+    calls = [lambda o: ctx.apply_dslash(psi, o, -RHO), lambda o: ctx.apply_Hw(psi, o, -RHO),
+             lambda o: ctx.apply_overlap(psi, o, 0.1), lambda o: ctx.apply_normal(psi, o, 0.1)]
+    for call in calls:
+        call(ref)
+        g, mark = torch.cuda.CUDAGraph(), torch.zeros(1, device="cuda")
+        torch.cuda.synchronize()
+        with torch.cuda.graph(g):
+            mark += 1
+            with pytest.raises(OverlapError) as e:
+                call(out)
+        assert e.value.status == -3  # OV_ECUDA
+        out.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert float(mark) == 1 and not host(out).any()
+        call(out)
+        assert np.array_equal(host(out), host(ref))
