@@ -228,12 +228,11 @@ bool verbose()
 }
 
 // Flags set by kernels whose bounded waits ran out (derr[2]); read and cleared.  Only the bulk-copy dslash
-// variants wait: with none launched since the last look the call stays asynchronous (the read and its
-// synchronisation were 25 of the 39 us of an H_w application at 4^4).
+// variants wait: a context that has launched none stays asynchronous (the read and its synchronisation were
+// 25 of the 39 us of an H_w application at 4^4).
 int check_kernel_flags(ov_ctx* c, cudaStream_t st)
 {
-    if (!c->wait_pending) return OV_OK;
-    c->wait_pending = false;
+    if (!c->waits) return OV_OK;
     unsigned f = 0;
     OV_CUDA(c, cudaMemcpyAsync(&f, c->derr + 2, sizeof f, cudaMemcpyDeviceToHost, st));
     OV_CUDA(c, cudaStreamSynchronize(st));
@@ -315,10 +314,7 @@ int dslash_apply(ov_ctx* c, const FieldDesc& in, const FieldDesc& out, double a,
     auto it = c->shape.find({in.prec, in.nrhs});
     std::tuple<int, int, int> sh = it != c->shape.end() ? it->second : default_shape(c->g, in.prec, in.nrhs);
     OV_CUDA(c, launch_dslash(A, in.prec, gprec, ny, std::get<0>(sh), std::get<1>(sh), std::get<2>(sh), st));
-    if (std::get<2>(sh) == 4 || std::get<2>(sh) == 5) {
-        c->wait_pending = true;
-        if (c->pdl) c->wait_in_graphs = true;
-    }
+    if (std::get<2>(sh) == 4 || std::get<2>(sh) == 5) c->waits = true;
     c->dslash_launches++;
     return OV_OK;
 }
@@ -549,7 +545,6 @@ void graphs_clear(ov_ctx* c)
     cudaDeviceSynchronize();
     for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second.first);
     c->graphs.clear();
-    c->wait_in_graphs = false;
 }
 
 // Run `body(s)` (a fixed sequence of kernel launches on stream s) through a
@@ -587,7 +582,6 @@ static int with_graph(ov_ctx* c, int kind, const FieldDesc& in, const FieldDesc&
     auto it = c->graphs.find(key);
     if (it != c->graphs.end()) {
         OV_CUDA(c, cudaGraphLaunch(it->second.first, gs));
-        if (c->wait_in_graphs) c->wait_pending = true;
         c->dslash_launches += it->second.second;
         c->graph_replays++;
         return join();
@@ -1539,6 +1533,7 @@ int ov_tune_dslash(ov_ctx* c, int prec, int nrhs, int* bx, int* by, int* variant
     cudaStream_t st = (cudaStream_t)stream;
     CallScope call(c, st);
     OV_TRY(call.begin());
+    const bool waited = c->waits;
     FieldDesc fi, fo;
     OV_TRY(ws_field(c, WS_IN, prec, nrhs, &fi));
     OV_TRY(ws_field(c, WS_OUT, prec, nrhs, &fo));
@@ -1619,7 +1614,9 @@ int ov_tune_dslash(ov_ctx* c, int prec, int nrhs, int* bx, int* by, int* variant
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    OV_TRY(check_kernel_flags(c, st));
+    const int fs = check_kernel_flags(c, st);
+    c->waits = waited;  // the candidates' launches are over and their flag is read
+    OV_TRY(fs);
     c->shape[{prec, nrhs}] = bsh;
     if (bx) *bx = std::get<0>(bsh);
     if (by) *by = std::get<1>(bsh);

@@ -111,9 +111,9 @@ struct ov_ctx {
     cudaStream_t gstream = nullptr;
     cudaEvent_t gev[2] = {nullptr, nullptr};
 
-    // bounded waits: launches of the bulk-copy dslash variants (the only ones that wait) whose timeout flag
-    // has not been read yet, and whether a captured graph holds such launches
-    bool wait_pending = false, wait_in_graphs = false;
+    // a bulk-copy dslash variant (the only kind that waits) has been launched or captured: from then on every
+    // canonical call reads the timeout flag, since a graph, also one of the caller's, may launch it at any time
+    bool waits = false;
 
     // instrumentation: number of dslash launches issued through this context
     long long dslash_launches = 0;

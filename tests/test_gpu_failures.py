@@ -96,3 +96,33 @@ def test_bulk_copy_wait_timeout_is_reported(variant):
     ctx.apply_dslash(dev(psi), out, -RHO, prec="f32")
     ref = oracle.dslash(dims, ABC, U, -RHO, psi[0])
     assert rel(host(out), ref) <= 1e-5
+
+
+def test_timeout_in_a_graph_of_the_caller_is_reported():
+    """The caller's replay of a captured bulk-copy launch times out: the next canonical call reports it, also
+    when other canonical calls ran between the capture and the replay."""
+    from paper_1106_4964_gb300 import Context, OverlapError
+
+    dims = (8, 8, 8, 8)
+    psi = dev(synth.gaussian_spinor(dims, 6))
+    ctx = Context(dims, ABC)
+    ctx.set_gauge(dev(synth.gauge_field(dims, 4, 0.5)))
+    fi, fo = ctx.field(1, "f32"), ctx.field(1, "f32")
+    fi.load(psi)
+    ctx.set_dslash_shape("f32", 1, 128, 1, 4)
+    out = torch.empty_like(psi)
+    ctx.dslash_field(fi, fo, -RHO)
+    ctx.apply_dslash(psi, out, -RHO, prec="f64")
+    ctx.set_option("wait_polls", 0)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        ctx.dslash_field(fi, fo, -RHO)
+    ctx.set_option("wait_polls", 1 << 22)
+    ctx.apply_dslash(psi, out, -RHO, prec="f64")
+    g.replay()
+    with pytest.raises(OverlapError) as e:
+        ctx.apply_dslash(psi, out, -RHO, prec="f64")
+    assert e.value.status == -6  # OV_ETIMEOUT
+    ctx.apply_dslash(psi, out, -RHO, prec="f64")
+    fi.close()
+    fo.close()
