@@ -1533,7 +1533,6 @@ int ov_tune_dslash(ov_ctx* c, int prec, int nrhs, int* bx, int* by, int* variant
     cudaStream_t st = (cudaStream_t)stream;
     CallScope call(c, st);
     OV_TRY(call.begin());
-    const bool waited = c->waits;
     FieldDesc fi, fo;
     OV_TRY(ws_field(c, WS_IN, prec, nrhs, &fi));
     OV_TRY(ws_field(c, WS_OUT, prec, nrhs, &fo));
@@ -1585,25 +1584,51 @@ int ov_tune_dslash(ov_ctx* c, int prec, int nrhs, int* bx, int* by, int* variant
     // the Clenshaw step.)
     const auto dsh = default_shape(c->g, prec, nrhs);
     cand.insert(cand.begin(), dsh);
-    cudaEvent_t e0, e1;
-    OV_CUDA(c, cudaEventCreate(&e0));
-    OV_CUDA(c, cudaEventCreate(&e1));
+    // timing sets the shape: what was set before comes back on every path out but the last
+    struct Restore {
+        ov_ctx* c;
+        std::pair<int, int> key;
+        std::tuple<int, int, int> sh;
+        bool had;
+        cudaEvent_t e[2] = {nullptr, nullptr};
+        bool waited;
+        ~Restore()
+        {
+            c->waits = waited;  // the candidates' launches are over and their flag is read
+            for (cudaEvent_t ev : e)
+                if (ev) cudaEventDestroy(ev);
+            if (had)
+                c->shape[key] = sh;
+            else
+                c->shape.erase(key);
+        }
+    };
+    OV_TRY(check_kernel_flags(c, st));  // earlier launches' timeouts are not the candidates'
+    const auto key = std::make_pair(prec, nrhs);
+    const auto old = c->shape.find(key);
+    Restore rs{c, key, old != c->shape.end() ? old->second : dsh, old != c->shape.end()};
+    rs.waited = c->waits;
+    OV_CUDA(c, cudaEventCreate(&rs.e[0]));
+    OV_CUDA(c, cudaEventCreate(&rs.e[1]));
     float best = 1e30f, limit = 0.f;
     bool first = true;
     std::tuple<int, int, int> bsh = cand[0];
     for (auto sh : cand) {
-        c->shape[{prec, nrhs}] = sh;
+        c->shape[key] = sh;
         for (int i = 0; i < (first ? 10 : 1); ++i)  // warm up
             OV_TRY(dslash_apply(c, fi, fo, 4.0, -0.5, 0, 0, 0, nullptr, nullptr, st));
-        OV_CUDA(c, cudaEventRecord(e0, st));
+        OV_CUDA(c, cudaEventRecord(rs.e[0], st));
         for (int i = 0; i < 10; ++i) OV_TRY(dslash_apply(c, fi, fo, 4.0, -0.5, 0, 0, 0, nullptr, nullptr, st));
-        OV_CUDA(c, cudaEventRecord(e1, st));
-        OV_CUDA(c, cudaEventSynchronize(e1));
+        OV_CUDA(c, cudaEventRecord(rs.e[1], st));
+        OV_CUDA(c, cudaEventSynchronize(rs.e[1]));
         float ms = 0;
-        OV_CUDA(c, cudaEventElapsedTime(&ms, e0, e1));
+        OV_CUDA(c, cudaEventElapsedTime(&ms, rs.e[0], rs.e[1]));
         if (verbose())
             fprintf(stderr, "[ov] tune prec %d nrhs %d: block %d x %d variant %d: %.2f us\n", prec, nrhs,
                     std::get<0>(sh), std::get<1>(sh), std::get<2>(sh), 100.0f * ms);
+        const int fs = check_kernel_flags(c, st);
+        if (fs == OV_ETIMEOUT) continue;  // this candidate did not do its work: no candidate
+        OV_TRY(fs);
         if (first) {
             limit = ms * (ms < 0.2f ? 0.95f : 0.995f);  // ms: ten launches
             first = false;
@@ -1612,12 +1637,8 @@ int ov_tune_dslash(ov_ctx* c, int prec, int nrhs, int* bx, int* by, int* variant
             bsh = sh;
         }
     }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    const int fs = check_kernel_flags(c, st);
-    c->waits = waited;  // the candidates' launches are over and their flag is read
-    OV_TRY(fs);
-    c->shape[{prec, nrhs}] = bsh;
+    rs.sh = bsh;
+    rs.had = true;
     if (bx) *bx = std::get<0>(bsh);
     if (by) *by = std::get<1>(bsh);
     if (variant) *variant = std::get<2>(bsh);

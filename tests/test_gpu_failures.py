@@ -126,3 +126,21 @@ def test_timeout_in_a_graph_of_the_caller_is_reported():
     ctx.apply_dslash(psi, out, -RHO, prec="f64")
     fi.close()
     fo.close()
+
+
+def test_autotuner_takes_no_candidate_that_timed_out():
+    """With the bulk-copy candidates' waits running out at once the autotuner takes another launch, reports no
+    error and leaves a working context."""
+    from paper_1106_4964_gb300 import Context
+
+    dims = (8, 8, 8, 8)
+    U = synth.gauge_field(dims, 4, 0.5)
+    psi = synth.gaussian_spinor(dims, 6)
+    ctx = Context(dims, ABC)
+    ctx.set_gauge(dev(U))
+    ctx.set_option("wait_polls", 0)
+    bx, by, variant = ctx.tune_dslash("f32", 1)
+    assert variant not in (4, 5)
+    out = torch.empty_like(dev(psi))
+    ctx.apply_dslash(dev(psi), out, -RHO, prec="f32")
+    assert rel(host(out), oracle.dslash(dims, ABC, U, -RHO, psi[0])) <= 1e-5
