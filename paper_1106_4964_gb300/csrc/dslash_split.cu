@@ -94,7 +94,7 @@ __device__ __forceinline__ void load_half(const DslashArgs& A, const char* in_q,
     Real v[24];
     load_spinor<SP, Real, false>(in_q, nullptr, A.g.Vh, sn, v);
     project_hop<Real>(w, v, h);
-    if (cross && A.g.fbc[w >> 1] != 1.f) {
+    if (cross && A.g.bc[w >> 1] != 1.0) {
         const Real f = (Real)A.g.bc[w >> 1];
 #pragma unroll
         for (int i = 0; i < 12; ++i) h[i] *= f;

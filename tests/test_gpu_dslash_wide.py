@@ -122,3 +122,20 @@ def test_autotuner_candidates(prec, nrhs):
     got = host(out)
     for r in range(nrhs):
         assert rel(got[r], oracle.dslash(DIMS, ABC, U, -RHO, psi[r])) <= TOL[prec]
+
+
+@pytest.mark.parametrize("prec", ["f64", "df64"])
+def test_phase_next_to_one(prec):
+    """A real boundary phase that FP32 rounds to 1 is applied."""
+    from paper_1106_4964_gb300 import Context
+
+    bc = (1.0, 1.0 - 2.0 ** -27, 1.0, 1.0 + 2.0 ** -25)
+    U = synth.gauge_field(DIMS, 1, 0.5)
+    psi = synth.gaussian_spinor(DIMS, 2)
+    ctx = Context(DIMS, bc)
+    ctx.set_gauge(dev(U))
+    out = torch.empty_like(dev(psi))
+    ctx.apply_dslash(dev(psi), out, -RHO, prec=prec)
+    ref = oracle.dslash(DIMS, bc, U, -RHO, psi[0])
+    assert rel(oracle.dslash(DIMS, (1.0,) * 4, U, -RHO, psi[0]), ref) > 100 * TOL[prec]
+    assert rel(host(out), ref) <= TOL[prec]
