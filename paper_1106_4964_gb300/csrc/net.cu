@@ -41,6 +41,7 @@ struct NetState {
     int adam_t = 0;
     int adj_valid = 0;  // Wadj matches W
     int batch = 0;      // fields the work fields hold
+    int batch_max = 16; // fields the device had room for
     // recorded training pairs: residuals and iterates (then errors), f32 single-rhs fields
     int recording = 0;
     FieldDesc pr{}, px{};
@@ -434,33 +435,50 @@ int net_init(ov_ctx* c)
     return OV_OK;
 }
 
-// work fields of a batch of nb: h, gh (16 channels each), z (9 paths), y, gy; grown when a larger batch
-// is asked for (at most net_batch fields, so that they stay below about 2 GB)
+// fields of a batch: the number asked for, such that the work fields stay below about 2 GB
 int net_batch(const ov_ctx* c, int want)
 {
-    const double per = (2.0 * NET_C + 9 + 2) * 192.0 * c->g.Vh;
+    const double per = (2.0 * NET_C + 2) * 192.0 * c->g.Vh;
     const int cap = (int)std::min(16.0, std::max(1.0, 2e9 / per));
     return std::min(want, cap);
 }
 
 struct NetWork {
-    FieldDesc h, gh, z, y, gy;
+    FieldDesc h, gh, z, y, gy, a, b, d;
 };
 
-int net_work(ov_ctx* c, int nb, NetWork* w)
+// Work fields of a batch of *nb: h and gh (16 channels each), y, gy, and those that the preconditioner asks for
+// (a, b: FP32 copies of its input and output, d: the adjoint's result).  z, the 9 paths' fields of the 16 -> 1
+// layer, lies in gh, which is written after z's last use.  They are kept, and grown when a larger batch is asked
+// for; where the device has no room for it the batch is halved (*nb) and stays there.
+int net_work(ov_ctx* c, int* nb, bool a, bool b, bool d, NetWork* w)
 {
     NetState* n = c->net;
-    if (n->batch < nb) {
-        cudaDeviceSynchronize();  // queued kernels may still use the smaller fields
-        for (int slot : {WS_NET_H, WS_NET_GH, WS_NET_Z, WS_NET_Y, WS_NET_G}) ws_release(c, slot);
-        n->batch = nb;
+    const int slots[] = {WS_NET_H, WS_NET_GH, WS_NET_Y, WS_NET_G, WS_NET_A, WS_NET_B, WS_NET_S};
+    for (int want = std::max(std::min(*nb, n->batch_max), n->batch);; want /= 2) {
+        if (n->batch < want) {
+            cudaDeviceSynchronize();  // queued kernels may still use the smaller fields
+            for (int slot : slots) ws_release(c, slot);
+        }
+        n->batch = want;
+        int s = ws_field(c, WS_NET_H, P_F32, NET_C * want, &w->h);
+        if (s == OV_OK) s = ws_field(c, WS_NET_GH, P_F32, NET_C * want, &w->gh);
+        if (s == OV_OK) s = ws_field(c, WS_NET_Y, P_F32, want, &w->y);
+        if (s == OV_OK) s = ws_field(c, WS_NET_G, P_F32, want, &w->gy);
+        if (s == OV_OK && a) s = ws_field(c, WS_NET_A, P_F32, want, &w->a);
+        if (s == OV_OK && b) s = ws_field(c, WS_NET_B, P_F32, want, &w->b);
+        if (s == OV_OK && d) s = ws_field(c, WS_NET_S, P_F32, want, &w->d);
+        if (s == OV_OK) {
+            w->z = w->gh;
+            *nb = std::min(*nb, want);
+            return OV_OK;
+        }
+        cudaDeviceSynchronize();
+        for (int slot : slots) ws_release(c, slot);
+        n->batch = 0;
+        if (s != OV_ENOMEM || want == 1) return s;
+        n->batch_max = want / 2;
     }
-    nb = n->batch;
-    OV_TRY(ws_field(c, WS_NET_H, P_F32, NET_C * nb, &w->h));
-    OV_TRY(ws_field(c, WS_NET_GH, P_F32, NET_C * nb, &w->gh));
-    OV_TRY(ws_field(c, WS_NET_Z, P_F32, 9 * nb, &w->z));
-    OV_TRY(ws_field(c, WS_NET_Y, P_F32, nb, &w->y));
-    return ws_field(c, WS_NET_G, P_F32, nb, &w->gy);
 }
 
 // layer (or its adjoint) on nb fields; z: work field of the 16 -> 1 form
@@ -498,9 +516,9 @@ int loss_grad(ov_ctx* c, const FieldDesc& pr, const FieldDesc& pe, int k0, int k
     NetState* n = c->net;
     const Geom& g = c->g;
     const int np = k1 - k0;
-    const int B = net_batch(c, np);
+    int B = net_batch(c, np);
     NetWork w;
-    OV_TRY(net_work(c, B, &w));
+    OV_TRY(net_work(c, &B, false, false, false, &w));
     const int nblk_max = 4 * 152;
     const size_t need = (size_t)nblk_max * NET_X;
     if (n->partials_n < need) {
@@ -580,14 +598,12 @@ int net_apply_precond(ov_ctx* c, const FieldDesc& r, const FieldDesc& z, cudaStr
         OV_TRY(refresh_adjoint(c, st));
         n->adj_valid = 1;
     }
-    const int R = r.nrhs, B = net_batch(c, R);
+    const int R = r.nrhs;
+    int B = net_batch(c, R);
     NetWork w;
-    OV_TRY(net_work(c, B, &w));
-    FieldDesc a, b, d;
     const bool f32in = r.prec == P_F32, f32out = z.prec == P_F32;
-    if (!f32in) OV_TRY(ws_field(c, WS_NET_A, P_F32, B, &a));
-    if (!f32out) OV_TRY(ws_field(c, WS_NET_B, P_F32, B, &b));
-    if (sym) OV_TRY(ws_field(c, WS_NET_S, P_F32, B, &d));
+    OV_TRY(net_work(c, &B, !f32in, !f32out, sym, &w));
+    const FieldDesc &a = w.a, &b = w.b, &d = w.d;
     for (int q = 0; q < R; q += B) {
         const int nb = std::min(B, R - q);
         FieldDesc rq = some(r, q, nb), zq = some(z, q, nb);

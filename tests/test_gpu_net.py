@@ -154,3 +154,45 @@ def test_train_and_flexible_cg_chiral():
                                    cf["ev"], cf["eta"])
         assert rel(Ax, b[r]) <= 1e-10
     print(f"chiral FCG: loss/pair {loss:.3e}, iterations {fcg['iterations']}, fallback {fcg['fallback']}")
+
+
+def test_batch_falls_back_on_a_full_device():
+    """Eight fields at 16^3 x 32 want a batch of four (1.7 GB of work fields): with room for less the network
+    runs smaller batches, with the same results, and later calls work too."""
+    from paper_1106_4964_gb300 import Context
+
+    dims = (16, 16, 16, 32)
+    U = dev(synth.gauge_field(dims, 21, 0.6))
+    w1, w2 = rand_weights(0)
+    x = dev(synth.gaussian_spinor(dims, 3, nrhs=8))
+
+    def make():
+        ctx = Context(dims, ABC)
+        ctx.set_gauge(U)
+        ctx.net_set_weights(np.concatenate([w1.reshape(-1), w2.reshape(-1)]))
+        return ctx
+
+    ctx = make()
+    ref, out = torch.empty_like(x), torch.empty_like(x)
+    ctx.net_apply(x, ref)
+    loss, grad = ctx.net_loss_grad(x, ref)
+    ctx.close()
+    ctx = make()
+    ctx.net_apply(x[:1].contiguous(), out[:1])
+    ctx.net_loss_grad(x, ref)  # its fields outside the batch exist
+    ctx.close()
+    ctx = make()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (1400 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        ctx.net_apply(x, out)
+        got = host(out)
+        l2, g2 = ctx.net_loss_grad(x, ref)
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert np.array_equal(got, host(ref))
+    assert abs(l2 - loss) <= 1e-5 * max(loss, 1e-30) and rel(g2, grad) <= 1e-5
+    ctx.net_apply(x, out)
+    assert np.array_equal(host(out), got)
