@@ -7,8 +7,8 @@
 // of 2^-62, and the colour multiply sums 32 x 32 -> 64-bit products: with x = x1 2^32 + x0, x0 in
 // [-2^31, 2^31),
 //   u h / 2^64 = u1 h1 + (u1 h0 + u0 h1) / 2^32 + (u0 h0) / 2^64,
-// the last term below the unit of the result and dropped.  The sum over the eight hops is a 64-bit
-// integer in units of 2^-58 of the largest component met.  Conversions, dropped terms and shifts are
+// the last term below the unit of the result and dropped, the sum rounded to nearest; zeros stay exactly zero.
+// The sum over the eight hops is a 64-bit integer in units of 2^-58 of the largest component met.  Conversions, dropped terms and shifts are
 // each below 2^-54 (double-float) or 2^-57 (FP64) of a hop's largest component, where FP64 rounds every
 // product and partial sum to 2^-53 of itself: relative to the field around the site the sum's error is
 // that of the floating-point sum or smaller.
@@ -102,8 +102,12 @@ __host__ __device__ __forceinline__ Fix to_fix(double x, uint32_t emax)
     return r;
 }
 
-// -x (one unit low in the low word)
-__host__ __device__ __forceinline__ Fix fix_neg(Fix x) { return Fix{-x.h, ~x.l}; }
+// -x, exactly (a low word of -2^31 counts as -2^31 + 1).  Zero stays zero: a complement would leave one unit in
+// every vanishing product, and fields that are exactly zero in some colours or spins (a free field's point
+// source) would fill with noise there.
+__host__ __device__ __forceinline__ Fix fix_neg(Fix x) { return Fix{-x.h, -(x.l > -2147483647 ? x.l : -2147483647)}; }
+// x or -x for m = 0 or -1; the low word of a link is never -2^31 (link_to_fix)
+__host__ __device__ __forceinline__ Fix fix_sign(Fix x, int m) { return Fix{(x.h ^ m) - m, (x.l ^ m) - m}; }
 
 // links: |u| <= 1 in units of 2^-62
 __host__ __device__ __forceinline__ Fix link_to_fix(double u)
@@ -112,6 +116,7 @@ __host__ __device__ __forceinline__ Fix link_to_fix(double u)
     Fix r;
     r.l = (int)(uint32_t)q;
     r.h = (int)((q - (long long)r.l) >> 32);
+    if (r.l == -2147483647 - 1) r.l = -2147483647;  // one unit: fix_sign
     return r;
 }
 __host__ __device__ __forceinline__ double fix_to_link(Fix a)
@@ -128,7 +133,10 @@ __host__ __device__ __forceinline__ void fix_mac(FixProd& s, Fix a, Fix b)
     s.mid += (long long)a.h * b.l;
     s.mid += (long long)a.l * b.h;
 }
-__host__ __device__ __forceinline__ long long fix_sum(const FixProd& s) { return s.hi + (s.mid >> 32); }
+__host__ __device__ __forceinline__ long long fix_sum(const FixProd& s)
+{
+    return s.hi + ((s.mid + 0x80000000ll) >> 32);  // |mid| stays below 2^63 - 2^31
+}
 
 // Exponent field of the largest of the 12 components (0: every component is zero or subnormal), FIX_BAD
 // when the format does not hold them

@@ -117,17 +117,13 @@ __device__ __forceinline__ void colour_fix(const int4* lb, int Vh, bool fwd, rea
         for (int i = 0; i < 6; ++i) f[i] = Wide<SP>::fix(h[i], emax);
 #pragma unroll
         for (int i = 0; i < 3; ++i) n[i] = fix_neg(f[2 * i + 1]);
-        if (emax == 0) {  // a vanishing hop contributes exactly nothing
-#pragma unroll
-            for (int i = 0; i < 3; ++i) n[i].l = 0;
-        }
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             FixProd re = {}, im = {};
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
                 const int4 t = __ldg(lb + i * si + j * sj);
-                const Fix ur{t.x, t.y}, ui{(t.z ^ m) - m, t.w ^ m};
+                const Fix ur{t.x, t.y}, ui = fix_sign(Fix{t.z, t.w}, m);
                 fix_mac(re, ur, f[2 * j]);
                 fix_mac(re, ui, n[j]);
                 fix_mac(im, ur, f[2 * j + 1]);

@@ -69,6 +69,37 @@ int main()
             if (fabsl((long double)a + b - tv) > ldexpl(fabsl(tv), -47) || std::fabs(b) > std::ldexp(std::fabs(a), -24))
                 return fail("to df", a, (double)tv);
         }
+        // exact zeros stay zero, whatever the link, forward and backward
+        if (t % 8 == 0) {
+            const double hz[12] = {0, 0, h[2], h[3], 0, 0, 0, 0, 0, 0, 0, 0};
+            const uint32_t ez = fix_range(hz);
+            if (ez != FIX_BAD && ez != 0) {
+                Fix f[6];
+                for (int i = 0; i < 6; ++i) f[i] = to_fix(hz[i], ez);
+                for (int m = 0; m >= -1; --m) {
+                    FixProd zr{}, zi{};
+                    const double uz[6] = {u[0], u[1], 0, 0, u[4], -u[5]};  // no coupling to the filled colour
+                    for (int j = 0; j < 3; ++j) {
+                        const Fix ur = link_to_fix(uz[2 * j]), ui = fix_sign(link_to_fix(uz[2 * j + 1]), m);
+                        fix_mac(zr, ur, f[2 * j]);
+                        fix_mac(zr, ui, fix_neg(f[2 * j + 1]));
+                        fix_mac(zi, ur, f[2 * j + 1]);
+                        fix_mac(zi, ui, f[2 * j]);
+                    }
+                    if (fix_sum(zr) != 0 || fix_sum(zi) != 0) return fail("zero product", (double)fix_sum(zr), (double)fix_sum(zi));
+                }
+            }
+        }
+        // negation and the link's conjugate are exact
+        for (int i = 0; i < 12; ++i) {
+            const Fix x = to_fix(h[i], em), y = fix_neg(x);
+            const long long vx = (long long)x.h * 4294967296ll + x.l, vy = (long long)y.h * 4294967296ll + y.l;
+            if (vx + vy != (x.l == -2147483647 - 1 ? -1 : 0)) return fail("negation", (double)vx, (double)vy);
+        }
+        for (int j = 0; j < 6; ++j) {
+            const Fix x = link_to_fix(u[j]), y = fix_sign(x, -1);
+            if (x.h != -y.h || x.l != -y.l || x.l == -2147483647 - 1) return fail("conjugate", u[j], 0);
+        }
         // double-float input
         float hh[12], hl[12], m = 0;
         for (int i = 0; i < 12; ++i) {

@@ -139,3 +139,45 @@ def test_phase_next_to_one(prec):
     ref = oracle.dslash(DIMS, bc, U, -RHO, psi[0])
     assert rel(oracle.dslash(DIMS, (1.0,) * 4, U, -RHO, psi[0]), ref) > 100 * TOL[prec]
     assert rel(host(out), ref) <= TOL[prec]
+
+
+def diagonal_links(dims, seed):
+    """SU(3) links that mix no colours: diag(e^ia, e^ib, e^-i(a+b))."""
+    rng = np.random.default_rng(seed)
+    a = rng.uniform(-3, 3, tuple(reversed(dims)) + (4, 2))
+    U = np.zeros(a.shape[:-1] + (3, 3), dtype=np.complex128)
+    for i, ph in enumerate((a[..., 0], a[..., 1], -a.sum(-1))):
+        U[..., i, i] = np.exp(1j * ph)
+    return U
+
+
+@pytest.mark.parametrize("unit", [True, False])
+@pytest.mark.parametrize("prec", ["f64", "df64"])
+def test_empty_colours_stay_empty(prec, unit):
+    """Links that mix no colours, sources in one colour: the others are exactly zero after any number of
+    applications, as with floating-point arithmetic."""
+    from paper_1106_4964_gb300 import Context
+
+    U = diagonal_links(DIMS, 3)
+    if unit:
+        U[:] = np.eye(3)
+    psi = synth.gaussian_spinor(DIMS, 2, nrhs=2)
+    psi[0][..., [0, 2]] = 0
+    psi[1] = 0
+    psi[1, 0, 0, 0, 0, 2, 1] = 1  # a point source
+    ctx = Context(DIMS, ABC)
+    ctx.set_gauge(dev(U))
+    f = [ctx.field(2, prec) for _ in range(2)]
+    f[0].load(dev(psi))
+    out = torch.empty_like(dev(psi))
+    ref = psi.copy()
+    for k in range(6):
+        ctx.dslash_field(f[k & 1], f[1 - (k & 1)], -RHO)
+        f[1 - (k & 1)].store(out)
+        got = host(out)
+        assert not got[..., [0, 2]].any()
+        for r in range(2):
+            ref[r] = oracle.dslash(DIMS, ABC, U, -RHO, ref[r]).reshape(ref[r].shape)
+            assert rel(got[r], ref[r]) <= TOL[prec]
+    for a in f:
+        a.close()
