@@ -261,7 +261,9 @@ __host__ __device__ __forceinline__ void fixd_from_fix(long long v, int e, float
     const float h0 = bits_f32(((uint32_t)ex << 23) + ((top >> 8) & 0x007fffffu) | s);
     // the next 24 bits: (1.f - 1) forms of units of 2^(ex - 24)
     const uint32_t rest = (uint32_t)(m >> 16) & 0x00ffffffu;
-    const float u = bits_f32((uint32_t)(ex - 23) << 23);  // 2^(value exponent - 23): one unit of h0's last place
+    // 2^(value exponent - 23), one unit of h0's last place; below the normal range (a sum far below hops that
+    // are themselves near the end of the range) the low word is nothing
+    const float u = bits_f32(ex > 23 ? (uint32_t)(ex - 23) << 23 : 0u);
     const float l0 = (float)(int)rest * 5.9604644775390625e-8f * (s ? -u : u);
     if (lz >= 64) {
         hi = lo = 0.f;

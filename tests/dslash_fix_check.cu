@@ -116,6 +116,16 @@ int main()
             if (fabsl(val - ((long double)hh[i] + hl[i])) > ldexpl(m, -50)) return fail("from df", hh[i], (double)val);
         }
     }
+    // sums of every size at every exponent of the double-float hops, down to the smallest
+    for (int e = (int)(FIXD_ELO >> 23); e < (int)(FIXD_EHI >> 23); ++e)
+        for (int k = 0; k < 62; ++k)
+            for (long long v : {1ll << k, -(1ll << k), (1ll << k) + (1ll << k) / 3, -(1ll << k) - (1ll << k) / 5}) {
+                float a, b;
+                fixd_from_fix(v, e, a, b);
+                const long double tv = ldexpl((long double)v, e - 184);
+                if (!(fabsl((long double)a + b - tv) <= ldexpl(fabsl(tv), -47) + ldexpl(1.0L, -126)))
+                    return fail("small to df", a, (double)tv);
+            }
     double z[12] = {};
     if (fix_range(z) != 0) return fail("zero", 0, 0);
     z[3] = 5e-324;
