@@ -156,8 +156,10 @@ def _stream(stream):
 def _lend(stream, *bufs):
     """Tell torch's allocator that device tensors are used on `stream` when that is not the current one: the calls
     return before their work is done, and a tensor that its owner drops would be handed out again."""
+    if stream is None:
+        return
     bufs = [b for b in bufs if getattr(b, "is_cuda", False)]
-    if stream is None or not bufs:
+    if not bufs:
         return
     import torch
 
