@@ -8,10 +8,11 @@
 // [-2^31, 2^31),
 //   u h / 2^64 = u1 h1 + (u1 h0 + u0 h1) / 2^32 + (u0 h0) / 2^64,
 // the last term below the unit of the result and dropped, the sum rounded to nearest; zeros stay exactly zero.
-// The sum over the eight hops is a 64-bit integer in units of 2^-58 of the largest component met.  Conversions, dropped terms and shifts are
-// each below 2^-54 (double-float) or 2^-57 (FP64) of a hop's largest component, where FP64 rounds every
-// product and partial sum to 2^-53 of itself: relative to the field around the site the sum's error is
-// that of the floating-point sum or smaller.
+// The sum over the eight hops is a 64-bit integer in units of 2^-58 of the power of two above the largest
+// component met.  Relative to a hop's largest component, cut conversions cost at most sqrt(6) 2^-59, dropped
+// terms 6 x 2^-59 and the rounding 2^-58: below 2^-55 together (2^-58 in the root mean square), where FP64
+// rounds every product and partial sum to 2^-53 of itself: relative to the field around the site the sum's
+// error is that of the floating-point sum or smaller.
 //
 // Bounds (|u row| = 1 to 1e-9, |h| < 2^60): sum of |u1 h0| <= sqrt(6) 2^61, sum of |u0 h1| <=
 // 6 x 2^59, together below 2^63; the sum of u1 h1 stays below 2^60; a hop's result is below
@@ -38,6 +39,18 @@ __host__ __device__ __forceinline__ uint32_t fix_shr(uint32_t hi, uint32_t lo, u
 #else
     const uint64_t v = ((uint64_t)hi << 32) | lo;
     return (uint32_t)(v >> (n < 32 ? n : 32));
+#endif
+}
+
+__host__ __device__ __forceinline__ unsigned long long fix_shr64(unsigned long long x, uint32_t n)
+{
+    // x >> n, 0 for n >= 64
+#ifdef __CUDA_ARCH__
+    unsigned long long r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));
+    return r;
+#else
+    return n < 64 ? x >> n : 0;
 #endif
 }
 
@@ -234,14 +247,13 @@ __host__ __device__ __forceinline__ Fix fixd_to_fix(float xh, float xl, uint32_t
     if (f == 0) m = sg = 0;
     const uint32_t d = (emax - f) >> 23;
     long long x = (long long)(((unsigned long long)(fix_shr(0u, m, d) ^ sg) << 32) | (fix_shr(m, 0u, d) ^ sg));
-    // low word, in units of 2^8 (2^-52 of the hop's largest component): at most 2^-21 of that component,
-    // so that a pair whose low word exceeds half a unit of its high word by a few bits is taken too
-    const uint32_t ml = ((lb << 7) & 0x3fffff80u) | 0x40000000u;
-    const uint32_t q = ((emax - fl) >> 23) - 21u;
-    int l = (int)fix_shr(0u, ml, q);
-    if (fl == 0) l = 0;
-    l = (int)lb < 0 ? -l : l;
-    x += (long long)l * 256;
+    // low word: 24 bits from 2^15 units up (2^-21 of the hop's largest component: a pair whose low word exceeds
+    // half a unit of its high word by a few bits is taken too), cut at one unit
+    // (a zero's exponent field shifts all of it out)
+    const unsigned long long l =
+        fix_shr64((unsigned long long)((lb & 0x007fffffu) | 0x00800000u) << 15, ((emax - fl) >> 23) - 21u);
+    const long long sl = (long long)((int)lb >> 31);
+    x += (long long)(l ^ (unsigned long long)sl) - sl;
     Fix r;
     r.l = (int)(uint32_t)x;
     r.h = (int)((uint32_t)(x >> 32) + ((uint32_t)r.l >> 31));

@@ -113,7 +113,8 @@ int main()
         for (int i = 0; i < 12; ++i) {
             const Fix f = fixd_to_fix(hh[i], hl[i], ed);
             const long double val = ldexpl((long double)(f.h * 4294967296.0L + f.l), (int)(ed >> 23) - 186);
-            if (fabsl(val - ((long double)hh[i] + hl[i])) > ldexpl(m, -50)) return fail("from df", hh[i], (double)val);
+            // two cut words, one unit each: 2^-59 of twice the largest component at most
+            if (fabsl(val - ((long double)hh[i] + hl[i])) > ldexpl(m, -58)) return fail("from df", hh[i], (double)val);
         }
     }
     // sums of every size at every exponent of the double-float hops, down to the smallest
