@@ -39,18 +39,21 @@
  *    eigenpairs, all workspaces and the network weights.
  *  - Every call returns OV_OK (0) or a negative ov_status; on error no
  *    output is guaranteed and ov_last_error() describes the failure.
- *  - Precision (ov_prec): OV_F64 stores and computes in FP64; OV_F32 in FP32;
+ *  - Precision (ov_prec): OV_F64 stores in FP64 and computes in FP64, the
+ *    hopping term apart (below); OV_F32 in FP32;
  *    OV_F16S / OV_BF16S store spinors and links in 16 bits (spinors with one
  *    FP32 scale per site) and compute in FP32; OV_DF64 stores every real as an
  *    unevaluated sum of two FP32 numbers (8 bytes, about 48 significand bits),
  *    an FP64-class result on the FP32 pipes.  The hopping term of the OV_F64
  *    and OV_DF64 dslash multiplies links and spinors as 64-bit fixed-point
- *    numbers on the integer pipes, scaled by each neighbour's largest
- *    component: the rounding, relative to the field around a site, is at most
- *    that of the floating-point sums.  Sites whose neighbourhood that format
- *    does not hold (infinities, NaN, exponents near the ends of the range,
- *    components that differ by more than 2^26 within a neighbour or 2^16
- *    between neighbours) use the floating-point arithmetic.  Dot products and
+ *    numbers on the integer pipes, scaled by the largest component of the
+ *    eight neighbours.  A complex component of its sum below 2^-6 (OV_F64) or
+ *    2^-9 (OV_DF64) of that scale is formed from its own products in the
+ *    format's floating-point arithmetic instead, so that every complex
+ *    component (not each of its two parts by itself) keeps the precision of
+ *    that arithmetic, also where links mix no colours, and exact zeros stay
+ *    zero.  Sites with infinities, NaN or exponents near the ends of the range
+ *    in their neighbourhood use floating point altogether.  Dot products and
  *    norms always accumulate in FP64.
  */
 #ifndef OVERLAP_GB300_H
@@ -105,8 +108,9 @@ const char* ov_last_error(const ov_ctx* ctx);
  * transporters on the links).  U: canonical complex128 gauge layout, host or
  * device.  The library packs it to reconstruct-12 form (rows 0 and 1 kept,
  * row 2 = conj(row0 x row1)) in FP32, FP16 and BF16, where the dslash is
- * bound by bandwidth, and keeps all three rows as 64-bit fixed-point numbers
- * (one copy) for FP64 and double-float, where it is bound by arithmetic.  Returns OV_EINVAL
+ * bound by bandwidth, and keeps all three rows, as 64-bit fixed-point numbers
+ * and in FP64, for FP64 and double-float, where it is bound by arithmetic.
+ * Returns OV_EINVAL
  * if any link deviates from SU(3) by more than 1e-9 (|U U^dag - 1| or the
  * reconstructed third row), since reconstruct-12 would change it. */
 int ov_set_gauge(ov_ctx* ctx, const void* U, void* stream);

@@ -289,7 +289,8 @@ int dslash_apply(ov_ctx* c, const FieldDesc& in, const FieldDesc& out, double a,
     A.g = c->g;
     A.err = c->derr + 2;
     A.wait_polls = c->wait_polls;
-    A.gauge = (const char*)c->gauge[gprec];
+    A.gauge = (const char*)c->gauge[wide(in.prec) ? P_DF64 : gprec];
+    A.gauge_r = (const char*)c->gauge[P_F64];
     A.in = in.data;
     A.in_n = in.norm;
     A.out = out.data;
@@ -898,7 +899,7 @@ int ov_destroy(ov_ctx* c)
     graphs_clear(c);
     net_free(c);
     for (int p = 0; p < NPREC; ++p)
-        if (c->gauge[p] && p != P_DF64) dev_free(c, c->gauge[p], (size_t)8 * c->g.Vh * gauge_link_bytes(p));
+        if (c->gauge[p]) dev_free(c, c->gauge[p], (size_t)8 * c->g.Vh * gauge_link_bytes(p));
     for (auto& e : c->eig) eig_clear(c, e);
     for (auto& kv : c->ws) field_free(c, &kv.second);
     if (c->partials) dev_free(c, c->partials, c->partials_bytes);
@@ -935,12 +936,11 @@ int ov_set_gauge(ov_ctx* c, const void* U, void* stream)
     if (c->gauge[0]) OV_CUDA(c, cudaDeviceSynchronize());  // ov_dslash_field launches, on any stream, read the links
     OV_TRY(stage_in(c, 0, U, bytes, st, &dU));
     for (int p = 0; p < NPREC; ++p) {
-        if (!c->gauge[p] && p != P_DF64) OV_TRY(dev_alloc(c, &c->gauge[p], (size_t)8 * c->g.Vh * gauge_link_bytes(p)));
+        if (!c->gauge[p]) OV_TRY(dev_alloc(c, &c->gauge[p], (size_t)8 * c->g.Vh * gauge_link_bytes(p)));
     }
-    c->gauge[P_DF64] = c->gauge[P_F64];  // one copy of the 64-bit links
     OV_CUDA(c, cudaMemsetAsync(c->derr, 0, 2 * sizeof(unsigned), st));
     for (int p = 0; p < NPREC; ++p)
-        if (p != P_DF64) OV_CUDA(c, launch_pack_gauge(c->g, dU, c->gauge[p], p, p == 0 ? c->derr : nullptr, st));
+        OV_CUDA(c, launch_pack_gauge(c->g, dU, c->gauge[p], p, p == 0 ? c->derr : nullptr, st));
     unsigned herr[2];
     OV_CUDA(c, cudaMemcpyAsync(herr, c->derr, sizeof herr, cudaMemcpyDeviceToHost, st));
     OV_CUDA(c, cudaStreamSynchronize(st));

@@ -139,6 +139,10 @@ template <int P>
 __device__ __forceinline__ void store_link(char* base, int Vh, int s, const double u[18])
 {
     if constexpr (P == P_F64) {  // all three rows
+        double2* b = reinterpret_cast<double2*>(base);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) b[(size_t)k * Vh + s] = make_double2(u[2 * k], u[2 * k + 1]);
+    } else if constexpr (P == P_DF64) {  // and as fixed-point numbers
         int4* b = reinterpret_cast<int4*>(base);
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
@@ -467,13 +471,7 @@ cudaError_t launch_unpack(const Geom& g, const FieldDesc& f, double* canon, cuda
 cudaError_t launch_pack_gauge(const Geom& g, const double* canon, void* out, int prec, unsigned* dev_err,
                               cudaStream_t st)
 {
-    switch (prec) {  // double-float uses the FP64 links
-    case P_F64: return GaugeRun<P_F64>::run(g, canon, out, dev_err, st);
-    case P_F32: return GaugeRun<P_F32>::run(g, canon, out, dev_err, st);
-    case P_F16: return GaugeRun<P_F16>::run(g, canon, out, dev_err, st);
-    case P_BF16: return GaugeRun<P_BF16>::run(g, canon, out, dev_err, st);
-    }
-    return cudaErrorInvalidValue;
+    return dispatch_prec<GaugeRun>(prec, g, canon, out, dev_err, st);
 }
 cudaError_t launch_convert(const Geom& g, const FieldDesc& in, const FieldDesc& out, cudaStream_t st)
 {

@@ -61,7 +61,7 @@ struct ov_ctx {
     int device = 0;
     long long bytes = 0;
 
-    void* gauge[ov::NPREC] = {};
+    void* gauge[ov::NPREC] = {};  // P_F64: the links in FP64; P_DF64: in fixed point, for both wide precisions
     bool have_gauge = false;
 
     double rho = 1.5, eps = 0.05, lmax = 0.0;

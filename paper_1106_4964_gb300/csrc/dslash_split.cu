@@ -15,8 +15,9 @@
 // rest waits on dependent operations and the block's barriers.
 //
 // A block walks over bx / 32 groups of sites and `by` right-hand sides (the innermost, so that a site
-// group's links are re-read from L1).  Sites that the fixed-point format does not hold send their
-// block through the same steps again in the field's own arithmetic.
+// group's links are re-read from L1).  A component far below the site's scale is formed again from its own
+// products (small_components); sites that the fixed-point format does not hold send their block through the
+// same steps again in the field's own arithmetic (hop_real).
 #include "dslash_common.cuh"
 
 namespace ov {
@@ -31,7 +32,7 @@ struct Wide;
 template <>
 struct Wide<P_F64> {
     using Real = double;
-    static constexpr int ESHIFT = 20;
+    static constexpr int ESHIFT = 20, KEEP = FIX_KEEP;
     __device__ static __forceinline__ uint32_t range(const double h[12]) { return fix_range(h); }
     __device__ static __forceinline__ Fix fix(double x, uint32_t e) { return to_fix(x, e); }
     __device__ static __forceinline__ double real(long long v, int e) { return fix_to_f64(v, e); }
@@ -45,6 +46,7 @@ struct Wide<P_F64> {
         re = __hiloint2double(t.y, t.x);
         im = __hiloint2double(t.w, t.z);
     }
+    __device__ static __forceinline__ bool zero(int4 t) { return (((t.y | t.w) << 1) | t.x | t.z) == 0; }
     __device__ static __forceinline__ int4 put(double re, double im)
     {
         return make_int4(__double2loint(re), __double2hiint(re), __double2loint(im), __double2hiint(im));
@@ -54,7 +56,7 @@ struct Wide<P_F64> {
 template <>
 struct Wide<P_DF64> {
     using Real = df64;
-    static constexpr int ESHIFT = 23;
+    static constexpr int ESHIFT = 23, KEEP = FIXD_KEEP;
     __device__ static __forceinline__ uint32_t range(const df64 h[12])
     {
         float a[12], b[12];
@@ -79,6 +81,7 @@ struct Wide<P_DF64> {
         re = df64(__int_as_float(t.x), __int_as_float(t.y));
         im = df64(__int_as_float(t.z), __int_as_float(t.w));
     }
+    __device__ static __forceinline__ bool zero(int4 t) { return (t.x | t.y | t.z | t.w) << 1 == 0; }
     __device__ static __forceinline__ int4 put(df64 re, df64 im)
     {
         return make_int4(__float_as_int(re.hi), __float_as_int(re.lo), __float_as_int(im.hi), __float_as_int(im.lo));
@@ -140,19 +143,196 @@ __device__ __forceinline__ void colour_fix(const int4* lb, int Vh, bool fwd, rea
 
 // hop w of one site in the field's own arithmetic (its own call: its registers stay out of the main path)
 template <int SP>
-__device__ __noinline__ void hop_real(const DslashArgs& A, const char* in_q, const char* lb, int w, int sn, int ls,
-                                      bool cross, int4* out)
+__device__ __noinline__ void hop_real(const DslashArgs& A, const char* in_q, int lp, int w, int sn, int ls, bool cross,
+                                      int4* out)
 {
     using Real = real_t<SP>;
     Real h[12], u[18], chi[12];
     load_half<SP>(A, in_q, w, sn, cross, h);
-    load_link<SP, Real>(lb, A.g.Vh, ls, u);
+    load_link<SP, Real>(A.gauge_r + (size_t)(lp * 4 + (w >> 1)) * A.g.Vh * 144, A.g.Vh, ls, u);
     if ((w & 1) == 0)
         link_mul<+1, Real>(u, h, chi);
     else
         link_mul<-1, Real>(u, h, chi);
 #pragma unroll
     for (int k = 0; k < 6; ++k) out[k * 32] = Wide<SP>::put(chi[2 * k], chi[2 * k + 1]);
+}
+
+template <int SP>
+struct Cplx {
+    real_t<SP> re, im;
+};
+
+// What hop w and colour j add to complex component k of the hop sum at a site of parity p, in the field's own
+// arithmetic with the FP64 links.  The link entry and the spinor's two numbers are loaded first (the loads of
+// several terms together), then multiplied; false when the link's entry or the spinor vanishes (finite fields
+// only).  Tests are on the bits: comparisons of doubles run on the FP64 pipe
+template <int SP>
+struct Term {
+    int sp, mu, a;  // output spin, direction, spin of the hop's result
+    bool fwd, cross;
+    int4 u, up, dn;
+
+    // s: the site, sn: its neighbour along hop w
+    __device__ __forceinline__ void load(const DslashArgs& A, const char* in_q, int p, int s, int sn, bool crossing, int k,
+                                         int w, int j)
+    {
+        const int Vh = A.g.Vh;
+        sp = k / 3;
+        const int col = k - 3 * sp, b = sp & 1;
+        mu = w >> 1;
+        fwd = (w & 1) == 0;
+        cross = crossing;
+        a = sp < 2 || mu >= 2 ? b : 1 - b;              // (sum_hops)
+        const int ad = 2 + (mu < 2 ? 1 - a : a);        // lower spin in its half spinor (project)
+        const int4* lb = reinterpret_cast<const int4*>(A.gauge_r) + (size_t)((fwd ? p : 1 - p) * 4 + mu) * Vh * 9;
+        const int4* v = reinterpret_cast<const int4*>(in_q) + sn;
+        u = __ldg(lb + (size_t)(fwd ? 3 * col + j : 3 * j + col) * Vh + (fwd ? s : sn));
+        up = ld_field<false>(v + (size_t)(3 * a + j) * Vh);
+        dn = ld_field<false>(v + (size_t)(3 * ad + j) * Vh);
+    }
+    __device__ __forceinline__ bool value(const DslashArgs& A, Cplx<SP>& t) const
+    {
+        using Real = real_t<SP>;
+        using W = Wide<SP>;
+        if (Wide<P_F64>::zero(u) || (W::zero(up) && W::zero(dn))) return false;
+        const bool turn = mu == 0 || mu == 2;
+        Real hr, hi, dr, di;
+        double ux, uy;
+        W::get(up, hr, hi);
+        W::get(dn, dr, di);
+        Wide<P_F64>::get(u, ux, uy);
+        // (A_mu d)_a: -i d1, -i d0 | -d1, d0 | -i d0, i d1 | d0, d1; h = up - S (A_mu d)_a
+        const bool add = ((mu == 1 && a == 0) || (mu == 2 && a == 1)) == fwd;
+        hr += W::flip(turn ? di : dr, !add);
+        hi += W::flip(turn ? -dr : di, !add);
+        if (cross && A.g.bc[mu] != 1.0) {
+            const Real f = (Real)A.g.bc[mu];
+            hr *= f;
+            hi *= f;
+        }
+        const Real ur = (Real)ux, ui = (Real)(fwd ? uy : -uy);
+        const Real re = fmac<Real>(-ui, hi, ur * hr), im = fmac<Real>(ui, hr, ur * hi);
+        if (sp < 2) {
+            t.re = re;
+            t.im = im;
+            return true;
+        }
+        // -S A_mu^dag chi (sum_hops)
+        const bool neg = fwd != ((mu == 1 || mu == 2) && (sp & 1));
+        t.re = W::flip(turn ? -im : re, neg);
+        t.im = W::flip(turn ? re : im, neg);
+        return true;
+    }
+};
+
+// The component as the sum of its 24 terms: one lane's own site, for warps where many lanes need it
+template <int SP>
+__device__ __forceinline__ Cplx<SP> component_lane(const DslashArgs& A, const char* in_q, int p, int s, int k)
+{
+    int c[4];
+    cb_coords(A.g, s, p, c);
+    Cplx<SP> sum{real_t<SP>(0), real_t<SP>(0)};
+#pragma unroll 1
+    for (int w = 0; w < 8; ++w) {
+        int sn;
+        bool cross;
+        hop_neighbour(A.g, w, s, c, sn, cross);
+        Term<SP> x[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) x[j].load(A, in_q, p, s, sn, cross, k, w, j);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            Cplx<SP> t;
+            if (!x[j].value(A, t)) continue;
+            sum.re += t.re;
+            sum.im += t.im;
+        }
+    }
+    return sum;
+}
+
+template <int SP>
+__device__ __forceinline__ real_t<SP> shfl_xor(real_t<SP> x, int m)
+{
+    if constexpr (SP == P_DF64)
+        return df64(__shfl_xor_sync(~0u, x.hi, m), __shfl_xor_sync(~0u, x.lo, m));
+    else
+        return __shfl_xor_sync(~0u, x, m);
+}
+
+// the same by the whole warp for one site: a term per lane
+template <int SP>
+__device__ __forceinline__ Cplx<SP> component_warp(const DslashArgs& A, const char* in_q, int p, int s, int k)
+{
+    const int lane = threadIdx.x & 31, w = lane / 3;
+    int c[4];
+    cb_coords(A.g, s, p, c);
+    Cplx<SP> t{real_t<SP>(0), real_t<SP>(0)};
+    if (lane < 24) {
+        int sn;
+        bool cross;
+        hop_neighbour(A.g, w, s, c, sn, cross);
+        Term<SP> x;
+        x.load(A, in_q, p, s, sn, cross, k, w, lane - 3 * w);
+        x.value(A, t);
+    }
+#pragma unroll
+    for (int m = 16; m; m >>= 1) {
+        t.re += shfl_xor<SP>(t.re, m);
+        t.im += shfl_xor<SP>(t.im, m);
+    }
+    return t;
+}
+
+// component k (hop sum re, im) of site s: epilogue and store
+template <int SP, int NY>
+__device__ __forceinline__ void store_component(const DslashArgs& A, int r, int p, int s, int k, real_t<SP> re,
+                                                real_t<SP> im)
+{
+    using Real = real_t<SP>;
+    using W = Wide<SP>;
+    const size_t off = ((size_t)r * 2 + p) * 192 * A.g.Vh + ((size_t)k * A.g.Vh + s) * 16;
+    // gamma5 on spins 2, 3: its signs on the coefficients
+    const bool low = k >= 6;
+    const Real a = W::flip(W::coef(A.a, A.da), low && (A.g5_core ^ A.g5_out));
+    const Real b = W::flip(W::coef(A.b, A.db), low && (A.g5_core ^ A.g5_out));
+    Real xr, xi;
+    W::get(ld_field<false>(reinterpret_cast<const int4*>(A.in + off)), xr, xi);
+    Real o0 = a * xr + b * re, o1 = a * xi + b * im;
+#pragma unroll
+    for (int j = 0; j < NY; ++j) {
+        const Real sj = W::flip(W::coef(A.sy[j], A.dsy[j]), low && A.g5_out);
+        W::get(ld_field<false>(reinterpret_cast<const int4*>(A.y[j] + off)), xr, xi);
+        o0 += sj * xr;
+        o1 += sj * xi;
+    }
+    *reinterpret_cast<int4*>(A.out + off) = W::put(o0, o1);
+}
+
+// Components w and w + 8 of the lanes of need0 and need1, which the main path has not stored (its own call: its
+// registers stay out of the main path).  Few lanes: a term per lane of the warp, site by site (one lane by itself
+// would hold up its block for the latency of 24 dependent steps: FP64 12 sources at 8^3 x 16 93 us, 57 this way)
+template <int SP, int NY>
+__device__ __noinline__ void small_components(const DslashArgs& A, const char* in_q, int r, int p, int s, int w,
+                                              unsigned need0, unsigned need1)
+{
+    const int lane = threadIdx.x & 31;
+    for (int k = w; k < 12; k += 8) {
+        unsigned need = k < 8 ? need0 : need1;
+        if (__popc(need) > 8) {
+            if (need >> lane & 1) {
+                const Cplx<SP> t = component_lane<SP>(A, in_q, p, s, k);
+                store_component<SP, NY>(A, r, p, s, k, t.re, t.im);
+            }
+            continue;
+        }
+        for (; need; need &= need - 1) {
+            const int src = __ffs((int)need) - 1;
+            const Cplx<SP> t = component_warp<SP>(A, in_q, p, __shfl_sync(~0u, s, src), k);
+            if (lane == src) store_component<SP, NY>(A, r, p, s, k, t.re, t.im);
+        }
+    }
 }
 
 template <int SP, int NY, int MINB>
@@ -193,28 +373,23 @@ __global__ void __launch_bounds__(SPLIT_THREADS, MINB) dslash_split_kernel(const
                 colour_fix<SP>(lf, g.Vh, fwd, h, e, &sh[w][0][lane]);
             }
             __syncthreads();
-            uint32_t emax = 0, emin = FIX_BAD;
+            uint32_t emax = 0;
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const uint32_t e = she[k][lane];
-                emax = max(emax, e);
-                emin = min(emin, e - 1u);  // a vanishing hop wraps to the top
-            }
-            const bool bad = emax == FIX_BAD || (emax != 0 && emax - emin > ((uint32_t)FIX_HOPS << W::ESHIFT) + 1u);
-            const bool redo = __syncthreads_or(bad);
+            for (int k = 0; k < 8; ++k) emax = max(emax, she[k][lane]);
+            const bool redo = __syncthreads_or(emax == FIX_BAD);
             if (redo) {
-                hop_real<SP>(A, in_q, lb, w, sn, ls, cross, &sh[w][0][lane]);
+                hop_real<SP>(A, in_q, fwd ? p : q, w, sn, ls, cross, &sh[w][0][lane]);
                 __syncthreads();
             }
             // 12 complex components over 8 warps
-            int d[8];  // right shift of each hop to the common unit (at most FIX_HOPS unless the block redoes)
-            if (!redo) {
+            uint32_t d[8];  // right shift of each hop to the common unit
 #pragma unroll
-                for (int k = 0; k < 8; ++k) d[k] = (int)((emax - she[k][lane]) >> W::ESHIFT) & 31;
-            }
+            for (int k = 0; k < 8; ++k) d[k] = (emax - she[k][lane]) >> W::ESHIFT;
+            unsigned need0 = 0, need1 = 0;  // lanes whose component w, w + 8 has to be formed again
             for (int k = w; k < 12; k += 8) {
                 const int sp = k / 3, col = k - 3 * sp;
                 Real re, im;
+                bool store = live;
                 if (redo) {
                     sum_hops<Real>(sp, [&](int hop, int a, Real& x, Real& y) { W::get(sh[hop][3 * a + col][lane], x, y); },
                                    re, im);
@@ -223,32 +398,24 @@ __global__ void __launch_bounds__(SPLIT_THREADS, MINB) dslash_split_kernel(const
                     sum_hops<long long>(sp,
                                         [&](int hop, int a, long long& x, long long& y) {
                                             const int4 t = sh[hop][3 * a + col][lane];
-                                            x = fix_sar(t.y, t.x, d[hop]);
-                                            y = fix_sar(t.w, t.z, d[hop]);
+                                            x = fix_sar(((long long)t.y << 32) | (uint32_t)t.x, d[hop]);
+                                            y = fix_sar(((long long)t.w << 32) | (uint32_t)t.z, d[hop]);
                                         },
                                         vr, vi);
                     const int e = (int)(emax >> W::ESHIFT);
                     re = W::real(vr, e);
                     im = W::real(vi, e);
+                    const bool small = fix_small(vr, vi, W::KEEP) && emax != 0 && live;
+                    const unsigned need = __ballot_sync(~0u, small);
+                    if (k < 8)
+                        need0 = need;
+                    else
+                        need1 = need;
+                    store = live && !small;
                 }
-                if (!live) continue;
-                const size_t off = ((size_t)r * 2 + p) * par_bytes + ((size_t)k * g.Vh + s) * 16;
-                // gamma5 on spins 2, 3: its signs on the coefficients
-                const bool low = sp >= 2;
-                const Real a = W::flip(W::coef(A.a, A.da), low && (A.g5_core ^ A.g5_out));
-                const Real b = W::flip(W::coef(A.b, A.db), low && (A.g5_core ^ A.g5_out));
-                Real xr, xi;
-                W::get(ld_field<false>(reinterpret_cast<const int4*>(A.in + off)), xr, xi);
-                Real o0 = a * xr + b * re, o1 = a * xi + b * im;
-#pragma unroll
-                for (int j = 0; j < NY; ++j) {
-                    const Real sj = W::flip(W::coef(A.sy[j], A.dsy[j]), low && A.g5_out);
-                    W::get(ld_field<false>(reinterpret_cast<const int4*>(A.y[j] + off)), xr, xi);
-                    o0 += sj * xr;
-                    o1 += sj * xi;
-                }
-                *reinterpret_cast<int4*>(A.out + off) = W::put(o0, o1);
+                if (store) store_component<SP, NY>(A, r, p, s, k, re, im);
             }
+            if (need0 | need1) small_components<SP, NY>(A, in_q, r, p, s, w, need0, need1);
             __syncthreads();  // shared memory is rewritten by the next right-hand side
         }
     }

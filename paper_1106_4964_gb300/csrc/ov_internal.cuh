@@ -17,8 +17,8 @@
 // Gauge links: forward links only; FP32 and 16-bit keep only rows 0 and 1 of
 // each SU(3) matrix (reconstruct-12): link[p][mu][k][s] = U_mu(n), n = site (p, s); chunks
 // are 3 float4 (FP32) or 3 x 4 16-bit values; FP64 and double-float keep all
-// three rows as 64-bit fixed point (dslash_fix.cuh), 9 int4 (re high, re low, im high,
-// im low), one copy for both.
+// three rows twice, one copy for both precisions: as 64-bit fixed point (dslash_fix.cuh), 9 int4 (re high, re
+// low, im high, im low), and in FP64, 9 double2.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -479,12 +479,12 @@ template <int P, typename Real>
 __device__ __forceinline__ void load_link_rows(const char* __restrict__ base, int Vh, int s, Real u[18])
 {
     if constexpr (P == P_DF64 || P == P_F64) {
-        const int4* b = reinterpret_cast<const int4*>(base);
+        const double2* b = reinterpret_cast<const double2*>(base);  // the FP64 links
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            const int4 t = __ldg(b + (size_t)k * Vh + s);
-            u[2 * k] = (Real)fix_to_link(Fix{t.x, t.y});
-            u[2 * k + 1] = (Real)fix_to_link(Fix{t.z, t.w});
+            const double2 t = __ldg(b + (size_t)k * Vh + s);
+            u[2 * k] = (Real)t.x;
+            u[2 * k + 1] = (Real)t.y;
         }
     } else if constexpr (P == P_F32) {
         const float4* b = reinterpret_cast<const float4*>(base);
@@ -550,12 +550,12 @@ __device__ __forceinline__ void load_link(const char* __restrict__ base, int Vh,
 {
     load_link_rows<P, Real>(base, Vh, s, u);
     if constexpr (P == P_DF64 || P == P_F64) {  // stored third row (9 chunks per link)
-        const int4* b = reinterpret_cast<const int4*>(base);
+        const double2* b = reinterpret_cast<const double2*>(base);
 #pragma unroll
         for (int k = 6; k < 9; ++k) {
-            const int4 t = __ldg(b + (size_t)k * Vh + s);
-            u[2 * k] = (Real)fix_to_link(Fix{t.x, t.y});
-            u[2 * k + 1] = (Real)fix_to_link(Fix{t.z, t.w});
+            const double2 t = __ldg(b + (size_t)k * Vh + s);
+            u[2 * k] = (Real)t.x;
+            u[2 * k + 1] = (Real)t.y;
         }
     } else {
         link_row2<Real>(u);

@@ -11,7 +11,8 @@ namespace ov {
 // ---------------------------------------------------------------- dslash
 struct DslashArgs {
     Geom g;
-    const char* gauge;           // packed links of the gauge precision
+    const char* gauge;           // packed links of the gauge precision (FP64 and double-float: in fixed point)
+    const char* gauge_r;         // FP64 links
     const char* in;              // input field (all rhs, both parities)
     const float* in_n;
     char* out;

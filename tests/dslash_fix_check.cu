@@ -1,6 +1,6 @@
 // Host-side check of the fixed-point hop (dslash_fix.cuh) against 80-bit sums: one row of the colour
 // multiply for random unit rows and half spinors over the exponent range, with zero components, with
-// every component at the bound, and the conversions to and from FP64 and double-float.  Prints "ok" or
+// every component at the bound, with components far below the largest, and the conversions to and from FP64 and double-float.  Prints "ok" or
 // the first failure.
 #include <cmath>
 #include <cstdio>
@@ -32,13 +32,7 @@ int main()
         for (double x : h) mx = std::fmax(mx, std::fabs(x));
         if (mx == 0) continue;
         const uint32_t em = fix_range(h);
-        if (em == FIX_BAD) {
-            double mn = mx;
-            for (double x : h)
-                if (x != 0) mn = std::fmin(mn, std::fabs(x));
-            if (mn * 33554432.0 > mx) return fail("refused", mn, mx);
-            continue;
-        }
+        if (em == FIX_BAD) return fail("refused", mx, 0);
         FixProd re{}, im{};
         long double rr = 0, ri = 0;
         for (int j = 0; j < 3; ++j) {
@@ -59,8 +53,8 @@ int main()
             const long double ex = ldexpl((long double)v, e - 1080), ref = k ? ri : rr;
             if (fabsl(ex - ref) > ldexpl(mx, -55)) return fail("row", (double)ex, (double)ref);
             if (fabsl(fix_to_f64(v, e) - ex) > ldexpl(fabsl(ex), -53)) return fail("to f64", fix_to_f64(v, e), (double)ex);
-            const int sh = (int)(g() % 32);
-            if (fix_sar((int)(v >> 32), (int)v, sh) != (v >> sh)) return fail("shift", (double)v, sh);
+            const uint32_t sh = (uint32_t)(g() % 100);
+            if (fix_sar(v, sh) != (v >> (sh < 63 ? sh : 63))) return fail("shift", (double)v, sh);
             // double-float result: 47 significand bits, low word at most half a unit of the high one
             float a, b;
             const int ed = 80 + (int)(g() % 160);
@@ -68,6 +62,42 @@ int main()
             const long double tv = ldexpl((long double)v, ed - 184);
             if (fabsl((long double)a + b - tv) > ldexpl(fabsl(tv), -47) || std::fabs(b) > std::ldexp(std::fabs(a), -24))
                 return fail("to df", a, (double)tv);
+        }
+        // links that mix no colours, components down to 2^-60 of the largest: what is not formed again keeps the
+        // field's precision relative to the complex component itself
+        if (t % 2) {
+            double hw[12];
+            float fh[12], fl[12];
+            for (int i = 0; i < 12; ++i) {
+                hw[i] = i == 11 ? sc : std::ldexp(n(g), -(int)(g() % 60)) * sc;
+                fh[i] = (float)(hw[i] / sc);
+                fl[i] = (float)(hw[i] / sc - fh[i]);
+            }
+            const uint32_t ew = fix_range(hw), efw = fixd_range(fh, fl);
+            if (ew == FIX_BAD || efw == FIX_BAD) return fail("wide refused", 0, 0);
+            const double ph = 0.7 + 1e-5 * t, cr = std::cos(ph), sr = std::sin(ph);
+            const Fix ur = link_to_fix(cr), ui = link_to_fix(sr);
+            for (int j = 0; j < 6; ++j)
+                for (int df = 0; df < 2; ++df) {
+                    const long double xr = df ? (long double)fh[2 * j] + fl[2 * j] : hw[2 * j];
+                    const long double xi = df ? (long double)fh[2 * j + 1] + fl[2 * j + 1] : hw[2 * j + 1];
+                    const Fix a = df ? fixd_to_fix(fh[2 * j], fl[2 * j], efw) : to_fix(hw[2 * j], ew);
+                    const Fix b = df ? fixd_to_fix(fh[2 * j + 1], fl[2 * j + 1], efw) : to_fix(hw[2 * j + 1], ew);
+                    FixProd pr{}, pi{};
+                    fix_mac(pr, ur, a);
+                    fix_mac(pr, ui, fix_neg(b));
+                    fix_mac(pi, ur, b);
+                    fix_mac(pi, ui, a);
+                    const long long vr = fix_sum(pr), vi = fix_sum(pi);
+                    if (fix_small(vr, vi, df ? FIXD_KEEP : FIX_KEEP)) continue;
+                    const int ex = df ? (int)(efw >> 23) - 184 : (int)(ew >> 20) - 1080;
+                    const long double er = ldexpl((long double)vr, ex) - ((long double)cr * xr - (long double)sr * xi);
+                    const long double ei = ldexpl((long double)vi, ex) - ((long double)cr * xi + (long double)sr * xr);
+                    const long double mag = hypotl(xr, xi), err = hypotl(er, ei);
+                    // per part: two conversions of one unit of 2^-60, dropped terms 2 x 2^-60 and half a unit of
+                    // 2^-58 (all below one unit of 2^-58) of a scale that is below 2^KEEP of the component
+                    if (err > ldexpl(mag, df ? FIXD_KEEP - 57 : FIX_KEEP - 57)) return fail("component", (double)(err / mag), df);
+                }
         }
         // exact zeros stay zero, whatever the link, forward and backward
         if (t % 8 == 0) {

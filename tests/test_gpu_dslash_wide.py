@@ -181,3 +181,73 @@ def test_empty_colours_stay_empty(prec, unit):
             assert rel(got[r], ref[r]) <= TOL[prec]
     for a in f:
         a.close()
+
+
+def reference(dims, bc, U, m, psi):
+    """D_w psi in extended precision, and the weight of its roundings: |4 + m| |psi| + 1/2 sum |U_ij| |h_j|."""
+    U, psi = U.astype(np.clongdouble), psi.astype(np.clongdouble)
+    up, dn = psi[..., :2, :], psi[..., 2:, :]
+    out, w = (4 + np.longdouble(m)) * psi, abs(4 + m) * np.abs(psi)
+
+    def amul(mu, d, g):  # A_mu d (g = -1) or A_mu^dag d (g = 1)
+        a, b = d[..., 0, :], d[..., 1, :]
+        x = [(1j * g * b, 1j * g * a), (g * b, -g * a), (1j * g * a, -1j * g * b), (a, b)][mu]
+        return np.stack(x, axis=-2)
+
+    for mu in range(4):
+        ax = 3 - mu
+        for s in (1, -1):
+            h = up - s * amul(mu, dn, -1)
+            u = U[..., mu, :, :]
+            edge = [slice(None)] * 6
+            edge[ax] = -1 if s > 0 else 0
+            if s > 0:
+                h = np.roll(h, -1, ax)
+            else:
+                u = np.conj(np.swapaxes(u, -1, -2))
+            chi, mag = np.einsum("...ij,...aj->...ai", u, h), np.einsum("...ij,...aj->...ai", np.abs(u), np.abs(h))
+            if s < 0:
+                chi, mag = np.roll(chi, 1, ax), np.roll(mag, 1, ax)
+            chi[tuple(edge)] *= bc[mu]
+            out[..., :2, :] -= chi / 2
+            out[..., 2:, :] += s * amul(mu, chi, 1) / 2
+            w[..., :2, :] += mag / 2
+            w[..., 2:, :] += mag[..., ::-1, :] / 2 if mu < 2 else mag / 2
+    return out, w
+
+
+def component_cases():
+    rng = np.random.default_rng(11)
+    base = synth.gaussian_spinor(DIMS, 2)
+    mixing, diag = synth.gauge_field(DIMS, 1, 0.5), diagonal_links(DIMS, 3)
+    weak = synth.gauge_field(DIMS, 1, 1e-9)  # off-diagonal entries of 1e-9: below the fixed-point links' last bits
+    colours = base * 2.0 ** np.array([0.0, -30.0, -50.0])
+    spread = base * 2.0 ** rng.integers(-35, 36, base.shape)
+    site = base * 2.0 ** rng.integers(-40, 41, base.shape[:5])[..., None, None]
+    one = base.copy()
+    one[..., 1:] = 0
+    near = base * 2.0 ** -rng.integers(0, 12, base.shape)  # across the line below which a component is formed again
+    return {"mixing": (mixing, base), "mixing_spread": (mixing, spread), "mixing_site": (mixing, site),
+            "mixing_near": (mixing, near), "diagonal_colours": (diag, colours), "diagonal_spread": (diag, spread),
+            "diagonal_site": (diag, site), "diagonal_near": (diag, near), "weak_one_colour": (weak, one),
+            "weak_colours": (weak, colours), "point": (diag, synth.point_sources(DIMS)[4:5])}
+
+
+@pytest.mark.parametrize("name", sorted(component_cases()))
+@pytest.mark.parametrize("prec", ["f64", "df64"])
+def test_every_component_keeps_its_precision(prec, name):
+    """Component by component against extended precision.  Floating point: 24 roundings of the products and
+    sums that make a component, and 4 of the epilogue.  Fixed point: 8 hops of at most 3.6 units of 2^-58 of the
+    scale, 2^6 (FP64) or 2^9 (double-float) times which the component is: 2^-47.1 or 2^-44.1 of it.  Both are
+    below 64 units of 2^-53 (FP64) or 2^-47 (double-float: 24 operations of 2^-46)."""
+    U, psi = component_cases()[name]
+    if prec == "df64":  # the pair's 48 bits
+        hi = psi.view(np.float64).astype(np.float32)
+        psi = (hi.astype(np.float64) + (psi.view(np.float64) - hi).astype(np.float32)).view(np.complex128)
+    got = apply(prec, U, psi)[0]
+    ref, w = reference(DIMS, ABC, U, -RHO, psi[0])
+    err = np.abs(got.astype(np.clongdouble) - ref).astype(np.float64)
+    bound = 64 * {"f64": 2.0 ** -53, "df64": 2.0 ** -47}[prec] * w.astype(np.float64)
+    worst = float((err / np.where(bound > 0, bound, 1)).max())
+    print(f"{prec} {name}: {worst:.2e} of the bound")
+    assert np.all(err <= bound), worst
