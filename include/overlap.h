@@ -47,12 +47,12 @@
  *    an FP64-class result on the FP32 pipes.  The hopping term of the OV_F64
  *    and OV_DF64 dslash multiplies links and spinors as 64-bit fixed-point
  *    numbers on the integer pipes, scaled by the largest component of the
- *    eight neighbours.  A complex component of its sum below 2^-6 (OV_F64) or
- *    2^-9 (OV_DF64) of that scale is formed from its own products in the
- *    format's floating-point arithmetic instead, so that every complex
- *    component (not each of its two parts by itself) keeps the precision of
- *    that arithmetic, also where links mix no colours, and exact zeros stay
- *    zero.  Sites with infinities, NaN or exponents near the ends of the range
+ *    eight neighbours.  A complex component to which no neighbour adds more than
+ *    2^-6 (OV_F64) or 2^-9 (OV_DF64) of that scale is formed from its own
+ *    products in the format's floating-point arithmetic instead, so that every
+ *    complex component (not each of its two parts by itself) keeps the
+ *    precision of that arithmetic, also where links mix no colours, and exact
+ *    zeros stay zero.  Sites with infinities, NaN or exponents near the ends of the range
  *    in their neighbourhood use floating point altogether.  Dot products and
  *    norms always accumulate in FP64.
  */

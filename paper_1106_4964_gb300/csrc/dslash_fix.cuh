@@ -20,15 +20,16 @@
 //
 // Where links mix colours, that error lies below the rounding of the larger products in every component.  Where
 // they do not (a free field, block-diagonal links, one filled colour) a component can be far below the largest
-// one and floating point would still hold it to all its bits.  So a complex component of the sum below
-// 2^-FIX_KEEP of the scale, exact zeros among them, is formed again from its own products in the field's
-// arithmetic with the links in FP64 (fix_small).  What stays has an error of at most 8 x 3.6 units of 2^-58 of
-// the scale, 2^FIX_KEEP times which it is: 2^-47 of itself in FP64, 2^-44 in double-float, some 2^-51 in the
-// root mean square.  Largest error of a component in units of 2^-53 of its |u| |h|, FP64 sums / this form:
-// Gaussian fields on mixing links 1.4 / 0.9, components spread over 2^12 on diagonal links 3.1 / 2.7, sites
-// spread over 2^80 there 5.2 / 10.9.  Gaussian fields send one component in 4000 that way (FP64; a few per
-// million in double-float): 24^3 x 64 427 -> 450 us in FP64 (613 -> 596 in double-float, which gains by the
-// range checks it no longer needs).
+// one and floating point would still hold it to all its bits.  So a complex component of which the sum and all
+// eight hops' parts are below 2^-FIX_KEEP of the scale, exact zeros among them, is formed again from its own
+// products in the field's arithmetic with the links in FP64 (fix_small).  (A small sum of larger parts is
+// left: floating point rounds the parts as well.)  What stays has an error of at most 8 x 3.6 units of 2^-58
+// of the scale, 2^FIX_KEEP times which its largest part is: 2^-47 of that in FP64, 2^-44 in double-float, some
+// 2^-51 in the root mean square.  Largest error of a component in units of 2^-53 of its |u| |h|, FP64 sums /
+// this form: Gaussian fields on mixing links 1.4 / 0.9, components spread over 2^12 on diagonal links 3.1 / 2.7,
+// sites spread over 2^80 there 5.2 / 10.9.  24^3 x 64, us per launch without and with it: FP64 427 / 436,
+// double-float (which needs no range checks any more) 613 / 600; 12 point sources' solve at 8^4 with FP64
+// residuals 329 / 356 ms (510 with a test of the sum alone: the colours that the links hardly reach).
 //
 // What the format does not hold at all goes to the field's own arithmetic, block by block: infinities, NaN,
 // values near the ends of the exponent range.

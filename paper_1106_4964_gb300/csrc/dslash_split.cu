@@ -405,7 +405,15 @@ __global__ void __launch_bounds__(SPLIT_THREADS, MINB) dslash_split_kernel(const
                     const int e = (int)(emax >> W::ESHIFT);
                     re = W::real(vr, e);
                     im = W::real(vi, e);
-                    const bool small = fix_small(vr, vi, W::KEEP) && emax != 0 && live;
+                    bool small = fix_small(vr, vi, W::KEEP) && emax != 0 && live;
+                    if (small) {  // unless by cancellation between the hops, which floating point rounds as well
+#pragma unroll 1
+                        for (int hop = 0; hop < 8 && small; ++hop) {
+                            const int4 t = sh[hop][3 * (sp < 2 || hop >= 4 ? sp & 1 : 1 - (sp & 1)) + col][lane];
+                            const uint32_t n = (emax - she[hop][lane]) >> W::ESHIFT;
+                            small = fix_small(fix_sar((long long)t.y << 32, n), fix_sar((long long)t.w << 32, n), W::KEEP);
+                        }
+                    }
                     const unsigned need = __ballot_sync(~0u, small);
                     if (k < 8)
                         need0 = need;
