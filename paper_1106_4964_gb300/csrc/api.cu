@@ -259,14 +259,16 @@ static std::tuple<int, int, int> default_shape(const Geom& g, int prec, int nrhs
 {
     const long n = 2L * g.Vh * nrhs;
     // FP64, double-float: one block of eight warps per 32 sites and right-hand side (64-site blocks: 12.4
-    // against 10.3 us at 8^3 x 16).  Two blocks per SM while there are few (us, variants 0 / 1 / 2: FP64
-    // 8^3 x 16 7.9 / 8.3 / 8.7, double-float 4^4 6.0 / 6.4 / 6.7), then three (12 sources: FP64 8^4 34.1 / 29.2 /
-    // 29.4, double-float 8^3 x 16 74.1 / 69.7 / 72.3, 24^3 x 64 645 / 598 / 611), and four where the FP64 launch
-    // is long enough for the spills of 64 registers not to matter (24^3 x 64 555 / 450 / 423)
-    if (wide(prec)) return {32, 1, n <= 20000 ? 0 : (prec == P_F64 && n > 200000 ? 2 : 1)};
+    // against 10.3 us at 8^3 x 16).  Two blocks per SM (variant 0) while there are few, then three, and four where
+    // the FP64 launch is long enough for the spills of 64 registers not to matter.  us for variants 0 / 1 / 2 by
+    // sites x right-hand sides: FP64 256 6.2 / 6.4 / 6.6, 8192 8.2 / 8.5 / 9.1, 16384 14.4 / 13.9 / 13.7, 49152
+    // 35.6 / 29.7 / 30.4, 98304 64.8 / 53.6 / 53.9, 131072 88.5 / 71.0 / 69.3, 884736 573 / 451 / 436; double-float
+    // 8192 9.2 / 10.0 / 10.6, 16384 16.3 / 16.1 / 16.7, 98304 73.9 / 70.8 / 72.6, 884736 628 / 601 / 614
+    if (wide(prec)) return {32, 1, n <= 12000 ? 0 : (prec == P_F64 && n > 110000 ? 2 : 1)};
     // FP32 arithmetic by sites x right-hand sides.  One warp per hop while one site per thread would leave most
-    // of the chip idle (us, against 64 x 1 variant 0: 4^4 2.2 / 2.8, 8^4 2.3 / 3.0, FP16 8^3 x 16 3.1 / 3.5, two
-    // sources at 8^4 3.1 / 3.3; three 3.9 / 3.6 in BF16, 12^4 4.4 / 4.3); then unbounded registers while the
+    // of the chip idle (us, variant 12 against 64 x 1 variant 0, FP32 | FP16 | BF16: 256 2.1 / 3.0 | 2.5 / 3.0 |
+    // 2.5 / 3.4, 4096 2.4 / 3.2 | 2.5 / 3.1 | 2.6 / 3.5, 8640 3.1 / 3.4 | 3.1 / 3.3 | 3.2 / 3.7, 10000 3.3 / 3.6 |
+    // 3.5 / 3.2 | 3.6 / 3.7, 12288 3.4 / 3.5 | 3.8 / 3.2 | 3.9 / 3.6); then unbounded registers while the
     // blocks fit at once, and more resident warps beyond (variant 1 against 0: 12 sources at 8^3 x 16 9.1 / 9.0,
     // two at 16^3 x 32 20.0 / 20.3, 12 there 101.7 / 107.5; blocks of 32 sites x 12 sources 157)
     if (n <= 9000) return {32, 1, 12};
