@@ -391,8 +391,7 @@ struct UpArgs {
     int stages;
     int R;
     int Vh;
-    int mode;              // 0: FP32 fields, out1 = psi - corr, out2 = gamma5 w; 1: out1 = corr, out2 = gamma5 w
-    const float* psi;      // FP32 field (mode 0)
+    const float* psi;      // FP32 field (MODE 0)
     float* out1;
     float* out2;           // may be null
     int* err;
@@ -407,6 +406,10 @@ __device__ __forceinline__ uint64_t smem_desc_mn(const void* p, uint32_t lbo)
            (1ull << 46) | (2ull << 61);
 }
 
+// MODE 0: out1 = psi - corr (FP32 fields); 1: out1 = corr, subtracted by proj_combine_kernel (16-bit fields).  The
+// epilogue is a chain of one warp per scheduler: code for psi that mode 1 only steps over cost it a third of its
+// time (12 right-hand sides and 100 rows at 16^3 x 32: 263 us with one kernel for both, 176 by itself)
+template <int MODE>
 __global__ void __launch_bounds__(UP_THREADS, 1)
     proj_update_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmAlo,
                           const __grid_constant__ CUtensorMap tmB, UpArgs P)
@@ -529,17 +532,19 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
         constexpr int RMAX = 16;
         float ps[RMAX];
         auto load_psi = [&](long long it) {
+            if (MODE != 0) return;
             const long long k = (blockIdx.x + it * gridDim.x) * UP_M + row;
 #pragma unroll
             for (int r = 0; r < RMAX; ++r)
-                ps[r] = (P.mode == 0 && r < P.R && it < my_tiles) ? __ldg(P.psi + r * rhs_reals + k) : 0.f;
+                ps[r] = (r < P.R && it < my_tiles) ? __ldg(P.psi + r * rhs_reals + k) : 0.f;
         };
         load_psi(0);
         for (long long it = 0; it < my_tiles; ++it) {
             const int a = (int)(it & 1);
             float cur[RMAX];
 #pragma unroll
-            for (int r = 0; r < RMAX; ++r) cur[r] = ps[r];
+            for (int r = 0; r < RMAX; ++r)
+                if (MODE == 0) cur[r] = ps[r];
             load_psi(it + 1);
             if (*(volatile int*)&abort_flag) break;
             if (!mbar_wait(&tfull[a], (uint32_t)((it >> 1) & 1))) {
@@ -569,7 +574,7 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
                     const float YWp = __shfl_xor_sync(0xffffffffu, YW, 1);
                     if (r < P.R) {
                         const float corr = X + sg * Yp, w = XW + sg * YWp;
-                        o1[r * rhs_reals] = P.mode == 0 ? cur[r] - corr : corr;
+                        o1[r * rhs_reals] = MODE == 0 ? cur[r] - corr : corr;
                         if (o2) o2[r * rhs_reals] = g5 * w;
                     }
                 }
@@ -720,9 +725,11 @@ int proj_update_tc(ov_ctx* c, int which, const FieldDesc& psi, const double2* dc
     const int stages = std::min(4, (int)((kSmemMax - 1024 - (int)bbytes) / (int)stage_bytes));
     if (stages < 2) return set_err(c, OV_EINVAL, "tensor-core update: tiles do not fit in shared memory");
     const size_t smem = (size_t)stages * stage_bytes + bbytes + 1024;
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(proj_update_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
-    OV_CUDA(c, attr);
+    const auto kernel = P == P_F32 ? proj_update_tc_kernel<0> : proj_update_tc_kernel<1>;
+    static const cudaError_t attr[2] = {
+        cudaFuncSetAttribute(proj_update_tc_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax),
+        cudaFuncSetAttribute(proj_update_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax)};
+    OV_CUDA(c, attr[P == P_F32 ? 0 : 1]);
     if (!c->tc_err) {
         void* p = nullptr;
         OV_TRY(dev_alloc(c, &p, sizeof(int)));
@@ -742,21 +749,19 @@ int proj_update_tc(ov_ctx* c, int which, const FieldDesc& psi, const double2* dc
     a.err = c->tc_err;
     FieldDesc corr{}, wf{};
     if (P == P_F32) {
-        a.mode = 0;
         a.psi = (const float*)psi.data;
         a.out1 = (float*)out1.data;
         a.out2 = out2.data ? (float*)out2.data : nullptr;
     } else {
         OV_TRY(ws_field(c, WS_TC0, P_F32, R, &corr));
         if (out2.data) OV_TRY(ws_field(c, WS_TC1, P_F32, R, &wf));
-        a.mode = 1;
         a.out1 = (float*)corr.data;
         a.out2 = out2.data ? (float*)wf.data : nullptr;
     }
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     const int grid = (int)std::min<long long>(a.ntiles, sms);
-    proj_update_tc_kernel<<<grid, UP_THREADS, smem, st>>>(ma, malo, mb, a);
+    kernel<<<grid, UP_THREADS, smem, st>>>(ma, malo, mb, a);
     OV_CUDA(c, cudaGetLastError());
     if (P != P_F32) {
         const dim3 g2((2 * c->g.Vh + 127) / 128, R);
