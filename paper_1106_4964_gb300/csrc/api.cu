@@ -268,10 +268,16 @@ static std::tuple<int, int, int> default_shape(const Geom& g, int prec, int nrhs
     // FP32 arithmetic by sites x right-hand sides.  One warp per hop while one site per thread would leave most
     // of the chip idle (us, variant 12 against 64 x 1 variant 0, FP32 | FP16 | BF16: 256 2.1 / 3.0 | 2.5 / 3.0 |
     // 2.5 / 3.4, 4096 2.4 / 3.2 | 2.5 / 3.1 | 2.6 / 3.5, 8640 3.1 / 3.4 | 3.1 / 3.3 | 3.2 / 3.7, 10000 3.3 / 3.6 |
-    // 3.5 / 3.2 | 3.6 / 3.7, 12288 3.4 / 3.5 | 3.8 / 3.2 | 3.9 / 3.6); then unbounded registers while the
-    // blocks fit at once, and more resident warps beyond (variant 1 against 0: 12 sources at 8^3 x 16 9.1 / 9.0,
-    // two at 16^3 x 32 20.0 / 20.3, 12 there 101.7 / 107.5; blocks of 32 sites x 12 sources 157)
+    // 3.5 / 3.2 | 3.6 / 3.7, 12288 3.4 / 3.5 | 3.8 / 3.2 | 3.9 / 3.6).  Then unbounded registers, all sources of 32
+    // sites in one block while that is a wave or two, 64-site blocks of one source beyond (FP32, us per launch of an
+    // overlap application, 32 x R against 64 x 1: three sources at 8^4 4.4 / 5.3, seven 5.9 / 6.1, twelve 5.7 / 6.3, seven
+    // at 8^3 x 16 6.1 / 6.2 (bare launch 6.2 / 5.8), twelve 10.2 / 8.9, five at 12^4 10.0 / 9.8, twelve 29.5 / 21.2);
+    // one and two sources keep theirs longer (128 x 1 against 64 x 1 at 16^3 x 32 11.1 / 11.4, 12^4 6.11 / 6.06;
+    // 32 x 2 12.2 / 12.4 at 14 x 10 x 18 x 30, 24.5 / 24.7 at 16^3 x 32).  More resident warps last (variant 1 against
+    // 0: 12 sources at 8^3 x 16 8.9 / 8.9, five at 14 x 10 x 18 x 30 34.4 / 34.6, three at 16^3 x 32 35.3 / 36.5)
     if (n <= 9000) return {32, 1, 12};
+    if (nrhs == 1 && n > 45000 && n <= 300000) return {128, 1, 0};
+    if (nrhs > 1 && n <= (nrhs == 2 ? 300000 : 50000)) return {32, nrhs < 16 ? nrhs : 16, 0};
     return {64, 1, n <= 200000 ? 0 : 1};
 }
 
@@ -432,7 +438,7 @@ static int overlap_core(ov_ctx* c, const FieldDesc& in, const FieldDesc& out, do
             OV_CUDA(c, launch_proj_finalize((double2*)c->partials, nparts, (int)ncoef, dcoef, st));
         }
         // the update of one FP32 right-hand side streams the rows once on the CUDA cores, faster than the
-        // tensor cores' rows plus remainder rows (measured 0.24 against 0.32 ms at 16^3 x 32, 100 rows)
+        // tensor cores' rows plus remainder rows (measured 0.24 against 0.26 ms at 16^3 x 32, 100 rows)
         if (tc && !(P == P_F32 && R == 1))
             OV_TRY(proj_update_tc(c, 0, in, dcoef, E.d_sign, ph, w, st));
         else

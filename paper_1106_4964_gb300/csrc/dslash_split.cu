@@ -9,10 +9,11 @@
 // the multiply in the instruction cache instead of eight (the straight-line double-float kernel was
 // 14 000 instructions and stalled on instruction fetch for three quarters of its time).
 //
-// us per launch at 24^3 x 64 / 12 right-hand sides at 8^3 x 16 / one at 4^4: FP64 423 / 54 / 5.9 (one thread
-// per site and FP64 multiply-adds: 1583 / 190 / 33), double-float 592 / 70 / 6.0 (973 / 209 / 28).  The integer
-// multiply pipe is 57 %, the integer and FP64 pipes 42 % busy (FP64); half of the issue slots are used, the
-// rest waits on dependent operations and the block's barriers.
+// us per launch at 24^3 x 64 / 12 right-hand sides at 8^3 x 16 / one at 4^4: FP64 436 / 54 / 5.8 (one thread
+// per site and FP64 multiply-adds: 1583 / 190 / 33), double-float 600 / 71 / 5.8 (973 / 209 / 28).  12 right-hand
+// sides at 8^3 x 16: FP64 51 % of the integer multiply pipe, 45 % of the FP64 and 37 % of the integer pipe;
+// double-float 58 % of the integer pipe; half of the issue slots are used, the rest waits on dependent
+// operations and the block's barriers.
 //
 // A block walks over bx / 32 groups of sites and `by` right-hand sides (the innermost, so that a site
 // group's links are re-read from L1).  A component far below the site's scale is formed again from its own
