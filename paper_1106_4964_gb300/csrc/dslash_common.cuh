@@ -219,17 +219,37 @@ struct Bounds {
 // Programmatic dependent launch: a kernel lets its successor's blocks start as soon as all of its own have
 // started, and waits for its predecessor to complete before it touches memory (fields by ordinary loads, see
 // ld_field; only the links, which no launch of a graph writes, by read-only ones), so that inside a captured
-// graph the launch and the index arithmetic of one launch run under the tail of the one before (FP64 overlap
-// at 4^4, 201 launches: 1307 -> 1191 us; 12-source CG at 8^4 361 -> 347 ms; nothing at 16^3 x 32 and above).
+// graph the launch and the index arithmetic of one launch run under the tail of the one before.
 __device__ __forceinline__ void pdl_begin()
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Only while the launch is small or fills the chip: in between, the blocks that wait settle unevenly on the SMs
+// that have room, and the launch takes as long as the fullest of them.  The limits are in warps per SM, one pair
+// for each kernel, where overlap applications with and without it cross (us per launch, with / without, by
+// sites x sources):
+//  one site per thread: off in (3, 9.5]: 10000 4.1 / 4.5, 16384 5.3 / 4.6, 20736 5.9 / 4.8, 41472 6.3 / 5.5, 49152
+//    5.3 / 5.8, 131072 11.2 / 11.7; and on for up to half as many blocks as SMs: 15552, 12 sources, 6.1 / 6.6
+//  FP32, one warp per hop: off above 6.7: 256 1.9 / 2.5, 2592 2.4 / 2.7, 3888 2.5 / 2.7, 4096 2.6 / 2.5, 5184
+//    3.6 / 3.1, 8192 3.2 / 2.9
+//  FP64 and double-float: off in (2.2, 8], between a quarter and one block per SM: FP64 1024 6.2 / 6.5, 1296
+//    6.5 / 6.5, 2592 7.8 / 6.8, 4096 7.9 / 6.6, 5184 8.0 / 8.8; double-float 1024 6.1 / 6.2, 2048 7.9 / 6.5, 4096
+//    8.8 / 6.7, 5184 8.9 / 9.7
+struct PdlRange {
+    float off_above, on_above;  // warps per SM
+    unsigned on_blocks;         // on for up to so many blocks in any case
+};
+constexpr PdlRange PDL_SITE{3.f, 9.5f, 76}, PDL_HOP32{6.7f, 64.f, 0}, PDL_SPLIT{2.2f, 8.f, 0};
+
 template <class... P, class... Args>
-cudaError_t launch_kernel(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t st, bool pdl, const Args&... args)
+cudaError_t launch_kernel(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t st, bool pdl, PdlRange range,
+                          const Args&... args)
 {
+    constexpr float SMS = 152.f;
+    const float warps = (float)grid.x * (float)((block.x * block.y + 31) / 32) / SMS;
+    if (warps > range.off_above && warps <= range.on_above && grid.x > range.on_blocks) pdl = false;
     if (!pdl) {
         k<<<grid, block, 0, st>>>(P(args)...);
         return cudaGetLastError();

@@ -141,10 +141,10 @@ struct Hop32 {
     {
         const dim3 grid = block_grid(A.g.Vh, 32, A.nrhs), block(HOP_THREADS);
         switch (ny) {
-        case 0: return launch_kernel(dslash_hop_kernel<SP, GP, 0>, grid, block, st, A.pdl, A);
-        case 1: return launch_kernel(dslash_hop_kernel<SP, GP, 1>, grid, block, st, A.pdl, A);
-        case 2: return launch_kernel(dslash_hop_kernel<SP, GP, 2>, grid, block, st, A.pdl, A);
-        case 3: return launch_kernel(dslash_hop_kernel<SP, GP, 3>, grid, block, st, A.pdl, A);
+        case 0: return launch_kernel(dslash_hop_kernel<SP, GP, 0>, grid, block, st, A.pdl, PDL_HOP32, A);
+        case 1: return launch_kernel(dslash_hop_kernel<SP, GP, 1>, grid, block, st, A.pdl, PDL_HOP32, A);
+        case 2: return launch_kernel(dslash_hop_kernel<SP, GP, 2>, grid, block, st, A.pdl, PDL_HOP32, A);
+        case 3: return launch_kernel(dslash_hop_kernel<SP, GP, 3>, grid, block, st, A.pdl, PDL_HOP32, A);
         }
         return cudaErrorInvalidValue;
     }

@@ -10,10 +10,10 @@ cudaError_t launch_var(const DslashArgs& A, int ny, dim3 grid, dim3 block, cudaS
 {
     if ((int)(block.x * block.y) > Bounds<SP, VAR>::maxt) return cudaErrorInvalidValue;
     switch (ny) {
-    case 0: return launch_kernel(dslash_kernel<SP, GP, 0, VAR>, grid, block, st, A.pdl, A);
-    case 1: return launch_kernel(dslash_kernel<SP, GP, 1, VAR>, grid, block, st, A.pdl, A);
-    case 2: return launch_kernel(dslash_kernel<SP, GP, 2, VAR>, grid, block, st, A.pdl, A);
-    case 3: return launch_kernel(dslash_kernel<SP, GP, 3, VAR>, grid, block, st, A.pdl, A);
+    case 0: return launch_kernel(dslash_kernel<SP, GP, 0, VAR>, grid, block, st, A.pdl, PDL_SITE, A);
+    case 1: return launch_kernel(dslash_kernel<SP, GP, 1, VAR>, grid, block, st, A.pdl, PDL_SITE, A);
+    case 2: return launch_kernel(dslash_kernel<SP, GP, 2, VAR>, grid, block, st, A.pdl, PDL_SITE, A);
+    case 3: return launch_kernel(dslash_kernel<SP, GP, 3, VAR>, grid, block, st, A.pdl, PDL_SITE, A);
     }
     return cudaErrorInvalidValue;
 }

@@ -435,10 +435,10 @@ cudaError_t launch_ny(const DslashArgs& A, int ny, int ngrp, int by, cudaStream_
 {
     const dim3 grid = block_grid(A.g.Vh, 32 * ngrp, (A.nrhs + by - 1) / by);
     switch (ny) {
-    case 0: return launch_kernel(dslash_split_kernel<SP, 0, MINB>, grid, dim3(SPLIT_THREADS), st, A.pdl, A, ngrp, by);
-    case 1: return launch_kernel(dslash_split_kernel<SP, 1, MINB>, grid, dim3(SPLIT_THREADS), st, A.pdl, A, ngrp, by);
-    case 2: return launch_kernel(dslash_split_kernel<SP, 2, MINB>, grid, dim3(SPLIT_THREADS), st, A.pdl, A, ngrp, by);
-    case 3: return launch_kernel(dslash_split_kernel<SP, 3, MINB>, grid, dim3(SPLIT_THREADS), st, A.pdl, A, ngrp, by);
+    case 0: return launch_kernel(dslash_split_kernel<SP, 0, MINB>, grid, dim3(SPLIT_THREADS), st, A.pdl, PDL_SPLIT, A, ngrp, by);
+    case 1: return launch_kernel(dslash_split_kernel<SP, 1, MINB>, grid, dim3(SPLIT_THREADS), st, A.pdl, PDL_SPLIT, A, ngrp, by);
+    case 2: return launch_kernel(dslash_split_kernel<SP, 2, MINB>, grid, dim3(SPLIT_THREADS), st, A.pdl, PDL_SPLIT, A, ngrp, by);
+    case 3: return launch_kernel(dslash_split_kernel<SP, 3, MINB>, grid, dim3(SPLIT_THREADS), st, A.pdl, PDL_SPLIT, A, ngrp, by);
     }
     return cudaErrorInvalidValue;
 }
