@@ -52,9 +52,9 @@ __device__ __forceinline__ void block_sum(double v[NC])
 // A block of unpack converts PK_SITES consecutive canonical sites (one contiguous block of complex128)
 // through shared memory, so that both sides move whole lines: thread t < 64 holds the parity-0 site of site pair
 // t, the others the parity-1 sites (Lx is even: a pair shares its row and its checkerboard index).
-// FP64 operations are kept out (2 per clock and SM): signs and the FP32 conversions are integer work
-// (f64_to_f32, f32_to_f64).  12 FP32 right-hand sides at 24^3 x 64, 3.06 GB: unpack 480 us, 645 with one
-// site per thread, FP64 sign products and conversions.
+// FP64 operations are kept out (2 per clock and SM): the FP32 conversions are integer work (f32_to_f64; the
+// double-float pack's too).  12 FP32 right-hand sides at 24^3 x 64, 3.06 GB: unpack 480 us, 645 with one site per
+// thread, FP64 sign products and conversions.
 constexpr int PK_SITES = 128;
 constexpr int PK_STRIDE = 13;  // double2 per staged site (12, padded against bank conflicts)
 
@@ -79,9 +79,11 @@ __device__ __forceinline__ PackSite pack_site(const Geom& g, long n0)
 }
 
 // pack reads its sites directly: a thread's twelve 16-byte loads share their lines with its neighbours' in
-// L1 (staging them through shared memory: 519 against 449 us for the 3.06 GB above)
+// L1 (staging them through shared memory: 519 against 449 us for the 3.06 GB above).  One FP64 conversion per real
+// is hidden behind the loads; the integer form of it and a bound on the block's size, which lets the compiler take
+// registers for all loads at once, cost 17 and 10 % (12 FP32 right-hand sides at 16^3 x 32: 73.5 us, 86 and 80)
 template <int P>
-__global__ void __launch_bounds__(PK_SITES) pack_kernel(Geom g, const double2* __restrict__ canon, char* data, float* norm)
+__global__ void pack_kernel(Geom g, const double2* __restrict__ canon, char* data, float* norm)
 {
     const long V = 2L * g.Vh, n = (long)blockIdx.x * PK_SITES + threadIdx.x;
     const int r = blockIdx.y;
@@ -97,8 +99,13 @@ __global__ void __launch_bounds__(PK_SITES) pack_kernel(Geom g, const double2* _
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
         const double2 c = __ldg(src + k);
-        v[2 * k] = from_f64<Real>(c.x);
-        v[2 * k + 1] = from_f64<Real>(c.y);
+        if constexpr (std::is_same<Real, float>::value) {
+            v[2 * k] = (float)c.x;
+            v[2 * k + 1] = (float)c.y;
+        } else {
+            v[2 * k] = from_f64<Real>(c.x);
+            v[2 * k + 1] = from_f64<Real>(c.y);
+        }
     }
     constexpr size_t CH = nchunk_dev<P>() * 16;
     const size_t rp = (size_t)r * 2 + p;
