@@ -29,7 +29,7 @@
 // this form: Gaussian fields on mixing links 1.4 / 0.9, components spread over 2^12 on diagonal links 3.1 / 2.7,
 // sites spread over 2^80 there 5.2 / 10.9.  24^3 x 64, us per launch without and with it: FP64 427 / 436,
 // double-float (which needs no range checks any more) 613 / 600; 12 point sources' solve at 8^4 with FP64
-// residuals 329 / 356 ms (510 with a test of the sum alone: the colours that the links hardly reach).
+// residuals, whose fields have such components, 337 / 351 ms (a test of the sum alone would make it 510).
 //
 // What the format does not hold at all goes to the field's own arithmetic, block by block: infinities, NaN,
 // values near the ends of the exponent range.

@@ -166,8 +166,8 @@ struct Cplx {
 
 // What hop w and colour j add to complex component k of the hop sum at a site of parity p, in the field's own
 // arithmetic with the FP64 links.  The link entry and the spinor's two numbers are loaded first (the loads of
-// several terms together), then multiplied; false when the link's entry or the spinor vanishes (finite fields
-// only).  Tests are on the bits: comparisons of doubles run on the FP64 pipe
+// several terms together), then multiplied; nothing is done when the link's entry or the spinor vanishes (finite
+// fields only).  Tests are on the bits: comparisons of doubles run on the FP64 pipe
 template <int SP>
 struct Term {
     int sp, mu, a;  // output spin, direction, spin of the hop's result
@@ -192,11 +192,12 @@ struct Term {
         up = ld_field<false>(v + (size_t)(3 * a + j) * Vh);
         dn = ld_field<false>(v + (size_t)(3 * ad + j) * Vh);
     }
-    __device__ __forceinline__ bool value(const DslashArgs& A, Cplx<SP>& t) const
+    // t += the term
+    __device__ __forceinline__ void add_to(const DslashArgs& A, Cplx<SP>& t) const
     {
         using Real = real_t<SP>;
         using W = Wide<SP>;
-        if (Wide<P_F64>::zero(u) || (W::zero(up) && W::zero(dn))) return false;
+        if (Wide<P_F64>::zero(u) || (W::zero(up) && W::zero(dn))) return;
         const bool turn = mu == 0 || mu == 2;
         Real hr, hi, dr, di;
         double ux, uy;
@@ -212,22 +213,21 @@ struct Term {
             hr *= f;
             hi *= f;
         }
-        const Real ur = (Real)ux, ui = (Real)(fwd ? uy : -uy);
-        const Real re = fmac<Real>(-ui, hi, ur * hr), im = fmac<Real>(ui, hr, ur * hi);
-        if (sp < 2) {
-            t.re = re;
-            t.im = im;
-            return true;
+        if (sp >= 2) {  // -S A_mu^dag chi (sum_hops): chi, or i chi, with a sign
+            const bool neg = fwd != ((mu == 1 || mu == 2) && (sp & 1));
+            const Real x = turn ? -hi : hr, y = turn ? hr : hi;
+            hr = W::flip(x, neg);
+            hi = W::flip(y, neg);
         }
-        // -S A_mu^dag chi (sum_hops)
-        const bool neg = fwd != ((mu == 1 || mu == 2) && (sp & 1));
-        t.re = W::flip(turn ? -im : re, neg);
-        t.im = W::flip(turn ? re : im, neg);
-        return true;
+        const Real ur = (Real)ux, ui = (Real)(fwd ? uy : -uy);
+        t.re = fmac<Real>(ur, hr, t.re);
+        t.im = fmac<Real>(ur, hi, t.im);
+        t.re = fmac<Real>(-ui, hi, t.re);
+        t.im = fmac<Real>(ui, hr, t.im);
     }
 };
 
-// The component as the sum of its 24 terms: one lane's own site, for warps where many lanes need it
+// The component as the sum of its 24 terms by one lane
 template <int SP>
 __device__ __forceinline__ Cplx<SP> component_lane(const DslashArgs& A, const char* in_q, int p, int s, int k)
 {
@@ -243,12 +243,7 @@ __device__ __forceinline__ Cplx<SP> component_lane(const DslashArgs& A, const ch
 #pragma unroll
         for (int j = 0; j < 3; ++j) x[j].load(A, in_q, p, s, sn, cross, k, w, j);
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            Cplx<SP> t;
-            if (!x[j].value(A, t)) continue;
-            sum.re += t.re;
-            sum.im += t.im;
-        }
+        for (int j = 0; j < 3; ++j) x[j].add_to(A, sum);
     }
     return sum;
 }
@@ -260,30 +255,6 @@ __device__ __forceinline__ real_t<SP> shfl_xor(real_t<SP> x, int m)
         return df64(__shfl_xor_sync(~0u, x.hi, m), __shfl_xor_sync(~0u, x.lo, m));
     else
         return __shfl_xor_sync(~0u, x, m);
-}
-
-// the same by the whole warp for one site: a term per lane
-template <int SP>
-__device__ __forceinline__ Cplx<SP> component_warp(const DslashArgs& A, const char* in_q, int p, int s, int k)
-{
-    const int lane = threadIdx.x & 31, w = lane / 3;
-    int c[4];
-    cb_coords(A.g, s, p, c);
-    Cplx<SP> t{real_t<SP>(0), real_t<SP>(0)};
-    if (lane < 24) {
-        int sn;
-        bool cross;
-        hop_neighbour(A.g, w, s, c, sn, cross);
-        Term<SP> x;
-        x.load(A, in_q, p, s, sn, cross, k, w, lane - 3 * w);
-        x.value(A, t);
-    }
-#pragma unroll
-    for (int m = 16; m; m >>= 1) {
-        t.re += shfl_xor<SP>(t.re, m);
-        t.im += shfl_xor<SP>(t.im, m);
-    }
-    return t;
 }
 
 // component k (hop sum re, im) of site s: epilogue and store
@@ -312,13 +283,15 @@ __device__ __forceinline__ void store_component(const DslashArgs& A, int r, int 
 }
 
 // Components w and w + 8 of the lanes of need0 and need1, which the main path has not stored (its own call: its
-// registers stay out of the main path).  Few lanes: a term per lane of the warp, site by site (one lane by itself
-// would hold up its block for the latency of 24 dependent steps: FP64 12 sources at 8^3 x 16 93 us, 57 this way)
+// registers stay out of the main path).  Where many lanes need it, each takes its own site; else four sites at a
+// time, eight lanes each, a lane the three terms of one hop.  us per FP64 launch for 12 sources at 8^4, Gaussian fields
+// (no such component) / a propagator's columns (one in a few hundred): 30.9 / 36.6; a term per lane and one site at a
+// time 30.4 / 40.6.  24^3 x 64, unit links, one filled colour: 1037, without the lanes' own form 2283.
 template <int SP, int NY>
 __device__ __noinline__ void small_components(const DslashArgs& A, const char* in_q, int r, int p, int s, int w,
                                               unsigned need0, unsigned need1)
 {
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, hop = lane & 7;
     for (int k = w; k < 12; k += 8) {
         unsigned need = k < 8 ? need0 : need1;
         if (__popc(need) > 8) {
@@ -328,10 +301,30 @@ __device__ __noinline__ void small_components(const DslashArgs& A, const char* i
             }
             continue;
         }
-        for (; need; need &= need - 1) {
-            const int src = __ffs((int)need) - 1;
-            const Cplx<SP> t = component_warp<SP>(A, in_q, p, __shfl_sync(~0u, s, src), k);
-            if (lane == src) store_component<SP, NY>(A, r, p, s, k, t.re, t.im);
+        while (need) {
+            unsigned mine = need;  // the lowest set lane that is left to these eight lanes
+            for (int i = lane >> 3; i; --i) mine &= mine - 1;
+            const int sm = __shfl_sync(~0u, s, mine ? __ffs((int)mine) - 1 : 0);
+            Cplx<SP> t{real_t<SP>(0), real_t<SP>(0)};
+            if (mine) {
+                int c[4], sn;
+                bool cross;
+                cb_coords(A.g, sm, p, c);
+                hop_neighbour(A.g, hop, sm, c, sn, cross);
+                Term<SP> x[3];
+#pragma unroll
+                for (int j = 0; j < 3; ++j) x[j].load(A, in_q, p, sm, sn, cross, k, hop, j);
+#pragma unroll
+                for (int j = 0; j < 3; ++j) x[j].add_to(A, t);
+            }
+#pragma unroll
+            for (int m = 4; m; m >>= 1) {
+                t.re += shfl_xor<SP>(t.re, m);
+                t.im += shfl_xor<SP>(t.im, m);
+            }
+            if (mine && hop == 0) store_component<SP, NY>(A, r, p, sm, k, t.re, t.im);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) need &= need - 1;
         }
     }
 }
