@@ -281,7 +281,7 @@ __host__ __device__ __forceinline__ Fix fixd_to_fix(float xh, float xl, uint32_t
     return r;
 }
 
-// v 2^-184 2^e as a normalised pair (24 + 24 significand bits)
+// v 2^-184 2^e as a normalised pair (24 + 24 significand bits), rounded to nearest
 __host__ __device__ __forceinline__ void fixd_from_fix(long long v, int e, float& hi, float& lo)
 {
     const unsigned long long sg = (unsigned long long)(v >> 63);
@@ -292,12 +292,13 @@ __host__ __device__ __forceinline__ void fixd_from_fix(long long v, int e, float
     const uint32_t s = (uint32_t)sg & 0x80000000u;
     const uint32_t top = (uint32_t)(m >> 32);
     const float h0 = bits_f32(((uint32_t)ex << 23) + ((top >> 8) & 0x007fffffu) | s);
-    // the next 24 bits: (1.f - 1) forms of units of 2^(ex - 24)
-    const uint32_t rest = (uint32_t)(m >> 16) & 0x00ffffffu;
+    // the next 32 bits, rounded to nearest as they become a float (cut, every sum would come out short by 2^-48 on
+    // average, and a chain of applications shrinks with it)
+    const uint32_t rest = (uint32_t)(m >> 8);
     // 2^(value exponent - 23), one unit of h0's last place; below the normal range (a sum far below hops that
     // are themselves near the end of the range) the low word is nothing
     const float u = bits_f32(ex > 23 ? (uint32_t)(ex - 23) << 23 : 0u);
-    const float l0 = (float)(int)rest * 5.9604644775390625e-8f * (s ? -u : u);
+    const float l0 = (float)rest * 2.3283064365386962890625e-10f * (s ? -u : u);
     if (lz >= 64) {
         hi = lo = 0.f;
         return;

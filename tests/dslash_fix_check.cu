@@ -20,6 +20,7 @@ int main()
 {
     std::mt19937_64 g(1);
     std::normal_distribution<double> n;
+    double bias = 0;  // mean relative error of the conversion to pairs
     for (int t = 0; t < 200000; ++t) {
         double u[6], nn = 0, h[12], mx = 0;
         for (double& x : u) {
@@ -62,6 +63,7 @@ int main()
             const long double tv = ldexpl((long double)v, ed - 184);
             if (fabsl((long double)a + b - tv) > ldexpl(fabsl(tv), -47) || std::fabs(b) > std::ldexp(std::fabs(a), -24))
                 return fail("to df", a, (double)tv);
+            if (v) bias += (double)(((long double)a + b - tv) / tv) / 400000.0;
         }
         // links that mix no colours, components down to 2^-60 of the largest: what is not formed again keeps the
         // field's precision relative to the complex component itself
@@ -147,6 +149,8 @@ int main()
             if (fabsl(val - ((long double)hh[i] + hl[i])) > ldexpl(m, -58)) return fail("from df", hh[i], (double)val);
         }
     }
+    // rounding to nearest: 2^-49 in the root mean square, 2^-58 in the mean of 400 000 (cut: -2^-48.5)
+    if (std::fabs(bias) > std::ldexp(1.0, -54)) return fail("bias", bias, 0);
     // sums of every size at every exponent of the double-float hops, down to the smallest
     for (int e = (int)(FIXD_ELO >> 23); e < (int)(FIXD_EHI >> 23); ++e)
         for (int k = 0; k < 62; ++k)

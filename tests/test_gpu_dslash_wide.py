@@ -251,3 +251,29 @@ def test_every_component_keeps_its_precision(prec, name):
     worst = float((err / np.where(bound > 0, bound, 1)).max())
     print(f"{prec} {name}: {worst:.2e} of the bound")
     assert np.all(err <= bound), worst
+
+
+@pytest.mark.parametrize("prec,tol", [("f64", 6e-16), ("double_float", 5e-15)])
+def test_roundings_do_not_add_up(prec, tol):
+    """Twelve applications against extended precision: an unbiased rounding grows with the root of their number
+    (2.5e-15 and 1.5e-16 for one, mostly the pair's and FP64's rounding of the result, of which D_w averages
+    nine), a sum that is always cut short with the number itself (2.6e-15 each in double-float)."""
+    from paper_1106_4964_gb300 import Context
+
+    prec = {"double_float": "df64"}.get(prec, prec)
+    U, psi = synth.gauge_field(DIMS, 1, 0.5), synth.gaussian_spinor(DIMS, 2)
+    ctx = Context(DIMS, ABC)
+    ctx.set_gauge(dev(U))
+    f = [ctx.field(1, prec) for _ in range(2)]
+    f[0].load(dev(psi))
+    ref = psi[0].astype(np.clongdouble)
+    for k in range(12):
+        ctx.dslash_field(f[k & 1], f[1 - (k & 1)], -RHO)
+        ref = reference(DIMS, ABC, U, -RHO, ref)[0]
+    out = torch.empty_like(dev(psi))
+    f[0].store(out)
+    err = float(np.linalg.norm((host(out)[0] - ref).ravel()) / np.linalg.norm(ref.ravel()))
+    print(f"{prec}: {err:.2e}")
+    for a in f:
+        a.close()
+    assert err <= tol
