@@ -268,16 +268,18 @@ static std::tuple<int, int, int> default_shape(const Geom& g, int prec, int nrhs
     // FP32 arithmetic by sites x right-hand sides.  One warp per hop while one site per thread would leave most
     // of the chip idle (us, variant 12 against 64 x 1 variant 0, FP32 | FP16 | BF16: 256 2.1 / 3.0 | 2.5 / 3.0 |
     // 2.5 / 3.4, 4096 2.4 / 3.2 | 2.5 / 3.1 | 2.6 / 3.5, 8640 3.1 / 3.4 | 3.1 / 3.3 | 3.2 / 3.7, 10000 3.3 / 3.6 |
-    // 3.5 / 3.2 | 3.6 / 3.7, 12288 3.4 / 3.5 | 3.8 / 3.2 | 3.9 / 3.6).  Then unbounded registers, all sources of 32
-    // sites in one block while that is a wave or two, 64-site blocks of one source beyond (FP32, us per launch of an
+    // 3.5 / 3.2 | 3.6 / 3.7, 12288 3.4 / 3.5 | 3.8 / 3.2 | 3.9 / 3.6; FP32 overlap applications 10000 3.5 / 4.1, 12288
+    // 3.6 / 4.7, 15552 4.1 / 4.6, where the bare launch is 4.1 / 3.7).  Then unbounded registers, all sources of 32
+    // sites in one block while that is a wave or two (of 128 blocks or more: 12 sources at 6^4, 42 blocks, 6.1
+    // against 4.6), 64-site blocks of one source beyond (FP32, us per launch of an
     // overlap application, 32 x R against 64 x 1: three sources at 8^4 4.4 / 5.3, seven 5.9 / 6.1, twelve 5.7 / 6.3, seven
     // at 8^3 x 16 6.1 / 6.2 (bare launch 6.2 / 5.8), twelve 10.2 / 8.9, five at 12^4 10.0 / 9.8, twelve 29.5 / 21.2);
     // one and two sources keep theirs longer (128 x 1 against 64 x 1 at 16^3 x 32 11.1 / 11.4, 12^4 6.11 / 6.06;
     // 32 x 2 12.2 / 12.4 at 14 x 10 x 18 x 30, 24.5 / 24.7 at 16^3 x 32).  More resident warps last (variant 1 against
     // 0: 12 sources at 8^3 x 16 8.9 / 8.9, five at 14 x 10 x 18 x 30 34.4 / 34.6, three at 16^3 x 32 35.3 / 36.5)
-    if (n <= 9000) return {32, 1, 12};
+    if (n <= (prec == P_F32 ? 13000 : 9000)) return {32, 1, 12};
     if (nrhs == 1 && n > 45000 && n <= 300000) return {128, 1, 0};
-    if (nrhs > 1 && n <= (nrhs == 2 ? 300000 : 50000)) return {32, nrhs < 16 ? nrhs : 16, 0};
+    if (nrhs > 1 && 2 * g.Vh >= 4096 && n <= (nrhs == 2 ? 300000 : 50000)) return {32, nrhs < 16 ? nrhs : 16, 0};
     return {64, 1, n <= 200000 ? 0 : 1};
 }
 
