@@ -33,8 +33,9 @@
  *    a call on another stream waits on the device for the one before.
  *    (ov_dslash_field, ov_field_import and ov_field_export use no shared
  *    buffer and are ordered by their stream alone; launches that the caller
- *    captured into its own graph are the caller's to order.)  One host thread
- *    at a time uses a context.  The caller owns every
+ *    captured into its own graph are the caller's to order.  ov_apply_* on a
+ *    stream that is being captured return OV_ECUDA and record nothing.)  One
+ *    host thread at a time uses a context.  The caller owns every
  *    buffer it passes; the library owns the packed gauge field, the
  *    eigenpairs, all workspaces and the network weights.
  *  - Every call returns OV_OK (0) or a negative ov_status; on error no
