@@ -156,10 +156,6 @@ __host__ __device__ __forceinline__ Fix link_to_fix(double u)
     if (r.l == -2147483647 - 1) r.l = -2147483647;  // one unit: fix_sign
     return r;
 }
-__host__ __device__ __forceinline__ double fix_to_link(Fix a)
-{
-    return (double)a.h * 9.31322574615478515625e-10 + (double)a.l * 2.16840434497100886801490560173988e-19;
-}
 
 struct FixProd {
     long long hi, mid;

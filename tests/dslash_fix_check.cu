@@ -16,6 +16,8 @@ static int fail(const char* what, double a, double b)
     return 1;
 }
 
+static double fix_to_link(Fix a) { return std::ldexp((double)a.h, -30) + std::ldexp((double)a.l, -62); }
+
 int main()
 {
     std::mt19937_64 g(1);

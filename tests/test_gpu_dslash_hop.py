@@ -42,7 +42,9 @@ def test_hop_variant(dims, nrhs, prec):
 
 
 @pytest.mark.parametrize("prec", ["f32", "f16", "bf16", "f64", "df64"])
-@pytest.mark.parametrize("dims,nrhs", [((6, 6, 6, 10), 4), ((6, 6, 6, 10), 5)])  # 8640 and 10800 sites x sources
+# sites x sources on either side of the limits: 9000 (16-bit) and 13 000 (FP32), 12 000 (FP64, double-float), 50 000
+@pytest.mark.parametrize("dims,nrhs", [((6, 6, 6, 10), 4), ((6, 6, 6, 10), 5), ((6, 6, 6, 10), 7), ((8, 8, 8, 8), 4),
+                                       ((8, 8, 8, 8), 13), ((16, 8, 8, 16), 1), ((16, 8, 8, 16), 2)])
 def test_default_launch(dims, nrhs, prec):
     from paper_1106_4964_gb300 import Context
 
